@@ -150,14 +150,15 @@ __device__ __forceinline__ uint32_t conv3_tap_mask(const Conv3Geo& G, const uint
 // activations are all zero; accumulate flags are compile-time constants (the
 // first issued MMA of the tile is peeled).
 template <int CO>
-__device__ __forceinline__ void conv3_issue(uint32_t d, uint64_t adesc0, uint64_t bdesc0, int Wp, uint32_t tapmask) {
+__device__ __forceinline__ void conv3_issue(uint32_t d, uint64_t adesc0, uint64_t bdesc0,
+                                            const uint64_t (&tap_off)[9], uint32_t tapmask) {
   constexpr uint32_t idesc = idesc_bf16_f32(kBM, CO);
   if (tapmask == 0x1FFu) {
     tc_mma_bf16(d, adesc0, bdesc0, idesc, 0u);
 #pragma unroll
     for (int i = 1; i < 36; ++i) {
       const int tap = i >> 2, ks = i & 3;
-      tc_mma_bf16(d, adesc0 + (uint64_t)((((tap / 3) * Wp + (tap % 3)) * 128) >> 4) + (uint64_t)(2 * ks),
+      tc_mma_bf16(d, adesc0 + tap_off[tap] + (uint64_t)(2 * ks),
                   bdesc0 + (uint64_t)((tap * CO * 128) >> 4) + (uint64_t)(2 * ks), idesc, 1u);
     }
     return;
@@ -170,7 +171,10 @@ __device__ __forceinline__ void conv3_issue(uint32_t d, uint64_t adesc0, uint64_
   }
   const int ftap = __ffs((int)tapmask) - 1;
   {
-    const uint64_t ad = adesc0 + (uint64_t)((((ftap / 3) * Wp + (ftap % 3)) * 128) >> 4);
+    uint64_t ad = adesc0;
+#pragma unroll
+    for (int tap = 1; tap < 9; ++tap)
+      if (tap == ftap) ad = adesc0 + tap_off[tap];
     const uint64_t bd = bdesc0 + (uint64_t)((ftap * CO * 128) >> 4);
     tc_mma_bf16(d, ad, bd, idesc, 0u);
 #pragma unroll
@@ -179,7 +183,7 @@ __device__ __forceinline__ void conv3_issue(uint32_t d, uint64_t adesc0, uint64_
 #pragma unroll
   for (int tap = 1; tap < 9; ++tap) {
     if (tap <= ftap || !((tapmask >> tap) & 1u)) continue;
-    const uint64_t ad = adesc0 + (uint64_t)((((tap / 3) * Wp + (tap % 3)) * 128) >> 4);
+    const uint64_t ad = adesc0 + tap_off[tap];
     const uint64_t bd = bdesc0 + (uint64_t)((tap * CO * 128) >> 4);
 #pragma unroll
     for (int ks = 0; ks < 4; ++ks) tc_mma_bf16(d, ad + (uint64_t)(2 * ks), bd + (uint64_t)(2 * ks), idesc, 1u);
@@ -329,14 +333,20 @@ __global__ void __maxnreg__(128)
     }
   } else if (warp == kMmaWarp) {
     // -------------------------------------------------------------- MMA issue
-    if (lane == 0) {
+    // (the warp stays converged; one elected lane issues)
+    const bool el = elect_one();
+    uint64_t tap_off[9];  // start-address offsets of the taps' slab rows
+#pragma unroll
+    for (int tap = 0; tap < 9; ++tap) tap_off[tap] = (uint64_t)((((tap / 3) * Wp + (tap % 3)) * 128) >> 4);
+    const uint64_t bdesc0 = smem_desc_kmajor<64>(sW);
+    {
       int j = 0;
       bool ok = true;
       for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++j) {
         const int b = j & 1;
-        ok = mbar_wait_spin(bar_acce + 8 * b, (uint32_t)(((j >> 1) & 1) ^ 1), err, s_abort, kErrTimeoutAcc, wlim) &&
-             mbar_wait_spin(bar_full + 8 * b, (uint32_t)((j >> 1) & 1), err, s_abort, kErrTimeoutFull, wlim) &&
-             (!skip || mbar_wait_spin(bar_mask + 8 * b, (uint32_t)((j >> 1) & 1), err, s_abort, kErrTimeoutFull, wlim));
+        ok = mbar_wait_warp(bar_acce + 8 * b, (uint32_t)(((j >> 1) & 1) ^ 1), err, s_abort, kErrTimeoutAcc, wlim) &&
+             mbar_wait_warp(bar_full + 8 * b, (uint32_t)((j >> 1) & 1), err, s_abort, kErrTimeoutFull, wlim) &&
+             (!skip || mbar_wait_warp(bar_mask + 8 * b, (uint32_t)((j >> 1) & 1), err, s_abort, kErrTimeoutFull, wlim));
         if (!ok) break;
         tc_fence_after();
         const int q0 = (t - (t / G.tiles_per_img) * G.tiles_per_img) * kBM;
@@ -346,23 +356,25 @@ __global__ void __maxnreg__(128)
         // descriptors of tap 0 / k-step 0; the others differ only in the
         // start-address field (byte offset >> 4), which never carries out
         const uint64_t adesc0 = smem_desc_kmajor<64>(slab + (uint32_t)(qoff * 128));
-        const uint64_t bdesc0 = smem_desc_kmajor<64>(sW);
         const uint32_t tapmask = skip ? s_tapm[b] : 0x1FFu;
         if (j == 0) {
-          ok = mbar_wait_spin(bar_w, 0u, err, s_abort, kErrTimeoutFull, wlim);
+          ok = mbar_wait_warp(bar_w, 0u, err, s_abort, kErrTimeoutFull, wlim);
           if (!ok) break;
           tc_fence_after();
         }
-        conv3_issue<CO>(d, adesc0, bdesc0, Wp, tapmask);
-        tc_commit(bar_empty + 8 * b);  // slab and mask buffer free once these MMAs are done
-        // (the fault injection of the error-path tests leaves the first
-        // accumulator unsignalled: the epilogue's bounded wait runs out)
-        if (!(P.fault == kFaultSkipFirstAccCommit && j == 0)) tc_commit(bar_accf + 8 * b);
+        if (el) {
+          conv3_issue<CO>(d, adesc0, bdesc0, tap_off, tapmask);
+          tc_commit(bar_empty + 8 * b);  // slab and mask buffer free once these MMAs are done
+          // (the fault injection of the error-path tests leaves the first
+          // accumulator unsignalled: the epilogue's bounded wait runs out)
+          if (!(P.fault == kFaultSkipFirstAccCommit && j == 0)) tc_commit(bar_accf + 8 * b);
+        }
+        __syncwarp();
       }
       // TMEM is freed below only after the epilogue has read the last two
       // accumulators (the waits a further two tiles would make)
       for (int k = 0; k < 2 && ok; ++k, ++j)
-        ok = mbar_wait(bar_acce + 8 * (j & 1), (uint32_t)(((j >> 1) & 1) ^ 1), err, s_abort, kErrTimeoutAcc, wlim);
+        ok = mbar_wait_warp(bar_acce + 8 * (j & 1), (uint32_t)(((j >> 1) & 1) ^ 1), err, s_abort, kErrTimeoutAcc, wlim);
     }
   } else if (warp >= kFirstEpiWarp) {
     // -------------------------------------------------------------- epilogue
@@ -512,7 +524,7 @@ __global__ void __maxnreg__(128)
         mbar_drain(bar_full + 8 * (i & 1), (uint32_t)((i >> 1) & 1), wlim);
       }
     }
-    if (warp == kMmaWarp && lane == 0) {
+    if (warp == kMmaWarp && elect_one()) {
       tc_commit(bar_drain);
       mbar_drain(bar_drain, 0u, wlim);
     }

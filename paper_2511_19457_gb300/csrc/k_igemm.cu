@@ -48,6 +48,7 @@
 
 #include <mutex>
 
+#include "igemm_geo.cuh"
 #include "sparoa_kernels.h"
 
 namespace sparoa {
@@ -59,7 +60,6 @@ constexpr int kMaxSplit = 4;  // K split: at most this many units per output til
 constexpr int kEpiThreads = 32 * kEpiWarps;
 constexpr int kMmaWarp = 4 + kEpiWarps;
 constexpr int kThreads = 32 * (kMmaWarp + 1);  // 4 producer warps, epilogue warps, MMA warp
-constexpr int kBM = 128;
 constexpr int kMaxKWords = 128;  // K-block occupancy bits: up to 4096 blocks
 constexpr int kMaxTaps = 64;
 constexpr int kStgBytes = 128 * 128;  // output staging: per epilogue warp 2 blocks of 32 rows x 64 bytes
@@ -109,77 +109,6 @@ struct Cfg {
   static_assert(kStages >= 2, "stages");
   static_assert(kSmem <= 227 * 1024, "shared memory");
 };
-
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint32_t bar, int c0,
-                                            int c1, int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
-      : "memory");
-}
-
-// Launch geometry copied out of the kernel parameters into registers once:
-// reading IgemmArgs fields through a reference is a memory load, and every
-// asm statement with a memory clobber would force it again.
-struct Geo {
-  int conv, M, N, Nimg, H, W, Cp, Ho, Wo, kh, kw, stride, pad, bw, bh, bn, tw, th, Ktot;
-};
-
-__device__ __forceinline__ Geo make_geo(const IgemmArgs& a) {
-  Geo g;
-  g.conv = a.conv; g.M = a.M; g.N = a.N; g.Nimg = a.Nimg; g.H = a.H; g.W = a.W; g.Cp = a.Cp;
-  g.Ho = a.Ho; g.Wo = a.Wo; g.kh = a.kh; g.kw = a.kw; g.stride = a.stride; g.pad = a.pad;
-  g.bw = a.bw; g.bh = a.bh; g.bn = a.bn; g.tw = a.tw; g.th = a.th; g.Ktot = a.Ktot;
-  return g;
-}
-
-struct TileGeo {
-  int m0, tn0, th0, tw0, n0;
-};
-
-__device__ __forceinline__ TileGeo tile_geo(const Geo& p, int t, int nt, int BN) {
-  TileGeo g;
-  const int mi = nt == 1 ? t : t / nt;
-  g.n0 = (t - mi * nt) * BN;
-  g.m0 = 0;
-  g.tn0 = g.th0 = g.tw0 = 0;
-  if (p.conv == 2) {
-    const int per_img = p.th * p.tw;
-    g.tn0 = (mi / per_img) * p.bn;
-    const int rem = mi - (mi / per_img) * per_img;
-    g.th0 = (rem / p.tw) * p.bh;
-    g.tw0 = (rem - (rem / p.tw) * p.tw) * p.bw;
-  } else {
-    g.m0 = mi * kBM;
-  }
-  return g;
-}
-
-// Output pixel / row of tile row r and whether it exists.
-__device__ __forceinline__ int64_t tile_row(const Geo& p, const TileGeo& g, int r, bool& valid,
-                                            int& img, int& oh, int& ow) {
-  if (p.conv == 2) {
-    const int wl = r % p.bw, hl = (r / p.bw) % p.bh, nl = r / (p.bw * p.bh);
-    img = g.tn0 + nl;
-    oh = g.th0 + hl;
-    ow = g.tw0 + wl;
-    valid = img < p.Nimg && oh < p.Ho && ow < p.Wo;
-    return ((int64_t)img * p.Ho + oh) * p.Wo + ow;
-  }
-  const int64_t m = (int64_t)g.m0 + r;
-  valid = m < p.M;
-  if (p.conv == 1) {
-    const int hw = p.Ho * p.Wo;
-    img = valid ? (int)(m / hw) : 0;
-    const int rem = (int)(m - (int64_t)img * hw);
-    oh = valid ? rem / p.Wo : 0;
-    ow = valid ? rem - oh * p.Wo : 0;
-  } else {
-    img = oh = ow = 0;
-  }
-  return m;
-}
 
 // One row's 32 accumulator values (fp32 bits) through the column affine
 // (scale and shift from shared memory; none when sc is null), the residual
@@ -283,6 +212,11 @@ __device__ __forceinline__ UnitGeo unit_geo(const Geo& p, int u, int KS, int kbl
   q.ix0 = q.g.tw0 * p.stride - p.pad;
   return q;
 }
+
+template <bool B>
+struct BoolConst {
+  static constexpr bool value = B;
+};
 
 template <int BN, int BK, int LEAN>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -677,79 +611,97 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------------ MMA issue
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16_f32(kBM, BN);
-      int it = 0, j = 0;
-      bool ok = true;
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++j) {
-        const int b = j & 1;
-        if (!mbar_wait(bar_acce + 8 * b, (uint32_t)(((j >> 1) & 1) ^ 1), err, s_abort,
-                       kErrTimeoutAcc, wlim))
-          break;
-        tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)b * C::kAccCols;
-        bool first = true;
-        int slot = it % S;
-        uint32_t ph = (uint32_t)((it / S) & 1);
-        while (true) {
-          if (!mbar_wait(bar_full + 8 * slot, ph, err, s_abort, kErrTimeoutFull, wlim)) {
+    // The warp stays converged; `el` (one lane) issues.  The ring position is
+    // carried as descriptors and barrier addresses, so a stage costs a wait, a
+    // few uniform additions, its MMAs and a commit.
+    constexpr uint32_t idesc = idesc_bf16_f32(kBM, BN);
+    const bool el = elect_one();
+    const uint64_t ad0 = smem_desc_kmajor<BK>(sA), bd0 = smem_desc_kmajor<BK>(sB);
+    uint64_t ad = ad0, bd = bd0;
+    int slot = 0, j = 0;
+    uint32_t ph = 0;
+    auto next = [&]() {
+      ad += C::kAStage / 16;
+      bd += C::kBStage / 16;
+      if (++slot == S) {
+        slot = 0;
+        ph ^= 1u;
+        ad = ad0;
+        bd = bd0;
+      }
+    };
+    // One dense stage.  k-steps advance the start-address field by 32 B (2
+    // units); the accumulate flag is a constant of each MMA (a flag computed
+    // at run time roughly halves the issue rate).
+    auto stage = [&](uint32_t d, auto first) -> bool {
+      if (!mbar_wait_warp(bar_full + 8 * slot, ph, err, s_abort, kErrTimeoutFull, wlim)) return false;
+      tc_fence_after();
+      if (el) {
+        tc_mma_bf16(d, ad, bd, idesc, decltype(first)::value ? 0u : 1u);
+#pragma unroll
+        for (int k = 1; k < BK / 16; ++k) tc_mma_bf16(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, 1u);
+        tc_commit(bar_empty + 8 * slot);
+      }
+      __syncwarp();
+      next();
+      return true;
+    };
+    bool ok = true;
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++j) {
+      const int b = j & 1;
+      if (!mbar_wait_warp(bar_acce + 8 * b, (uint32_t)(((j >> 1) & 1) ^ 1), err, s_abort, kErrTimeoutAcc, wlim))
+        break;
+      tc_fence_after();
+      const uint32_t d = tmem + (uint32_t)b * C::kAccCols;
+      if (!skip) {
+        // every K block of the unit
+        const int ks = KS == 1 ? 0 : u - (u / KS) * KS;
+        const int n = KS == 1 ? kblocks : (ks + 1) * kblocks / KS - ks * kblocks / KS;
+        ok = stage(d, BoolConst<true>{});
+        for (int i = 1; i < n && ok; ++i) ok = stage(d, BoolConst<false>{});
+      } else {
+        // the occupied ones: the producer marks a unit's last stage (bit 0)
+        bool first = true, last = false;
+        while (!last) {
+          if (!mbar_wait_warp(bar_full + 8 * slot, ph, err, s_abort, kErrTimeoutFull, wlim)) {
             ok = false;
             break;
           }
           tc_fence_after();
           const int sflags = stage_last[slot];
-          const bool last = (sflags & 1) != 0;
-          const uint32_t a = sA + slot * C::kAStage;
-          const uint32_t bb = sB + slot * C::kBStage;
-          if (compact) {
-            // one or two 32-column groups, each 128 (A) / BN (B) rows of 64
-            // bytes with the 64-byte swizzle: two k-steps of 16 per group
-            const uint64_t a0 = smem_desc_sw64(a), b0 = smem_desc_sw64(bb);
-            if (first) tc_mma_bf16(d, a0, b0, idesc, 0u);
-            else tc_mma_bf16(d, a0, b0, idesc, 1u);
-            tc_mma_bf16(d, a0 + 2, b0 + 2, idesc, 1u);
-            if (!(sflags & 2)) {
-              const uint64_t a1 = smem_desc_sw64(a + kBM * 64), b1 = smem_desc_sw64(bb + BN * 64);
-              tc_mma_bf16(d, a1, b1, idesc, 1u);
-              tc_mma_bf16(d, a1 + 2, b1 + 2, idesc, 1u);
+          last = (sflags & 1) != 0;
+          if (el) {
+            if (compact) {
+              // one or two 32-column groups, each 128 (A) / BN (B) rows of 64
+              // bytes with the 64-byte swizzle: two k-steps of 16 per group
+              const uint32_t a = sA + slot * C::kAStage, bb = sB + slot * C::kBStage;
+              const uint64_t a0 = smem_desc_sw64(a), b0 = smem_desc_sw64(bb);
+              if (first) tc_mma_bf16(d, a0, b0, idesc, 0u);
+              else tc_mma_bf16(d, a0, b0, idesc, 1u);
+              tc_mma_bf16(d, a0 + 2, b0 + 2, idesc, 1u);
+              if (!(sflags & 2)) {
+                const uint64_t a1 = smem_desc_sw64(a + kBM * 64), b1 = smem_desc_sw64(bb + BN * 64);
+                tc_mma_bf16(d, a1, b1, idesc, 1u);
+                tc_mma_bf16(d, a1 + 2, b1 + 2, idesc, 1u);
+              }
+            } else {
+              if (first) tc_mma_bf16(d, ad, bd, idesc, 0u);
+              else tc_mma_bf16(d, ad, bd, idesc, 1u);
+#pragma unroll
+              for (int k = 1; k < BK / 16; ++k)
+                tc_mma_bf16(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, 1u);
             }
-            first = false;
             tc_commit(bar_empty + 8 * slot);
-            ++it;
-            if (++slot == S) {
-              slot = 0;
-              ph ^= 1u;
-            }
-            if (last) break;
-            continue;
           }
-          // k-steps advance the start-address field by 32 B (2 units); the
-          // accumulate flags are constants on both branches (a per-MMA flag
-          // computed at run time roughly halves the issue rate)
-          const uint64_t ad = smem_desc_kmajor<BK>(a), bd = smem_desc_kmajor<BK>(bb);
-          if (first) {
-            tc_mma_bf16(d, ad, bd, idesc, 0u);
-#pragma unroll
-            for (int k = 1; k < BK / 16; ++k)
-              tc_mma_bf16(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, 1u);
-          } else {
-#pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-              tc_mma_bf16(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, 1u);
-          }
+          __syncwarp();
           first = false;
-          tc_commit(bar_empty + 8 * slot);
-          ++it;
-          if (++slot == S) {
-            slot = 0;
-            ph ^= 1u;
-          }
-          if (last) break;
+          next();
         }
-        // (the fault injection of the error-path tests leaves the first
-        // accumulator unsignalled: the epilogue's bounded wait runs out)
-        if (ok && !(P.fault == kFaultSkipFirstAccCommit && j == 0)) tc_commit(bar_accf + 8 * b);
       }
+      // (the fault injection of the error-path tests leaves the first
+      // accumulator unsignalled: the epilogue's bounded wait runs out)
+      if (ok && el && !(P.fault == kFaultSkipFirstAccCommit && j == 0)) tc_commit(bar_accf + 8 * b);
+      __syncwarp();
     }
   } else if constexpr (LEAN) {
     // ------------------------------------------------------------- lean epilogue
@@ -1304,7 +1256,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_drain(bar_full + 8 * (i % S), (uint32_t)((i / S) & 1), wlim);
       }
     }
-    if (warp == kMmaWarp && lane == 0) {
+    if (warp == kMmaWarp && elect_one()) {
       tc_commit(bar_drain);
       mbar_drain(bar_drain, 0u, wlim);
     }
@@ -1319,7 +1271,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
+}  // namespace
+
+PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   static std::once_flag once;
   std::call_once(once, [] {
@@ -1333,14 +1287,14 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   return fn;
 }
 
-CUtensorMapSwizzle swz_of(int inner_bytes) {
+static CUtensorMapSwizzle swz_of(int inner_bytes) {
   return inner_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
 }
 
 // 2-D bf16 tensor [rows, cols] (cols contiguous), box {box_cols, box_rows}.
 bool make_tmap_2d(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols,
                   uint32_t box_rows) {
-  auto enc = get_encode();
+  auto enc = tmap_encoder();
   if (!enc) return false;
   cuuint64_t dims[2] = {cols, rows};
   cuuint64_t strides[1] = {cols * 2};
@@ -1356,7 +1310,7 @@ bool make_tmap_2d(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols
 // element strides {1, stride, stride, 1}.
 bool make_tmap_nhwc(CUtensorMap* m, const void* base, int n, int h, int w, int c, int box_c, int bw,
                     int bh, int bn, int stride) {
-  auto enc = get_encode();
+  auto enc = tmap_encoder();
   if (!enc) return false;
   cuuint64_t dims[4] = {(cuuint64_t)c, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
   cuuint64_t strides[3] = {(cuuint64_t)c * 2, (cuuint64_t)w * c * 2, (cuuint64_t)h * w * c * 2};
@@ -1368,6 +1322,8 @@ bool make_tmap_nhwc(CUtensorMap* m, const void* base, int n, int h, int w, int c
                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
+
+namespace {
 
 template <int BN, int BK, int LEAN>
 cudaError_t launch_cfg(const IgemmArgs& a, const CUtensorMap& tA, const CUtensorMap& tB,
@@ -1406,7 +1362,6 @@ cudaError_t launch_bn(const IgemmArgs& a, int bn, int bk, const CUtensorMap& tA,
 
 }  // namespace
 
-PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder() { return get_encode(); }
 
 void choose_spatial_tile(IgemmArgs& a) {
   int64_t best = -1;

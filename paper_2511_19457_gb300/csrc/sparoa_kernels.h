@@ -92,6 +92,15 @@ struct IgemmArgs {
 // Picks the N tile and the K split, encodes the tensor maps and launches.
 cudaError_t launch_igemm(const IgemmArgs& a, cudaStream_t s);
 
+// bf16 tensor maps (k_igemm.cu): a [rows, cols] matrix with box {box_cols,
+// box_rows}; an NHWC tensor with box {box_c, bw, bh, bn} traversed with element
+// strides {1, stride, stride, 1}.  The swizzle is the box's inner extent, 64 or
+// 128 bytes.
+bool make_tmap_2d(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols,
+                  uint32_t box_rows);
+bool make_tmap_nhwc(CUtensorMap* m, const void* base, int n, int h, int w, int c, int box_c, int bw, int bh,
+                    int bn, int stride);
+
 // Streaming multiprocessors of the current device (cached per device).
 int device_sm_count();
 
