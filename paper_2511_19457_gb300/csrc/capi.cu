@@ -288,27 +288,19 @@ sparoa_status clear_ranges(sparoa_ctx* ctx, const std::vector<std::pair<uint32_t
   return SPAROA_OK;
 }
 
-// Split-K scratch offered to the implicit-GEMM kernel: 65536 arrival counters
+// Split-K scratch offered to the implicit-GEMM kernel's gather mode: 65536 arrival counters
 // (zeroed once when allocated; every launch leaves them zero) and 64 MiB of
 // fp32 partial tiles.  Allocated with the context.
 constexpr int kSplitCounters = 65536;
 constexpr size_t kSplitCntBytes = sizeof(unsigned) * kSplitCounters;
 constexpr size_t kSplitWsBytes = (size_t)64 << 20;
 
-// slot -1: the whole scratch; 0 / 1: disjoint halves, for two launches that
-// may run at the same time (split execution)
-sparoa_status offer_splitk(sparoa_ctx* ctx, IgemmArgs* a, int slot = -1) {
+sparoa_status offer_splitk(sparoa_ctx* ctx, IgemmArgs* a) {
   if (!ctx->splitk.p) return SPAROA_OK;  // no split K
   a->ws_cnt = static_cast<unsigned*>(ctx->splitk.p);
   a->ws_cnt_len = kSplitCounters;
   a->ws = reinterpret_cast<float*>(static_cast<char*>(ctx->splitk.p) + kSplitCntBytes);
   a->ws_bytes = kSplitWsBytes;
-  if (slot >= 0) {
-    a->ws_cnt_len = kSplitCounters / 2;
-    a->ws_cnt += slot * (kSplitCounters / 2);
-    a->ws_bytes = kSplitWsBytes / 2;
-    a->ws += slot * (kSplitWsBytes / 2 / sizeof(float));
-  }
   return SPAROA_OK;
 }
 
@@ -459,11 +451,12 @@ struct GemmPlan {
   sparoa_occupancy xo;  // occupancy of x (device)
   const sparoa_occupancy* yo;
   DispatchDev disp;
+  int early_w = 0;  // IgemmArgs::early_w
 };
 
 // count_out: the input's Eq. 1 count is not known yet; the fused small-FC
 // kernel measures it into count_out (which g.disp.in_nnz points at).
-sparoa_status run_gemm(sparoa_ctx* ctx, const GemmPlan& g, cudaStream_t stream, int ws_slot = -1,
+sparoa_status run_gemm(sparoa_ctx* ctx, const GemmPlan& g, cudaStream_t stream,
                        unsigned long long* count_out = nullptr) {
   const bool small_skip = g.M <= 128 && g.W_kn != nullptr && g.K <= 8192 && (g.N % 8) == 0;
   // small inputs: statistics, dispatch and either path's product in one kernel
@@ -526,7 +519,7 @@ sparoa_status run_gemm(sparoa_ctx* ctx, const GemmPlan& g, cudaStream_t stream, 
     a.err = ctx->d_err();
     a.wait_limit = ctx->wait_limit;
     a.fault = ctx->fault == 1 ? kFaultSkipFirstAccCommit : 0;
-    SP_TRY(offer_splitk(ctx, &a, ws_slot));
+    a.early_w = g.early_w;
     SP_CUDA(launch_igemm(a, stream));
   }
   return SPAROA_OK;
@@ -547,6 +540,7 @@ struct ConvPlan {
   // a kernel of this library was launched between the producers of x, w and
   // the epilogue's parameters and the conv (IgemmArgs::early)
   int early = 0;
+  int early_w = 0;  // the same of w and the epilogue's parameters (IgemmArgs::early_w)
 };
 
 sparoa_status run_conv(sparoa_ctx* ctx, const ConvPlan& c) {
@@ -583,12 +577,13 @@ sparoa_status run_conv(sparoa_ctx* ctx, const ConvPlan& c) {
   a.wait_limit = ctx->wait_limit;
   a.fault = ctx->fault == 1 ? kFaultSkipFirstAccCommit : 0;
   a.early = c.early;
+  a.early_w = c.early_w;
   if (!pointwise && conv3_supported(a)) {
     SP_CUDA(launch_conv3(a, ctx->stream));
     return SPAROA_OK;
   }
   if (a.conv == 2) choose_spatial_tile(a);
-  SP_TRY(offer_splitk(ctx, &a));
+  if (a.conv == 1) SP_TRY(offer_splitk(ctx, &a));
   SP_CUDA(launch_igemm(a, ctx->stream));
   return SPAROA_OK;
 }
@@ -834,6 +829,8 @@ sparoa_status sparoa_gemm(sparoa_ctx* ctx, const void* x, int64_t M, int64_t K, 
     SP_TRY(measure(ctx, x, M, K, &p.xo));
   }
   if (y_occ) SP_TRY(occ_clear(ctx, *y_occ));
+  // a clear or statistics kernel of this call runs before the product
+  p.early_w = y_occ || !(x_occ || fused_count) ? 1 : 0;
   p.disp.in_nnz = reinterpret_cast<const unsigned long long*>(p.xo.nnz);
   p.disp.numel = (unsigned long long)(M * K);
   p.disp.s_thr = t.s_thr;
@@ -841,7 +838,7 @@ sparoa_status sparoa_gemm(sparoa_ctx* ctx, const void* x, int64_t M, int64_t K, 
   p.disp.force = t.force_path;
   p.disp.path_out = ctx->d_path();
   if (M > 0)
-    SP_TRY(run_gemm(ctx, p, ctx->stream, -1,
+    SP_TRY(run_gemm(ctx, p, ctx->stream,
                     fused_count ? reinterpret_cast<unsigned long long*>(ctx->d_count()) : nullptr));
   if (!host_out) return SPAROA_OK;
   uint64_t nnz = 0;
@@ -935,12 +932,11 @@ sparoa_status sparoa_gemm_split(sparoa_ctx* ctx, const void* x, int64_t M, int64
   }
   if (Ms == 0) return run_gemm(ctx, b, ctx->stream);
   if (Ms == M) return run_gemm(ctx, a, ctx->stream);
-  // the two parts on two streams (each takes half of the split-K scratch),
-  // forked from and joined back into the context stream
+  // the two parts on two streams, forked from and joined back into the context stream
   SP_CUDA(cudaEventRecord(ctx->ev_fork, ctx->stream));
   SP_CUDA(cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
-  SP_TRY(run_gemm(ctx, a, ctx->aux, 1));
-  SP_TRY(run_gemm(ctx, b, ctx->stream, 0));
+  SP_TRY(run_gemm(ctx, a, ctx->aux));
+  SP_TRY(run_gemm(ctx, b, ctx->stream));
   SP_CUDA(cudaEventRecord(ctx->ev_join, ctx->aux));
   SP_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
   return SPAROA_OK;
@@ -1100,6 +1096,7 @@ sparoa_status sparoa_conv2d(sparoa_ctx* ctx, const void* x, int64_t N, int64_t H
       c.disp.force = t.force_path;
       c.disp.path_out = ctx->d_path();
       c.early = launched && c.Cp == C_in ? 1 : 0;  // (padding launches write x and w)
+      c.early_w = c.early;
       SP_TRY(run_conv(ctx, c));
     }
   }
@@ -1528,6 +1525,9 @@ sparoa_status sparoa_run_graph(sparoa_ctx* ctx, const sparoa_op* ops, int32_t n_
         c.disp.fpb_ok = intensity_ok(t, wk);
         c.disp.force = t.force_path;
         c.disp.path_out = d_paths + i;
+        // the walk's clear and statistics kernels run before every operator;
+        // only padded weights are written inside it
+        c.early_w = aux[(size_t)i].cp ? 0 : 1;
         SP_TRY(run_conv(ctx, c));
         break;
       }
@@ -1557,6 +1557,7 @@ sparoa_status sparoa_run_graph(sparoa_ctx* ctx, const sparoa_op* ops, int32_t n_
         p.disp.fpb_ok = intensity_ok(t, wk);
         p.disp.force = t.force_path;
         p.disp.path_out = d_paths + i;
+        p.early_w = 1;
         SP_TRY(run_gemm(ctx, p, ctx->stream));
         break;
       }

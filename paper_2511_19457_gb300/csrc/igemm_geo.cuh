@@ -1,4 +1,4 @@
-// Tile geometry of the implicit-GEMM kernel (k_igemm.cu).
+// Tile geometry of the implicit-GEMM kernels (k_igemm.cu, k_onetile.cu).
 #pragma once
 
 #include "sparoa_kernels.h"

@@ -46,6 +46,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+
 #include <mutex>
 
 #include "igemm_geo.cuh"
@@ -282,7 +283,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int nt = (p.N + BN - 1) / BN;
   const int mtiles = p.conv == 2 ? ((p.Nimg + p.bn - 1) / p.bn) * p.th * p.tw : (p.M + kBM - 1) / kBM;
   const int tiles = mtiles * nt;
-  // split K: work unit u = (tile u / KS, K range u % KS); KS consecutive units
+  // split K (gather mode only): work unit u = (tile u / KS, K range u % KS); KS consecutive units
   // (run by neighbouring CTAs at the same time) share one output tile
   const int KS = (!LEAN && P.ksplit > 1) ? P.ksplit : 1;
   const int units = tiles * KS;
@@ -1395,10 +1396,11 @@ void choose_spatial_tile(IgemmArgs& a) {
 // SMs.  On GB300, GEMMs with M 1024..8192, K 768..3072 and N 768..3072 follow
 // this ordering.  K blocks are 64 wide (128-byte swizzle) wherever the
 // channel layout allows: 32 wide ones were slower at every tile width.
-// Splitting K pays only while the tiles leave SMs idle, at most 4 ways and
-// with at least 8 K blocks per unit (the tile's last unit reads the other
-// partials alone); splitting further to even out the rounds was slower (the
-// partial stores and reads cost more than the main-loop time they save).
+// 64-wide tiles that number at most the SMs go to the one-tile-per-cluster
+// kernel (k_onetile.cu), which shares a tile's K range through distributed
+// shared memory.  The gather mode, which that kernel does not have, splits K
+// here while the tiles leave SMs idle, at most 4 ways and with at least 8 K
+// blocks per unit (the tile's last unit reads the other partials alone).
 static int k_block(const IgemmArgs& a) { return (a.conv == 2 ? (a.Cp % 64 == 0) : (a.Ktot > 32)) ? 64 : 32; }
 
 void choose_tiles(const IgemmArgs& a, int64_t mtiles, int* bn_out, int* ks_out) {
@@ -1424,7 +1426,7 @@ void choose_tiles(const IgemmArgs& a, int64_t mtiles, int* bn_out, int* ks_out) 
   const int bk = k_block(a);
   const int kblocks = (a.Ktot + bk - 1) / bk;
   int ks = 1;
-  if (a.ws && a.ws_cnt && tiles < sms && tiles <= a.ws_cnt_len) {
+  if (a.conv == 1 && a.ws && a.ws_cnt && tiles < sms && tiles <= a.ws_cnt_len) {
     ks = (int)(sms / tiles);
     if (ks > kMaxSplit) ks = kMaxSplit;
     while (ks > 1 && (kblocks < 8 * ks || (size_t)tiles * ks * kBM * bn * 4 > a.ws_bytes)) --ks;
@@ -1443,6 +1445,13 @@ cudaError_t launch_igemm(const IgemmArgs& a_in, cudaStream_t s) {
   choose_tiles(a, mtiles, &bn, &ks);
   a.ksplit = ks;
   const int bk = k_block(a);
+  if (bn == 64) {
+    const int split = onetile_split(a, mtiles, bk);
+    if (split > 0) {
+      a.ksplit = split;
+      return launch_onetile(a, mtiles, bk, s);
+    }
+  }
   CUtensorMap tA, tB, tY;
   memset(&tA, 0, sizeof(tA));
   memset(&tY, 0, sizeof(tY));

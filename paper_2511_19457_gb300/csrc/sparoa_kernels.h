@@ -34,6 +34,27 @@ cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
 }
 
+// launch_kernel for a grid of thread-block clusters of `cluster` consecutive CTAs.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_cluster_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, unsigned cluster, size_t smem,
+                                  cudaStream_t s, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl_enabled() ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
+}
+
 // Zero up to five word ranges (the fields of an occupancy block) in one launch.
 struct ClearArgs {
   uint32_t* p[5];
@@ -79,6 +100,8 @@ struct IgemmArgs {
   // when this grid starts and may be read before griddepcontrol.wait (every
   // kernel here triggers its dependents only after its own wait)
   int early = 0;
+  // 1: the same for w and the epilogue's parameters only
+  int early_w = 0;
   // split K (set by launch_igemm from the scratch offered here): fp32 partial
   // tiles [tiles][ksplit][128][BN] in `ws` (ws_bytes), one zeroed arrival
   // counter per output tile in `ws_cnt` (ws_cnt_len), left zero again
@@ -100,6 +123,12 @@ bool make_tmap_2d(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols
                   uint32_t box_rows);
 bool make_tmap_nhwc(CUtensorMap* m, const void* base, int n, int h, int w, int c, int box_c, int bw, int bh,
                     int bn, int stride);
+
+// One 128 x 64 output tile per cluster of up to 8 CTAs that share its K range
+// (k_onetile.cu).  onetile_split: the cluster size for K blocks of `bk`, 0
+// where the shape is not the kernel's (more tiles than SMs, or the gather mode).
+int onetile_split(const IgemmArgs& a, int64_t mtiles, int bk);
+cudaError_t launch_onetile(const IgemmArgs& a, int64_t mtiles, int bk, cudaStream_t s);  // a.ksplit set
 
 // Streaming multiprocessors of the current device (cached per device).
 int device_sm_count();
