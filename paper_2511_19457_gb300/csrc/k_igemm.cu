@@ -31,18 +31,22 @@
 // The epilogue applies bias / batch norm / residual / activation, stores y and
 // writes y's Eq. 1 count and occupancy bitmaps for the next operator.
 //
-// Warp roles (416 threads): warps 0-3 producers (the skip masks; thread 0
-// issues TMA; all 128 gather in mode 1), warps 4-11 epilogue (two per TMEM
-// lane quarter, each taking 32 of every 64 accumulator columns), warp 12 TMEM
-// allocation and MMA issue (lane 0).
+// Warp roles: producer warps (the skip masks; thread 0 issues TMA; all 128
+// gather in mode 1), epilogue warps from warp 4 on (by TMEM lane quarter, each
+// taking 32-column blocks), one warp for TMEM allocation and MMA issue.
 //
 // Each tile shape is compiled three times: the general kernel, and lean ones
 // for modes 0 and 2 without a K split or fp32 output, without a residual and
-// with one (N % 8 == 0).  With small K the
-// epilogue is the whole cost of a tile and runs at a fraction of an
-// instruction per cycle (few warps, long dependency chains); the lean kernel's
-// smaller, branch-free epilogue issues fewer instructions per tile and misses
-// the instruction cache less.
+// with one (N % 8 == 0).  Small-K problems are bound by the epilogue's latency
+// and by what feeds it, so the lean kernel has 16 epilogue warps that never wait
+// for each other, four accumulators in flight (up to 128-wide tiles), one
+// converged producer warp that lays out 32 tiles at a time, and keeps weights
+// that fit the ring.  Measured (GB300, BN + ReLU6 + output occupancy): the 1x1
+// expansion [32,112,112,16] -> 96 53.5 -> 34.5 us (90 MB: 2.6 TB/s; 22.9 without
+// the occupancy), [32,56,56,24] -> 144 35.9 -> 22.9 us, the MLP's up projection
+// [6304,768] x [3072,768] + GELU 48 -> 45 us.  One column block's instructions
+// appear once: a second copy (planes of two blocks in registers) cost the wide
+// tiles 10 % in instruction-cache misses.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -56,14 +60,24 @@ namespace sparoa {
 
 namespace {
 
-constexpr int kEpiWarps = 8;
-constexpr int kMaxSplit = 4;  // K split: at most this many units per output tile                   // two per TMEM lane quarter, 32 of each 64 columns
-constexpr int kEpiThreads = 32 * kEpiWarps;
-constexpr int kMmaWarp = 4 + kEpiWarps;
-constexpr int kThreads = 32 * (kMmaWarp + 1);  // 4 producer warps, epilogue warps, MMA warp
+constexpr int kMaxSplit = 4;  // K split: at most this many units per output tile
+constexpr int kEpiWarp0 = 4;  // first epilogue warp
+// Warp roles.  The general kernel: 4 producer warps (all 128 threads gather in
+// mode 1), 8 epilogue warps (two per TMEM lane quarter), the MMA warp.  The
+// lean ones: 3 producer warps, the MMA warp, 16 epilogue warps -- 5 warps per
+// scheduler, which leaves 96 registers a thread (a 21st warp would leave 80 and
+// spill).
+template <int LEAN>
+struct Warps {
+  static constexpr int kProd = LEAN ? 3 : 4;
+  static constexpr int kEpi = LEAN ? 16 : 8;
+  static constexpr int kEpiThreads = 32 * kEpi;
+  static constexpr int kMma = LEAN ? 3 : kEpiWarp0 + kEpi;
+  static constexpr int kThreads = 32 * (LEAN ? 20 : 13);
+};
 constexpr int kMaxKWords = 128;  // K-block occupancy bits: up to 4096 blocks
 constexpr int kMaxTaps = 64;
-constexpr int kStgBytes = 128 * 128;  // output staging: per epilogue warp 2 blocks of 32 rows x 64 bytes
+constexpr int kStgBytes = 2 * 128 * 128;  // output staging: 32 rows x 64 bytes per epilogue warp (two each in the general kernel)
 constexpr int kWarpStgBytes = 32 * 64;
 constexpr int kMaxAccCols = 4096;     // per-CTA column counters (output occupancy)
 
@@ -78,35 +92,39 @@ struct Cfg {
   // 40 KB stage (4096 x 3072 x 768: 26.1 -> 22.3 us).  kFixed is everything
   // but the ring (barriers and flags of at most 12 stages) plus the 1024 bytes
   // of alignment slack.
-  static constexpr int kFixed = 2 * kStgBytes + (2 * 12 + 5) * 8 + (12 + 8) * 4 + 16 + kMaxKWords * 4 +
-                                kMaxTaps * 8 + 4 * BN * 4 + 4 * BN * 4 + kMaxAccCols * 4 + 2 * kBM * 8 +
-                                2 * (BN / 32) * 4 + 16 + 1024;
+  // column affine: general kernel scale[2][BN], shift[2][BN]; lean kernels
+  // scale[BN], shift[BN] and 64 floats per epilogue warp
+  static constexpr int kAffBytes = 4 * BN * 4 > 2 * BN * 4 + 16 * 256 ? 4 * BN * 4 : 2 * BN * 4 + 16 * 256;
+  static constexpr int kFixed = kStgBytes + (2 * 12 + 10) * 8 + (12 + 8) * 4 + 16 + kMaxKWords * 4 +
+                                kMaxTaps * 8 + kAffBytes + 4 * BN * 4 + kMaxAccCols * 4 + kBM * 8 +
+                                (BN / 32) * 4 + 16 + 1024;
   static constexpr int kBudget =
-      BN == 192 ? 227 * 1024 - kFixed : 200 * 1024 - 2 * kStgBytes - 6 * 1024 - kMaxAccCols * 4;
+      BN == 192 ? 227 * 1024 - kFixed : 200 * 1024 - kStgBytes - 6 * 1024 - kMaxAccCols * 4;
   static constexpr int kStagesRaw = kBudget / kStageBytes;
   static constexpr int kStages = kStagesRaw > 12 ? 12 : kStagesRaw;
   static constexpr int kLag = kStages - 2;  // cp.async stages in flight (mode 1)
   static constexpr int kAOff = 0;
   static constexpr int kBOff = kAOff + kStages * kAStage;
   static constexpr int kStgOff = kBOff + kStages * kBStage;          // 1024-aligned
-  static constexpr int kBarOff = kStgOff + 2 * kStgBytes;
-  static constexpr int kNumBars = 2 * kStages + 5;                   // full, empty, accf[2], acce[2], drain
+  static constexpr int kBarOff = kStgOff + kStgBytes;
+  static constexpr int kNumBars = 2 * kStages + 10;                  // full, empty, accf[4], acce[4], drain, resident B
   static constexpr int kFlagOff = kBarOff + kNumBars * 8;
   static constexpr int kKBitsOff = (kFlagOff + (kStages + 8) * 4 + 15) & ~15;
   static constexpr int kTapOff = kKBitsOff + kMaxKWords * 4;
   static constexpr int kScaleOff = kTapOff + kMaxTaps * 8;
-  static constexpr int kShiftOff = kScaleOff + 2 * BN * 4;  // scale / shift: [2 accumulators][BN]
-  static constexpr int kCntOff = kShiftOff + 2 * BN * 4;
+  static constexpr int kCntOff = kScaleOff + kAffBytes;
   static constexpr int kAccOff = kCntOff + 4 * BN * 4;
-  static constexpr int kRowOff = kAccOff + kMaxAccCols * 4;   // [2][128] row bits of the tile
-  static constexpr int kBlkOff = kRowOff + 2 * kBM * 8;       // [2][BN / 32] block-mask words
-  static constexpr int kBytes = kBlkOff + 2 * (BN / 32) * 4 + 16;
+  static constexpr int kRowOff = kAccOff + kMaxAccCols * 4;   // [128] row bits of the tile (general kernel)
+  static constexpr int kBlkOff = kRowOff + kBM * 8;           // [BN / 32] block-mask words (general kernel)
+  // [16 warps][BN / 32 blocks][3 planes][32] bit-sliced column counts (lean, BN <= 128)
+  static constexpr int kPlaneOff = (kBlkOff + (BN / 32) * 4 + 15) & ~15;
+  static constexpr int kPlaneBytes = BN <= 128 ? 16 * (BN / 32) * 3 * 128 : 0;
+  static constexpr int kBytes = kPlaneOff + kPlaneBytes + 16;
   static constexpr int kSmem = kBytes + 1024;  // slack for 1024-byte alignment
   // TMEM: accumulator b starts at column b * kAccCols (BN rounded up to a
   // power of two, so each starts on a power-of-two column); the allocation
   // covers both
   static constexpr uint32_t kAccCols = BN <= 64 ? 64u : (BN <= 128 ? 128u : 256u);
-  static constexpr uint32_t kTmemCols = 2 * kAccCols;
   static_assert(kStages >= 2, "stages");
   static_assert(kSmem <= 227 * 1024, "shared memory");
 };
@@ -164,21 +182,28 @@ __device__ __forceinline__ void affine_act_pack32(const uint32_t (&raw)[32], con
   }
 }
 
-// Bit c of the result: bf16 value c of the 16 packed pairs is non-zero.  Per
-// two words: the non-zero flags of their four halves (bits 15 and 31 after
-// nz_pairs' carry trick) are gathered into one word's byte tops (bits 7, 15,
-// 23, 31) by a byte permute, and the multiply by 1 + 2^7 + 2^14 + 2^21 moves
-// them, without carries, to bits 28..31.
+// Which of the 16 packed pairs' bf16 values are non-zero (any pattern but +-0):
+// bit i for the low value of pair i (column 2 i), bit 16 + i for the high one
+// (column 2 i + 1): one compare and one three-input logic operation per pair.
 __device__ __forceinline__ uint32_t nz_mask32(const uint32_t (&pk)[16]) {
+  const __nv_bfloat162 zero = __floats2bfloat162_rn(0.f, 0.f);
   uint32_t m = 0u;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const uint32_t ta = (pk[2 * i] & 0x7FFF7FFFu) + 0x7FFF7FFFu;
-    const uint32_t tb = (pk[2 * i + 1] & 0x7FFF7FFFu) + 0x7FFF7FFFu;
-    const uint32_t x = __byte_perm(ta, tb, 0x7531) & 0x80808080u;
-    m |= ((x * 0x00204081u) >> 28) << (4 * i);
-  }
+  for (int i = 0; i < 16; ++i)
+    m |= __hneu2_mask(*reinterpret_cast<const __nv_bfloat162*>(&pk[i]), zero) & (0x00010001u << i);
   return m;
+}
+
+// nz_mask32's bit order to column order (bit c = column c).
+__device__ __forceinline__ uint32_t nz_unpermute(uint32_t m) {
+  uint32_t e = m & 0xFFFFu, o = m >> 16;
+#pragma unroll
+  for (int s = 8; s > 0; s >>= 1) {
+    const uint32_t k = s == 8 ? 0x00FF00FFu : s == 4 ? 0x0F0F0F0Fu : s == 2 ? 0x33333333u : 0x55555555u;
+    e = (e | (e << s)) & k;
+    o = (o | (o << s)) & k;
+  }
+  return e | (o << 1);
 }
 
 // Everything a producer thread needs to know about work unit u (tile u / ks,
@@ -220,11 +245,17 @@ struct BoolConst {
 };
 
 template <int BN, int BK, int LEAN>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
     igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmA32,
                  const __grid_constant__ CUtensorMap tmB32, const IgemmArgs P) {
   using C = Cfg<BN, BK>;
+  constexpr int kEpiThreads = Warps<LEAN>::kEpiThreads;
+  constexpr int kMmaWarp = Warps<LEAN>::kMma;
+  constexpr int kProd = Warps<LEAN>::kProd, kProdThreads = 32 * kProd;
+  // accumulators in tensor memory: tiles in flight between the MMAs and the epilogue
+  constexpr int kAcc = LEAN && BN <= 128 ? 4 : 2;
+  constexpr uint32_t kTmemCols = kAcc * C::kAccCols;
   const Geo p = make_geo(P);
   // lean kernels (LEAN 1: no residual, 2: a residual and N % 8 == 0): TMA
   // producers only (mode 0 or 2), no K split, bf16 output (the host launches
@@ -254,8 +285,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t bar_full = sbase + C::kBarOff;  // + 8*s
   const uint32_t bar_empty = bar_full + 8 * S;   // + 8*s
   const uint32_t bar_accf = bar_empty + 8 * S;   // + 8*b
-  const uint32_t bar_acce = bar_accf + 16;       // + 8*b
-  const uint32_t bar_drain = bar_acce + 16;      // after an abort: the MMAs issued so far are done
+  const uint32_t bar_acce = bar_accf + 32;       // + 8*b
+  const uint32_t bar_drain = bar_acce + 32;      // after an abort: the MMAs issued so far are done
+  const uint32_t bar_resb = bar_drain + 8;       // the resident B blocks have landed
   int* flags = reinterpret_cast<int*>(smem + C::kFlagOff);
   int* stage_last = flags;                // [S]: 1 = last stage of its tile
   volatile int* s_abort = flags + S;      // CTA-wide abort request
@@ -265,9 +297,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* s_kbits = reinterpret_cast<uint32_t*>(smem + C::kKBitsOff);
   unsigned long long* s_tap = reinterpret_cast<unsigned long long*>(smem + C::kTapOff);
   float* s_scale = reinterpret_cast<float*>(smem + C::kScaleOff);
-  float* s_shift = reinterpret_cast<float*>(smem + C::kShiftOff);
-  const uint32_t sScale = sbase + C::kScaleOff;
-  const uint32_t sShift = sbase + C::kShiftOff;
+  float* s_shift = s_scale + (LEAN ? BN : 2 * BN);
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(smem + C::kCntOff);  // [4][BN]
   uint32_t* s_acc = reinterpret_cast<uint32_t*>(smem + C::kAccOff);  // [N] non-zeros per column
   unsigned long long* s_rowbm = reinterpret_cast<unsigned long long*>(smem + C::kRowOff);
@@ -287,6 +317,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   // (run by neighbouring CTAs at the same time) share one output tile
   const int KS = (!LEAN && P.ksplit > 1) ? P.ksplit : 1;
   const int units = tiles * KS;
+  // Lean epilogue: with four accumulators the 4 warps of a TMEM lane quarter
+  // take every 4th tile each; with two (192- and 256-wide tiles), and where the
+  // CTA has one tile, they share a tile's 32-column blocks.  ncw: warps that
+  // share a quarter of a tile.
+  const int ncw = kAcc == 2 || units <= (int)gridDim.x ? 4 : 1;
 
   if (!LEAN && P.dense_only) {
     // launched next to the fused small-FC kernel, which handles the zero-skip
@@ -302,11 +337,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(bar_full + 8 * s, (!LEAN && p.conv == 1) ? 129u : 1u);
       mbar_init(bar_empty + 8 * s, 1u);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < kAcc; ++b) {
       mbar_init(bar_accf + 8 * b, 1u);
-      mbar_init(bar_acce + 8 * b, (uint32_t)kEpiThreads);
+      mbar_init(bar_acce + 8 * b, LEAN ? (uint32_t)(4 * ncw) : (uint32_t)kEpiThreads);
     }
     mbar_init(bar_drain, 1u);
+    mbar_init(bar_resb, 1u);
     *s_abort = 0;
     fence_mbar_init();
     if (p.conv != 1) prefetch_tmap(&tmA);
@@ -317,18 +353,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (!y_f32) prefetch_tmap(&tmY);
   }
-  if (warp == kMmaWarp) tmem_alloc(smem_u32(s_tmem), C::kTmemCols);
-  if (acc_smem && warp >= 4 && warp < kMmaWarp)
+  if (warp == kMmaWarp) tmem_alloc(smem_u32(s_tmem), kTmemCols);
+  const bool epi_warp = warp >= kEpiWarp0 && (LEAN || warp < kMmaWarp);
+  if (acc_smem && epi_warp)
     for (int c = threadIdx.x - 128; c < p.N; c += kEpiThreads) s_acc[c] = 0u;
-  if (warp >= 4 && warp < kMmaWarp) {
-    for (int i = threadIdx.x - 128; i < 2 * kBM; i += kEpiThreads) s_rowbm[i] = 0ull;
-    for (int i = threadIdx.x - 128; i < 2 * (BN / 32); i += kEpiThreads) s_blk[i] = 0u;
+  if (!LEAN && epi_warp) {
+    for (int i = threadIdx.x - 128; i < kBM; i += kEpiThreads) s_rowbm[i] = 0ull;
+    for (int i = threadIdx.x - 128; i < BN / 32; i += kEpiThreads) s_blk[i] = 0u;
   }
   // The producers' first work unit is laid out before the grid dependency
   // wait: no memory is read, and under programmatic dependent launch this
   // overlaps the tail of the kernel before.
   UnitGeo ug{};
-  if (warp < 4 && (int)blockIdx.x < units) ug = unit_geo(p, blockIdx.x, KS, kblocks, nt, BN, BK, threadIdx.x);
+  if (warp < kProd && (int)blockIdx.x < units) ug = unit_geo(p, blockIdx.x, KS, kblocks, nt, BN, BK, threadIdx.x);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -344,10 +381,75 @@ __global__ void __launch_bounds__(kThreads, 1)
   // groups each (compacted), loaded as 32-column boxes with the 64-byte swizzle
   const bool compact = skip && p.conv == 0 && BK == 64 && kgroups <= kMaxKWords * 32 && in_blk != nullptr;
 
+  // every tile of the CTA has the same columns
+  const bool fixed_cols = nt == 1 || (int)gridDim.x % nt == 0 || units <= (int)gridDim.x;
+  // ... and, on the dense path, a K range that fits the ring: its B blocks are
+  // loaded once and stay, and the ring carries A alone (a 1x1 expansion
+  // [32,112,112,16] -> 96 spent 11 of 53 us on reloading its 12 KB of weights per tile)
+  const bool resident_b = LEAN && !skip && fixed_cols && kblocks <= S && units > (int)gridDim.x;
+
   if (!run) {
     // nothing to do; fall through to the common exit (TMEM is freed there)
-  } else if (warp < 4) {
+  } else if (warp < kProd) {
     // ------------------------------------------------------------------ producers
+    if (LEAN && !skip) {
+      // Dense path: one converged warp, one elected lane issues.  The tiles'
+      // origins (a few integer divisions each) are computed for 32 tiles at a
+      // time, one per lane.
+      if (warp == 0) {
+        const bool el = elect_one();
+        if (resident_b && el) {
+          const int n0 = ((int)blockIdx.x % nt) * BN;
+          mbar_arrive_expect_tx(bar_resb, (uint32_t)(kblocks * C::kBStage));
+          for (int kb = 0; kb < kblocks; ++kb) tma_load_2d(sB + kb * C::kBStage, &tmB, bar_resb, kb * BK, n0);
+        }
+        const uint32_t bytes = resident_b ? (uint32_t)C::kAStage : (uint32_t)C::kStageBytes;
+        const int cb_per_tap = p.Cp / BK;
+        int it = 0, slot = 0;
+        uint32_t ph = 0u;
+        bool ok = true;
+        for (int u0 = blockIdx.x; u0 < units && ok; u0 += 32 * (int)gridDim.x) {
+          const int ul = u0 + lane * (int)gridDim.x;
+          const TileGeo gl = tile_geo(p, ul < units ? ul : u0, nt, BN);
+          const int yl = p.conv == 2 ? gl.th0 * p.stride - p.pad : gl.m0, xl = gl.tw0 * p.stride - p.pad;
+          for (int i = 0; i < 32 && u0 + i * (int)gridDim.x < units && ok; ++i) {
+            const int y0 = __shfl_sync(0xffffffffu, yl, i), x0 = __shfl_sync(0xffffffffu, xl, i);
+            const int b0 = __shfl_sync(0xffffffffu, gl.tn0, i), n0 = __shfl_sync(0xffffffffu, gl.n0, i);
+            int cb = 0, rr = 0, ss = 0;  // conv = 2: channel block and tap of block kb
+            for (int kb = 0; kb < kblocks; ++kb) {
+              // (the ring's first lap, whose slots are free, waits for nothing)
+              if (it >= S && !mbar_wait_warp(bar_empty + 8 * slot, ph ^ 1u, err, s_abort, kErrTimeoutEmpty, wlim)) {
+                ok = false;
+                break;
+              }
+              if (el) {
+                const uint32_t fb = bar_full + 8 * slot;
+                mbar_arrive_expect_tx(fb, bytes);
+                if (p.conv == 0)
+                  tma_load_2d(sA + slot * C::kAStage, &tmA, fb, kb * BK, y0);
+                else
+                  tma_load_4d(sA + slot * C::kAStage, &tmA, fb, cb * BK, x0 + ss, y0 + rr, b0);
+                if (!resident_b) tma_load_2d(sB + slot * C::kBStage, &tmB, fb, kb * BK, n0);
+              }
+              __syncwarp();
+              ++it;
+              if (++slot == S) {
+                slot = 0;
+                ph ^= 1u;
+              }
+              if (p.conv == 2 && ++cb == cb_per_tap) {
+                cb = 0;
+                if (++ss == p.kw) {
+                  ss = 0;
+                  ++rr;
+                }
+              }
+            }
+          }
+        }
+        if (lane == 0) *s_issued = it;  // stages this CTA filled (TMA copies issued)
+      }
+    } else {
     const int r = threadIdx.x;
     const int cb_per_tap = p.Cp / BK;
     int it = 0;        // stages filled so far (ring position)
@@ -356,7 +458,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // dense TMA modes: thread 0 issues everything, the other producer threads
     // have no part in the loop (their tile geometry would only take issue
     // slots from the epilogue warps on the same schedulers)
-    const bool lone = !skip && (LEAN || p.conv != 1);
+    const bool lone = !skip && p.conv != 1;
     for (int u = (lone && r != 0) ? units : (int)blockIdx.x; u < units; u += gridDim.x) {
       if (u != (int)blockIdx.x) ug = unit_geo(p, u, KS, kblocks, nt, BN, BK, r);
       const int kb0 = ug.kb0, kb1 = ug.kb1;
@@ -366,20 +468,20 @@ __global__ void __launch_bounds__(kThreads, 1)
       int last = kb1 - 1;
       if (skip) {
         // ---- occupied K blocks of this tile
-        named_bar_sync(1, 128);  // thread 0 is done with the previous tile's bits
+        named_bar_sync(1, kProdThreads);  // thread 0 is done with the previous tile's bits
         if (compact) {
           // occupied 32-column groups of this unit's K range in the tile's
           // 128-row block: one bit per group
           const int g0 = 2 * kb0, g1 = 2 * kb1 < kgroups ? 2 * kb1 : kgroups;
           const uint32_t* words = in_blk + (int64_t)(g.m0 >> 7) * in_C32;
-          for (int w0 = 0; w0 < kgroups && w0 < kMaxKWords * 32; w0 += 128) {
+          for (int w0 = 0; w0 < kgroups && w0 < kMaxKWords * 32; w0 += kProdThreads) {
             const int gi = w0 + r;
             const bool occ = gi >= g0 && gi < g1 && words[gi] != 0u;
             const uint32_t bits = __ballot_sync(0xffffffffu, occ);
             if (lane == 0 && (w0 >> 5) + warp < kMaxKWords) s_kbits[(w0 >> 5) + warp] = bits;
           }
         } else if (p.conv == 0) {
-          for (int w0 = 0; w0 < kblocks && w0 < kMaxKWords * 32; w0 += 128) {
+          for (int w0 = 0; w0 < kblocks && w0 < kMaxKWords * 32; w0 += kProdThreads) {
             const int kb = w0 + r;
             // a K block covers BK / 32 words of the 128-row block-column mask
             // (an input without block masks, such as the im2col rows of a
@@ -397,32 +499,38 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         } else {
           if (r < kMaxTaps) s_tap[r] = 0ull;
-          named_bar_sync(1, 128);
+          named_bar_sync(1, kProdThreads);
           const int taps = p.kh * p.kw < kMaxTaps ? p.kh * p.kw : kMaxTaps;
-          for (int t0 = 0; t0 < taps; t0 += 8) {
-            unsigned long long wv[8];
+          // (with 96 producer threads warp 0 takes the last 32 rows as well)
+          for (int row = r; row < kBM; row += kProdThreads) {
+            bool rv = rvalid;
+            int ri = img, ry = oh, rx = ow;
+            if (row != r) tile_row(p, g, row, rv, ri, ry, rx);
+            for (int t0 = 0; t0 < taps; t0 += 8) {
+              unsigned long long wv[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {  // issue 8 taps' loads before reducing any
-              const int tp = t0 + u;
-              const int ih = oh * p.stride - p.pad + tp / p.kw;
-              const int iw = ow * p.stride - p.pad + tp % p.kw;
-              wv[u] = 0ull;
-              if (in_rowbm && tp < taps && rvalid && ih >= 0 && ih < p.H && iw >= 0 && iw < p.W)
-                wv[u] = in_rowbm[(((int64_t)img * p.H + ih) * p.W + iw) * in_W64];
-            }
+              for (int u = 0; u < 8; ++u) {  // issue 8 taps' loads before reducing any
+                const int tp = t0 + u;
+                const int ih = ry * p.stride - p.pad + tp / p.kw;
+                const int iw = rx * p.stride - p.pad + tp % p.kw;
+                wv[u] = 0ull;
+                if (in_rowbm && tp < taps && rv && ih >= 0 && ih < p.H && iw >= 0 && iw < p.W)
+                  wv[u] = in_rowbm[(((int64_t)ri * p.H + ih) * p.W + iw) * in_W64];
+              }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              unsigned long long w = wv[u];
+              for (int u = 0; u < 8; ++u) {
+                unsigned long long w = wv[u];
 #pragma unroll
-              for (int s = 16; s > 0; s >>= 1) w |= __shfl_xor_sync(0xffffffffu, w, s);
-              if (lane == 0 && w) atomicOr(&s_tap[t0 + u], w);
+                for (int s = 16; s > 0; s >>= 1) w |= __shfl_xor_sync(0xffffffffu, w, s);
+                if (lane == 0 && w) atomicOr(&s_tap[t0 + u], w);
+              }
             }
           }
-          named_bar_sync(1, 128);
+          named_bar_sync(1, kProdThreads);
           // no per-tap masks (too many taps, wide rows, or an input given without
           // row bitmaps): keep every block
           const bool many = p.kh * p.kw > kMaxTaps || in_W64 > 1 || in_rowbm == nullptr;
-          for (int w0 = 0; w0 < kblocks && w0 < kMaxKWords * 32; w0 += 128) {
+          for (int w0 = 0; w0 < kblocks && w0 < kMaxKWords * 32; w0 += kProdThreads) {
             const int kb = w0 + r;
             bool occ = false;
             if (kb < kblocks) {
@@ -443,7 +551,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (lane == 0 && (w0 >> 5) + warp < kMaxKWords) s_kbits[(w0 >> 5) + warp] = bits;
           }
         }
-        named_bar_sync(1, 128);
+        named_bar_sync(1, kProdThreads);
         // last occupied block of this unit's K range; a range with none still
         // runs its first block (whose data is all zero)
         last = kb0;
@@ -610,6 +718,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       fence_proxy_async_smem();
       for (int q = pending; q > 0; --q) mbar_arrive(bar_full + 8 * ((it - q) % S));
     }
+    }
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------------ MMA issue
     // The warp stays converged; `el` (one lane) issues.  The ring position is
@@ -634,23 +743,24 @@ __global__ void __launch_bounds__(kThreads, 1)
     // One dense stage.  k-steps advance the start-address field by 32 B (2
     // units); the accumulate flag is a constant of each MMA (a flag computed
     // at run time roughly halves the issue rate).
-    auto stage = [&](uint32_t d, auto first) -> bool {
+    auto stage = [&](uint32_t d, uint64_t b0, auto first) -> bool {
       if (!mbar_wait_warp(bar_full + 8 * slot, ph, err, s_abort, kErrTimeoutFull, wlim)) return false;
       tc_fence_after();
       if (el) {
-        tc_mma_bf16(d, ad, bd, idesc, decltype(first)::value ? 0u : 1u);
+        tc_mma_bf16(d, ad, b0, idesc, decltype(first)::value ? 0u : 1u);
 #pragma unroll
-        for (int k = 1; k < BK / 16; ++k) tc_mma_bf16(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, 1u);
+        for (int k = 1; k < BK / 16; ++k) tc_mma_bf16(d, ad + (uint64_t)(2 * k), b0 + (uint64_t)(2 * k), idesc, 1u);
         tc_commit(bar_empty + 8 * slot);
       }
       __syncwarp();
       next();
       return true;
     };
-    bool ok = true;
+    bool ok = !resident_b || mbar_wait_warp(bar_resb, 0u, err, s_abort, kErrTimeoutFull, wlim);
+    if (resident_b) tc_fence_after();
     for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++j) {
-      const int b = j & 1;
-      if (!mbar_wait_warp(bar_acce + 8 * b, (uint32_t)(((j >> 1) & 1) ^ 1), err, s_abort, kErrTimeoutAcc, wlim))
+      const int b = j & (kAcc - 1);
+      if (!mbar_wait_warp(bar_acce + 8 * b, (uint32_t)(((j / kAcc) & 1) ^ 1), err, s_abort, kErrTimeoutAcc, wlim))
         break;
       tc_fence_after();
       const uint32_t d = tmem + (uint32_t)b * C::kAccCols;
@@ -658,8 +768,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         // every K block of the unit
         const int ks = KS == 1 ? 0 : u - (u / KS) * KS;
         const int n = KS == 1 ? kblocks : (ks + 1) * kblocks / KS - ks * kblocks / KS;
-        ok = stage(d, BoolConst<true>{});
-        for (int i = 1; i < n && ok; ++i) ok = stage(d, BoolConst<false>{});
+        ok = stage(d, resident_b ? bd0 : bd, BoolConst<true>{});
+        for (int i = 1; i < n && ok; ++i)
+          ok = stage(d, resident_b ? bd0 + (uint64_t)(i * (C::kBStage / 16)) : bd, BoolConst<false>{});
       } else {
         // the occupied ones: the producer marks a unit's last stage (bit 0)
         bool first = true, last = false;
@@ -708,15 +819,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ------------------------------------------------------------- lean epilogue
     // The general epilogue's blocks (32 rows of one TMEM lane quarter x 32
     // columns, staged with the 64-byte swizzle, one TMA store each) without
-    // K split or fp32 output, and with one barrier per tile: the
-    // output occupancy a tile leaves in shared memory (row bitmaps and block-
-    // column words, buffer j & 1) is written out after the next tile's
-    // barrier, and column counts go straight into the CTA's column sums.
+    // K split or fp32 output.  No barrier inside the tile loop: a warp waits
+    // for its tile's accumulator alone and writes its rows' bitmap words and
+    // its block-column words itself; column counts go straight into the CTA's
+    // column sums.  (With a barrier per tile the warps ran in lockstep, one
+    // block's latency, about 3400 cycles, per tile and round: 16 warps were no
+    // faster than 8.)
     const int q = warp & 3;
-    const int hf = (warp - 4) >> 2;
-    const int ew = warp - 4;
     const int r = q * 32 + lane;
-    const int et = threadIdx.x - 128;
+    const int lane_col = lane < 16 ? 2 * lane : 2 * lane - 31;  // column of bit `lane` in nz_mask32's order
+    const int ew = warp - kEpiWarp0;
+    const int slots = 4 / ncw;             // tiles in work at a time
+    const int slot = (ew >> 2) & (slots - 1);
+    const int cw = (ew >> 2) / slots;      // this warp's 32-column blocks: cw, cw + ncw, ...
     int sw_ = 0, sh_ = 0, sn_ = 0;
     if (p.conv == 2) {
       const int rho = q * 32;
@@ -724,85 +839,90 @@ __global__ void __launch_bounds__(kThreads, 1)
       sh_ = (rho / p.bw) % p.bh;
       sn_ = rho / (p.bw * p.bh);
     }
-    const uint32_t stg_base = sStg + (uint32_t)(ew * 2 * kWarpStgBytes);
-    const bool fixed_cols = nt == 1 || (int)gridDim.x % nt == 0 || units <= (int)gridDim.x;
-    if (fixed_cols && (int)blockIdx.x < units) {
+    const uint32_t stg = sStg + (uint32_t)(ew * kWarpStgBytes);
+    const bool affine = ep.bias != nullptr || ep.bn != nullptr;  // else the column affine is 1, 0
+    // The column affine: one table when every tile of the CTA has the same
+    // columns, else each warp computes a block's 32 columns ahead of it.
+    float* const own = s_scale + 2 * BN + ew * 64;  // this warp's block: scale[32], shift[32]
+    if (affine && fixed_cols) {
       const int n0 = ((int)blockIdx.x % nt) * BN;
-      for (int c = et; c < BN; c += kEpiThreads) {
+      for (int c = threadIdx.x - 128; c < BN; c += kEpiThreads) {
         float sc = 1.f, sh = 0.f;
         if (n0 + c < p.N) epi_affine(ep, p.N, n0 + c, sc, sh);
         s_scale[c] = sc;
         s_shift[c] = sh;
       }
+      named_bar_sync(2, kEpiThreads);
     }
-    const bool affine = ep.bias != nullptr || ep.bn != nullptr;  // else the column affine is 1, 0
     const OccDev o = P.out_occ;
-    // Writes out the occupancy that tile (m0, n0) left in buffer pb: the row
-    // bitmap word of row r (its half-0 thread) and the block-column words of
-    // its 128-row block (mode 0: the tile is that block).
-    auto flush_tile = [&](int pb, int64_t m_t, bool v_t, int m0_t, int n0_t) {
-      if (hf == 0) {
-        unsigned long long* const srow = s_rowbm + pb * kBM + r;
-        const unsigned long long v = *srow;
-        *srow = 0ull;
-        if (v_t) {
-          unsigned long long* dst = &o.row_bm[m_t * o.W64 + (n0_t >> 12)];
-          if (nt == 1) *dst = v;  // the tile spans the row's whole bitmap word
-          else if (v) atomicOr(dst, v);
+    // Column counts.  Up to 128-wide tiles (many small tiles per CTA): this
+    // warp's blocks cw, cw + ncw, ... are added bit-sliced, seven tiles in three
+    // planes in shared memory, before the planes are transposed.  Wider tiles:
+    // every block's bits are transposed.
+    constexpr bool kSliced = BN <= 128;
+    constexpr int kBpw = BN / 32;
+    uint32_t* const splane = reinterpret_cast<uint32_t*>(smem + C::kPlaneOff) + ew * (kBpw * 3 * 32) + lane;
+    if (kSliced && emit)
+#pragma unroll
+      for (int i = 0; i < kBpw * 3; ++i) splane[i * 32] = 0u;
+    int nsum = 0, n0_last = 0;
+    uint32_t pend_bits = 0u;  // block-column words on their way out
+    int pend_at = 0, npend = 0;
+    auto flush_words = [&]() {
+      if (lane < npend && pend_bits) atomicOr(&o.blk_mask[pend_at], nz_unpermute(pend_bits));
+      npend = 0;
+    };
+    auto flush_counts = [&](uint32_t (&pl)[3], int ncol0) {
+      // this lane's column (bit `lane` in nz_mask32's order): non-zeros in the warp's rows
+      uint32_t cnt = __popc(warp_transpose32(pl[0]));
+      if (kSliced && __any_sync(0xffffffffu, (pl[1] | pl[2]) != 0u))
+        cnt += 2u * __popc(warp_transpose32(pl[1])) + 4u * __popc(warp_transpose32(pl[2]));
+      pl[0] = pl[1] = pl[2] = 0u;
+      const int col = ncol0 + lane_col;
+      if (acc_smem) {
+        if (cnt) atomicAdd(&s_acc[col], cnt);
+      } else {
+        if (cnt) atomicAdd(&o.col_nnz[col], cnt);  // (columns past N have none)
+        const uint32_t sum = __reduce_add_sync(0xffffffffu, cnt);
+        if (lane == 0 && sum) {
+          atomicAdd(&o.tile_nnz[ncol0 >> 6], sum);
+          atomicAdd(o.nnz, (unsigned long long)sum);
         }
       }
-      if (p.conv != 2 && et < BN / 32) {
-        uint32_t* const sb = s_blk + pb * (BN / 32) + et;
-        const uint32_t v = *sb;
-        *sb = 0u;
-        const int word = (n0_t >> 5) + et;
-        if (word < o.C32) o.blk_mask[(m0_t >> 7) * o.C32 + word] = v;
-      }
     };
-    int j = 0;
-    int stg_count = 0;
-    int64_t m_prev = 0;
-    bool v_prev = false;
-    int m0_prev = 0, n0_prev = 0;
-    for (int u = blockIdx.x; u < units; u += gridDim.x, ++j) {
-      const int b = j & 1;
+    for (int j = slot;; j += slots) {
+      const int u = (int)blockIdx.x + j * (int)gridDim.x;
+      if (u >= units) break;
+      const int b = j & (kAcc - 1);
       const TileGeo g = tile_geo(p, u, nt, BN);
       bool mvalid;
       int img, oh, ow;
       const int64_t m = tile_row(p, g, r, mvalid, img, oh, ow);
+      const int ncb = p.N - g.n0 >= BN ? BN / 32 : (p.N - g.n0 + 31) >> 5;  // 32-column blocks of the tile
       if (LEAN == 2 && mvalid) {
         // this row's residual segments into L1 while the accumulator is pending
-        const __nv_bfloat16* rrow = residual + m * p.N + g.n0 + hf * 32;
-        for (int gc = 0; gc < BN / 64; ++gc)
-          if (g.n0 + gc * 64 + hf * 32 < p.N) prefetch_l1(rrow + gc * 64);
+        const __nv_bfloat16* rrow = residual + m * p.N + g.n0;
+        for (int c = cw; c < ncb; c += ncw) prefetch_l1(rrow + c * 32);
       }
-      float* const scb = s_scale + (fixed_cols ? 0 : b * BN);
-      float* const shb = s_shift + (fixed_cols ? 0 : b * BN);
-      if (!fixed_cols) {
-        for (int c = et; c < BN; c += kEpiThreads) {
-          float sc = 1.f, sh = 0.f;
-          if (g.n0 + c < p.N) epi_affine(ep, p.N, g.n0 + c, sc, sh);
-          scb[c] = sc;
-          shb[c] = sh;
-        }
-      }
-      const bool ok = mbar_wait(bar_accf + 8 * b, (uint32_t)((j >> 1) & 1), err, s_abort, kErrTimeoutAcc, wlim);
-      if (named_bar_or(2, kEpiThreads, !ok)) break;
-      if (emit && j > 0) flush_tile(b ^ 1, m_prev, v_prev, m0_prev, n0_prev);
-      tc_fence_after();
-      const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)b * C::kAccCols;
+      float nsc = 1.f, nsh = 0.f;  // the next block's affine of column `lane`
+      auto load_affine = [&](int cblk) {
+        const int c = g.n0 + cblk * 32 + lane;
+        if (cblk < ncb && c < p.N) epi_affine(ep, p.N, c, nsc, nsh);
+      };
+      if (affine && !fixed_cols) load_affine(cw);
       const int blk = mvalid ? (int)(m >> 7) : -1;
       const uint32_t grp = p.conv == 2 ? __match_any_sync(0xffffffffu, blk) : 0xffffffffu;
       const bool leader = (__ffs(grp) - 1) == lane;
-      unsigned long long tl = 0ull;
-      // One block: columns ncol0..+31 of 64-column group gcol, accumulator
-      // values in raw, staged in buffer stg; the TMA store and this block's
-      // share of the output occupancy.
-      auto block = [&](const uint32_t (&raw)[32], int gcol, uint32_t stg) {
-        const int nbase = g.n0 + gcol * 64;
-        const int ncol0 = nbase + hf * 32;
-        const float* scg = affine ? scb + gcol * 64 + hf * 32 : nullptr;
-        const float* shg = shb + gcol * 64 + hf * 32;
+      if (!mbar_wait_warp(bar_accf + 8 * b, (uint32_t)((j / kAcc) & 1), err, s_abort, kErrTimeoutAcc, wlim)) break;
+      tc_fence_after();
+      const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)b * C::kAccCols;
+      unsigned long long tl = 0ull;  // this row's occupied 64-column tiles
+      // One block: columns cblk * 32.. of the tile, accumulator values in raw;
+      // the TMA store and this block's share of the output occupancy.
+      auto block = [&](const uint32_t (&raw)[32], int cblk, uint32_t (&plane)[3]) {
+        const int ncol0 = g.n0 + cblk * 32;
+        const float* scg = !affine ? nullptr : fixed_cols ? s_scale + cblk * 32 : own;
+        const float* shg = fixed_cols ? s_shift + cblk * 32 : own + 32;
         const uint4* rp =
             residual && mvalid ? reinterpret_cast<const uint4*>(residual + m * p.N + ncol0) : nullptr;
         const int rvalid = p.N - ncol0 < 32 ? p.N - ncol0 : 32;
@@ -827,68 +947,86 @@ __global__ void __launch_bounds__(kThreads, 1)
           bulk_commit();
         }
         if (emit) {
-          uint32_t rw = nz_mask32(pk);  // bit c: column ncol0 + c of row r is non-zero
-          const int nvalid = p.N - ncol0;
+          // row r's non-zero bits, in nz_mask32's order
+          uint32_t rw = nz_mask32(pk);
           if (!mvalid) rw = 0u;
-          else if (nvalid < 32) rw &= nvalid > 0 ? ((1u << nvalid) - 1u) : 0u;
-          if (rw) tl |= 1ull << ((nbase >> 6) & 63);
+          else if (rvalid < 32) rw &= ((1u << (rvalid >> 1)) - 1u) * 0x00010001u;
+          if (rw) tl |= 1ull << ((ncol0 >> 6) & 63);
           const uint32_t bits = __reduce_or_sync(grp, rw);
           const int word = ncol0 >> 5;
-          if (leader && blk >= 0 && bits && word < o.C32) {
-            if (p.conv == 2) atomicOr(&o.blk_mask[blk * o.C32 + word], bits);
-            else atomicOr(&s_blk[b * (BN / 32) + gcol * 2 + hf], bits);  // the tile is the whole block
-          }
-          // lane c: non-zeros of column ncol0 + c in the warp's 32 rows
-          const uint32_t cnt = __popc(warp_transpose32(rw));
-          const int col = ncol0 + lane;
-          if (acc_smem) {
-            if (cnt) atomicAdd(&s_acc[col], cnt);
-          } else if (col < o.C) {
-            if (cnt) atomicAdd(&o.col_nnz[col], cnt);
-            const uint32_t sum = __reduce_add_sync(0xffffffffu, cnt);
-            if (lane == 0 && sum) {
-              atomicAdd(&o.tile_nnz[ncol0 >> 6], sum);
-              atomicAdd(o.nnz, (unsigned long long)sum);
+          if (p.conv == 2) {
+            if (leader && blk >= 0 && bits && word < o.C32)
+              atomicOr(&o.blk_mask[(int64_t)blk * o.C32 + word], nz_unpermute(bits));
+          } else {
+            // the tile is the whole block: its words wait, one per lane, and
+            // leave 32 at a time
+            if (lane == npend) {
+              pend_bits = bits;
+              pend_at = (g.m0 >> 7) * o.C32 + word;
             }
+            if (++npend == 32) flush_words();
           }
+          const uint32_t k1 = plane[0] & rw;
+          plane[0] ^= rw;
+          const uint32_t k2 = plane[1] & k1;
+          plane[1] ^= k1;
+          plane[2] |= k2;
         }
       };
-      // This warp's blocks of the tile (32-column halves past N have none).
       // (Two blocks per step, both accumulator loads in flight first, made
       // the kernel spill and was slower.)
-      int nblk = 0;
-      for (int gc = 0; gc < BN / 64; ++gc) nblk += (g.n0 + gc * 64 + hf * 32 < p.N) ? 1 : 0;
 #pragma unroll 1
-      for (int gcol = 0; gcol < nblk; ++gcol) {
-        const uint32_t stg = stg_base + (uint32_t)((stg_count & 1) * kWarpStgBytes);
-        if (lane == 0) bulk_wait_read<1>();  // the store that used this buffer has read it
-        __syncwarp();
+      for (int cblk = cw; cblk < ncb; cblk += ncw) {
         uint32_t raw[32];
-        tmem_ld32_nowait(tbase + (uint32_t)(gcol * 64 + hf * 32), raw);
+        tmem_ld32_nowait(tbase + (uint32_t)(cblk * 32), raw);
+        if (affine && !fixed_cols) {
+          own[lane] = nsc;
+          own[32 + lane] = nsh;
+          load_affine(cblk + ncw);
+        }
+        if (lane == 0) bulk_wait_read<0>();  // the last store from this buffer has read it
+        __syncwarp();
         tmem_wait_ld32(raw);
-        block(raw, gcol, stg);
-        ++stg_count;
+        if (cblk + ncw >= ncb) {  // accumulator b is free for the MMAs of tile j + kAcc
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_acce + 8 * b);
+        }
+        uint32_t* const sp = splane + (ncw == 1 ? cblk : 0) * 96;
+        uint32_t pl[3] = {0u, 0u, 0u};
+        if (kSliced && emit)
+#pragma unroll
+          for (int i = 0; i < 3; ++i) pl[i] = sp[i * 32];
+        block(raw, cblk, pl);
+        if (emit && (!kSliced || !fixed_cols || nsum == 6)) flush_counts(pl, g.n0 + cblk * 32);
+        if (kSliced && emit)
+#pragma unroll
+          for (int i = 0; i < 3; ++i) sp[i * 32] = pl[i];
       }
-      // accumulator b is free for the MMA of tile j + 2
-      tc_fence_before();
-      mbar_arrive(bar_acce + 8 * b);
-      if (emit) {
-        if (tl) atomicOr(&s_rowbm[b * kBM + r], tl);
-        m_prev = m;
-        v_prev = mvalid;
-        m0_prev = g.m0;
-        n0_prev = g.n0;
+      if (++nsum == 7) nsum = 0;
+      n0_last = g.n0;
+      if (cw >= ncb && lane == 0) mbar_arrive(bar_acce + 8 * b);  // no block of this tile
+      if (emit && mvalid) {
+        unsigned long long* dst = &o.row_bm[m * o.W64 + (g.n0 >> 12)];
+        if (nt == 1 && ncw == 1) *dst = tl;  // all columns of the row's bitmap word
+        else if (tl) atomicOr(dst, tl);
       }
     }
     if (emit) {
-      named_bar_sync(2, kEpiThreads);  // the last tile's shared-memory occupancy is complete
-      if (j > 0) flush_tile((j - 1) & 1, m_prev, v_prev, m0_prev, n0_prev);
+      flush_words();
+      if (kSliced && fixed_cols)
+        for (int k = 0; k < (ncw == 1 ? kBpw : 1); ++k) {
+          uint32_t pl[3];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) pl[i] = splane[k * 96 + i * 32];
+          flush_counts(pl, n0_last + (cw + k * ncw) * 32);
+        }
     }
     if (acc_smem) {
       named_bar_sync(2, kEpiThreads);
       unsigned long long total = 0ull;
       for (int c0 = 0; c0 < p.N; c0 += kEpiThreads) {
-        const int c = c0 + et;
+        const int c = c0 + (int)threadIdx.x - 128;
         const uint32_t cnt = c < p.N ? s_acc[c] : 0u;
         if (cnt) atomicAdd(&o.col_nnz[c], cnt);
         uint32_t sum = cnt;
@@ -929,8 +1067,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // same columns (one column tile, or a grid that is a multiple of the column
     // tiles) the column affine is computed once, into buffer 0, instead of per
     // tile (its global loads would otherwise sit on every tile's critical path)
-    const bool fixed_cols = KS == 1 && (nt == 1 || (int)gridDim.x % nt == 0 || units <= (int)gridDim.x);
-    if (fixed_cols && (int)blockIdx.x < units) {
+    const bool same_cols = KS == 1 && fixed_cols;
+    if (same_cols && (int)blockIdx.x < units) {
       const int n0 = ((int)blockIdx.x % nt) * BN;
       for (int c = et; c < BN; c += kEpiThreads) {
         float sc = 1.f, sh = 0.f;
@@ -948,11 +1086,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool mvalid;
       int img, oh, ow;
       const int64_t m = tile_row(p, g, r, mvalid, img, oh, ow);
-      float* const scb = s_scale + (fixed_cols ? 0 : b * BN);
-      float* const shb = s_shift + (fixed_cols ? 0 : b * BN);
+      float* const scb = s_scale + (same_cols ? 0 : b * BN);
+      float* const shb = s_shift + (same_cols ? 0 : b * BN);
       // column affine of this tile into buffer b (its readers of tile j - 2
       // passed tile j - 1's barrier before any thread gets here)
-      if (!fixed_cols) {
+      if (!same_cols) {
         for (int c = et; c < BN; c += kEpiThreads) {
           float sc = 1.f, sh = 0.f;
           if (g.n0 + c < p.N) epi_affine(ep, p.N, g.n0 + c, sc, sh);
@@ -1252,6 +1390,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // MMAs issued so far are done (each wait bounded again)
     if (threadIdx.x == 0) {
       const int issued = *s_issued;
+      if (resident_b) mbar_drain(bar_resb, 0u, wlim);
       for (int k = 0; k < S && k < issued; ++k) {
         const int i = issued - 1 - k;
         mbar_drain(bar_full + 8 * (i % S), (uint32_t)((i / S) & 1), wlim);
@@ -1265,7 +1404,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   if (warp == kMmaWarp) {
     tc_fence_after();
-    tmem_dealloc(tmem, C::kTmemCols);
+    tmem_dealloc(tmem, kTmemCols);
   }
 }
 
@@ -1335,7 +1474,7 @@ cudaError_t launch_cfg(const IgemmArgs& a, const CUtensorMap& tA, const CUtensor
   if (e0 != cudaSuccess) return e0;
   const int64_t units = tiles * (a.ksplit > 1 ? a.ksplit : 1);
   const int64_t grid = units < device_sm_count() ? units : device_sm_count();
-  cudaError_t e = launch_kernel(igemm_kernel<BN, BK, LEAN>, dim3((unsigned)grid), dim3(kThreads),
+  cudaError_t e = launch_kernel(igemm_kernel<BN, BK, LEAN>, dim3((unsigned)grid), dim3(Warps<LEAN>::kThreads),
                                 (size_t)Cfg<BN, BK>::kSmem, s, tA, tB, tY, tA32, tB32, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
@@ -1409,7 +1548,7 @@ void choose_tiles(const IgemmArgs& a, int64_t mtiles, int* bn_out, int* ks_out) 
   int64_t tiles = mtiles * ((a.N + bn - 1) / bn);
   if (bn == 128) {
     int64_t best = ((tiles + sms - 1) / sms) * (128 + 128);
-    for (int cand = 192; cand <= 256 && cand <= a.N; cand += 64) {
+    for (int cand = 192; cand <= 256 && cand < a.N + 64; cand += 64) {
       const int64_t t = mtiles * ((a.N + cand - 1) / cand);
       const int64_t cost = ((t + sms - 1) / sms) * (128 + cand);
       if (cost < best) {

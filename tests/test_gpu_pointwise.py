@@ -1,0 +1,54 @@
+"""Narrow 1x1 convolutions with many tiles per CTA (resident weights, bit-sliced
+column counts flushed every seven tiles, one epilogue warp per tile and lane
+quarter) against the oracle: one to six 32-column blocks, partial blocks, a last
+tile with few rows, tile counts at and around the flush period, every activation,
+residual, spatial (strided) tiles.  Counts and bitmaps bit for bit, values within
+the path's tolerance (bf16 rounding of the output, 2^-9)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as orc
+from paper_2511_19457_gb300 import synth
+from tests._parity import assert_close, assert_occ_equal
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sp():
+    from paper_2511_19457_gb300 import sparoa
+    return sparoa
+
+
+@pytest.fixture(scope="module")
+def ctx(sp):
+    c = sp.Context(0)
+    yield c
+    c.close()
+
+
+# rows = B H W; 152 CTAs x 4 warps per lane quarter x 7 tiles of 128 rows = 544,768 rows per flush period
+@pytest.mark.parametrize("B,H,W,C,Co,stride,act,res", [
+    (1, 700, 780, 16, 96, 1, 2, False), (1, 512, 1100, 8, 32, 1, 1, True), (1, 333, 501, 24, 144, 1, 2, False),
+    (1, 257, 300, 64, 24, 1, 0, True), (1, 200, 640, 160, 64, 1, 1, False), (1, 151, 257, 32, 192, 1, 3, False),
+    (3, 130, 131, 32, 40, 2, 1, False), (2, 160, 160, 64, 256, 1, 1, True)])
+@pytest.mark.parametrize("force", [1, 2])
+def test_pointwise(sp, ctx, B, H, W, C, Co, stride, act, res, force):
+    d = synth.conv_layer(seed=H + C, N=B, H=H, W=W, Cin=C, Cout=Co, k=1, stride=stride, pad=0, bn="random")
+    Ho, Wo = (H - 1) // stride + 1, (W - 1) // stride + 1
+    R = B * Ho * Wo
+    g = torch.Generator().manual_seed(3)
+    rb = synth.to_bf16_bits(torch.randn(R, Co, generator=g)) if res else None
+    y = torch.full((B, Ho, Wo, Co), float("nan"), dtype=torch.bfloat16, device="cuda")
+    yo = sp.OccupancyBuffer(R, Co)
+    yo.buf.fill_(0x5A)
+    x = sp.bits_to_device(d["x"]).view(B, H, W, C)
+    sp.sparoa_conv2d(ctx, x, sp.bits_to_device(d["w"]).view(Co, 1, 1, C), y, stride=stride, pad=0,
+                     bn=torch.from_numpy(d["bn"]).cuda(), act=act,
+                     residual=None if rb is None else sp.bits_to_device(rb).view(B, Ho, Wo, Co),
+                     thr=sp.thresholds(force_path=force), y_occ=yo)
+    assert ctx.last_path() == force
+    assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), R, Co), "occupancy")
+    ref = orc.conv2d(d["x"], B, H, W, C, d["w"], Co, 1, 1, stride, 0, bn=d["bn"], residual_bits=rb, act=act)
+    assert_close(y.float().cpu().numpy(), np.asarray(ref).reshape(y.shape), what="pointwise")
