@@ -599,8 +599,18 @@ __device__ __forceinline__ uint32_t nz_pairs(uint32_t w) {
 template <int ACT>
 __device__ __forceinline__ uint32_t act_pack2(float lo, float hi) {
   if (ACT == 3) {
-    lo = gelu_f(lo);
-    hi = gelu_f(hi);
+    // gelu_f on a packed pair: v (c0 + c1 v^2) in two FMAs and a product, then
+    // h + h tanh(.) with h = v / 2 (a GEMM epilogue with GELU and 256-wide tiles
+    // is bound by these instructions)
+    const f2_t v = f2(lo, hi), zero = f2(0.f, 0.f);
+    const f2_t v2 = ffma2(v, v, zero);
+    const f2_t u = ffma2(v, ffma2(v2, f2(0.0356774081f, 0.0356774081f), f2(0.7978845608f, 0.7978845608f)), zero);
+    float ul, uh, tl, th;
+    f2_split(u, ul, uh);
+    asm("tanh.approx.f32 %0, %1;" : "=f"(tl) : "f"(ul));
+    asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(uh));
+    const f2_t h = ffma2(v, f2(0.5f, 0.5f), zero);
+    f2_split(ffma2(h, f2(tl, th), h), lo, hi);
   }
   uint32_t d;
   if (ACT == 1 || ACT == 2)
