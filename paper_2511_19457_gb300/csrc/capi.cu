@@ -1167,9 +1167,15 @@ sparoa_status sparoa_layernorm(sparoa_ctx* ctx, const void* x, int64_t R, int64_
   if (!(eps >= 0.f)) return fail(ctx, SPAROA_ERR_INVALID_ARG, "layernorm: eps");
   SP_TRY(check_occ(ctx, y_occ, R, C, "layernorm y_occ"));
   DeviceGuard g(ctx->device, ctx->overlap);
+  const bool emit = y_occ && layernorm_emits((int)C);
+  OccDev o{};
+  if (emit) {
+    SP_TRY(occ_clear(ctx, *y_occ, true));
+    o = to_dev(*y_occ);
+  }
   SP_CUDA(launch_layernorm(static_cast<const __nv_bfloat16*>(x), R, (int)C, gamma_beta, eps,
-                           static_cast<__nv_bfloat16*>(y), ctx->stream));
-  if (y_occ) SP_TRY(run_stats(ctx, y, R, C, *y_occ));
+                           static_cast<__nv_bfloat16*>(y), o, emit ? 1 : 0, ctx->stream));
+  if (y_occ && !emit) SP_TRY(run_stats(ctx, y, R, C, *y_occ));
   return SPAROA_OK;
 }
 
@@ -1185,9 +1191,13 @@ sparoa_status sparoa_attention(sparoa_ctx* ctx, const void* qkv, int64_t N, int6
   const int64_t D = (int64_t)heads * head_dim;
   SP_TRY(check_occ(ctx, y_occ, N * T, D, "attention y_occ"));
   DeviceGuard g(ctx->device, ctx->overlap);
+  OccDev o{};
+  if (y_occ) {
+    SP_TRY(occ_clear(ctx, *y_occ));
+    o = to_dev(*y_occ);
+  }
   SP_CUDA(launch_attention(static_cast<const __nv_bfloat16*>(qkv), (int)N, (int)T, heads, head_dim,
-                           static_cast<__nv_bfloat16*>(y), ctx->stream));
-  if (y_occ) SP_TRY(run_stats(ctx, y, N * T, D, *y_occ));
+                           static_cast<__nv_bfloat16*>(y), o, y_occ ? 1 : 0, ctx->stream));
   return SPAROA_OK;
 }
 
@@ -1578,13 +1588,13 @@ sparoa_status sparoa_run_graph(sparoa_ctx* ctx, const sparoa_op* ops, int32_t n_
         break;
       case SPAROA_OP_LAYERNORM:
         SP_CUDA(launch_layernorm(static_cast<const __nv_bfloat16*>(act(op.input)), in.n * in.h * in.w,
-                                 (int)in.c, op.bn, op.bn_eps, static_cast<__nv_bfloat16*>(act(i + 1)),
-                                 ctx->stream));
+                                 (int)in.c, op.bn, op.bn_eps, static_cast<__nv_bfloat16*>(act(i + 1)), to_dev(*yo),
+                                 layernorm_emits((int)in.c) ? 1 : 0, ctx->stream));
         break;
       case SPAROA_OP_ATTENTION:
         SP_CUDA(launch_attention(static_cast<const __nv_bfloat16*>(act(op.input)), (int)in.n,
                                  (int)(in.h * in.w), op.groups, (int)(in.c / 3 / op.groups),
-                                 static_cast<__nv_bfloat16*>(act(i + 1)), ctx->stream));
+                                 static_cast<__nv_bfloat16*>(act(i + 1)), to_dev(*yo), 1, ctx->stream));
         break;
       case SPAROA_OP_TOKENS:
         SP_CUDA(launch_tokens(static_cast<const __nv_bfloat16*>(act(op.input)), (int)in.n,
@@ -1597,7 +1607,8 @@ sparoa_status sparoa_run_graph(sparoa_ctx* ctx, const sparoa_op* ops, int32_t n_
                               ctx->stream));
         break;
     }
-    if (op.kind >= SPAROA_OP_LAYERNORM) {
+    if (op.kind == SPAROA_OP_TOKENS || op.kind == SPAROA_OP_SELECT ||
+        (op.kind == SPAROA_OP_LAYERNORM && !layernorm_emits((int)in.c))) {
       // these kernels write no occupancy: the stats kernel measures the output
       // (the walk cleared every occupancy block when it started)
       SP_CUDA(launch_stats(static_cast<const __nv_bfloat16*>(act(i + 1)), out.n * out.h * out.w,

@@ -1153,33 +1153,47 @@ __global__ void __launch_bounds__(kTileThreads) dwconv_kernel(const DwArgs a_par
 }
 
 // ---------------------------------------------------------------------------
-// Global average pooling [N, HW, C] -> [N, C] (C % 8 == 0): one CTA per (image,
-// 64-channel slice).  Lane l of warp w sums pixels 4 w + l / 8 + 32 k of the 8
-// channels 8 (l % 8) .. + 7, so every load of the CTA is in flight at once;
-// the 32 pixel partial sums of a channel meet by shuffles and in shared
-// memory, and threads 0..63 finish one channel each: the mean, its bf16 value
-// and the output occupancy (atomics into the cleared block: row bit, column,
-// tile and total counts, block-column mask words).
+// Global average pooling [N, HW, C] -> [N, C] (C % 8 == 0): one cluster of 1 to
+// 8 CTAs per (image, 64-channel slice), which share its pixels, so that large
+// maps of few channels fill the chip ([32,56,56,64]: 32 CTAs, 29 us, before;
+// 256 CTAs now).  Lane l of warp w of CTA r sums pixels 32 r + 4 w + l / 8 + 32
+// S k of the 8 channels 8 (l % 8) .. + 7, four loads in flight; the partial sums
+// of a channel meet by shuffles, in shared memory and, in rank order, in the
+// first CTA's, whose threads 0..63 finish one channel each: the mean, its bf16
+// value and the output occupancy (atomics into the cleared block: row bit,
+// column, tile and total counts, block-column mask words).
 __global__ void __launch_bounds__(kTileThreads)
     avgpool_kernel(const __nv_bfloat16* __restrict__ x, int N, int HW, int C,
-                   __nv_bfloat16* __restrict__ y, OccDev o_param, int emit) {
+                   __nv_bfloat16* __restrict__ y, OccDev o_param, int emit, int S) {
   const OccDev o = o_param;
-  __shared__ float s_part[8 * 64];  // [warp][channel of the slice]
+  __shared__ float s_part[8 * 64];   // [warp][channel of the slice]
+  __shared__ float s_share[8 * 64];  // first CTA: [rank][channel of the slice]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int cg = lane & 7, pq = warp * 4 + (lane >> 3);  // channel group, pixel lane 0..31
   const int ctn = (C + 63) / 64;
-  const int n = (int)(blockIdx.x / ctn), ct = (int)(blockIdx.x - (blockIdx.x / ctn) * ctn);
+  const int slice = (int)blockIdx.x / S, rank = (int)blockIdx.x - slice * S;
+  const int n = slice / ctn, ct = slice - n * ctn;
   const int c0 = ct * 64 + cg * 8;
+  if (S > 1) cluster_arrive();  // (waited for below: every CTA of the cluster has started)
   pdl_wait();
   pdl_trigger();
   float a8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   if (c0 < C) {
     const __nv_bfloat16* p = x + (int64_t)n * HW * C + c0;
-    for (int q = pq; q < HW; q += 32) {
-      float f[8];
-      unpack8(__ldg(reinterpret_cast<const uint4*>(p + (int64_t)q * C)), f);
+    const int step = 32 * S;
+    for (int q = 32 * rank + pq; q < HW; q += 4 * step) {
+      uint4 u[4];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) a8[j] += f[j];
+      for (int i = 0; i < 4; ++i)
+        u[i] = q + i * step < HW ? __ldg(reinterpret_cast<const uint4*>(p + (int64_t)(q + i * step) * C))
+                                 : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float f[8];
+        unpack8(u[i], f);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) a8[j] += f[j];
+      }
     }
   }
   // lanes cg, cg + 8, cg + 16, cg + 24 of a warp hold the same channels
@@ -1193,11 +1207,25 @@ __global__ void __launch_bounds__(kTileThreads)
     for (int j = 0; j < 8; ++j) s_part[warp * 64 + lane * 8 + j] = a8[j];
   }
   __syncthreads();
+  if (S > 1) {
+    cluster_wait();
+    if (threadIdx.x < 64) {
+      float sum = 0.f;
+#pragma unroll
+      for (int w = 0; w < kTileThreads / 32; ++w) sum += s_part[w * 64 + threadIdx.x];
+      st_cluster_f32(cluster_map(smem_u32(s_share + rank * 64 + threadIdx.x), 0u), sum);
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    if (rank != 0) return;
+  }
   if (threadIdx.x < 64) {  // two full warps
     const int c = ct * 64 + (int)threadIdx.x;
+    const float* part = S > 1 ? s_share : s_part;
+    const int parts = S > 1 ? S : kTileThreads / 32;
     float sum = 0.f;
-#pragma unroll
-    for (int w = 0; w < kTileThreads / 32; ++w) sum += s_part[w * 64 + threadIdx.x];
+    for (int w = 0; w < parts; ++w) sum += part[w * 64 + threadIdx.x];
     const __nv_bfloat16 b = __float2bfloat16_rn(sum / (float)HW);
     const bool live = c < C;
     if (live) y[(int64_t)n * C + c] = b;
@@ -1383,8 +1411,14 @@ cudaError_t launch_avgpool(const __nv_bfloat16* x, int N, int HW, int C, __nv_bf
   if (C % 8) return cudaErrorInvalidValue;
   const int64_t ctas = (int64_t)N * ((C + 63) / 64);
   if (ctas >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
-  return launch_kernel(avgpool_kernel, dim3((unsigned)ctas), dim3(kTileThreads), 0, s, x, N, HW, C, y, o,
-                       emit);
+  // CTAs per slice: while two per SM are not reached and each keeps 64 pixels
+  // (two rounds of its pixel lanes; 7x7 maps stay whole)
+  int S = 1;
+  while (S < 8 && ctas * S * 2 <= 2 * device_sm_count() && HW >= 64 * S * 2) S *= 2;
+  if (S == 1)
+    return launch_kernel(avgpool_kernel, dim3((unsigned)ctas), dim3(kTileThreads), 0, s, x, N, HW, C, y, o, emit, 1);
+  return launch_cluster_kernel(avgpool_kernel, dim3((unsigned)(ctas * S)), dim3(kTileThreads), (unsigned)S, 0, s, x, N,
+                               HW, C, y, o, emit, S);
 }
 
 cudaError_t launch_bn_act(const __nv_bfloat16* x, int64_t R, int C, const EpiDev& ep,

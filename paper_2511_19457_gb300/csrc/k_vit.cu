@@ -2,8 +2,9 @@
 // ViT-B16): layer normalisation, multi-head self-attention, the token sequence
 // of a patch embedding, and token selection.  The token-wise linear layers of
 // a transformer are 1x1 convolutions over [N, 1, T, C] and run on the
-// threshold-dispatched GEMM path; these kernels are the rest.  Their outputs'
-// Eq. 1 statistics are measured by the stats kernel afterwards.
+// threshold-dispatched GEMM path; these kernels are the rest.  Layer norm (rows
+// of up to 1024 values) and attention emit their outputs' Eq. 1 statistics; the
+// others' are measured by the stats kernel afterwards.
 #include "sparoa_kernels.h"
 
 namespace sparoa {
@@ -14,10 +15,20 @@ constexpr int kVitThreads = 256;
 
 // ---------------------------------------------------------------------------
 // Layer normalisation: one warp per row of C values (C % 8 == 0), fp32: the
-// mean, then the mean square of the deviations.  Rows of up to 1024 values
-// are held in registers (every load of the row in flight at once, one pass
-// over memory); longer rows are re-read for each of the three steps.
-constexpr int kLnRegChunks = 4;  // 8-value chunks per lane held in registers
+// mean, then the mean square of the deviations.
+//
+// Rows of up to 1024 values (ln_rows_kernel): a warp takes a run of consecutive
+// rows; the row is held in registers (one pass over memory, the next row's
+// loads in flight while this one is reduced) and so are the lane's gamma and
+// beta, and the output's occupancy is emitted on the way: row bitmap words whole
+// (one word per row), block-column masks ORed over the run's rows of a 128-row
+// block, column counts in 16-bit register halves, added up in shared memory once
+// per CTA.  [6304, 768] with occupancy: 14.1 us + 9.5 us for a clear and a
+// statistics pass before (gamma and beta were re-read, value by value, for every
+// row).  Longer rows (layernorm_kernel) are re-read for each of the three steps.
+constexpr int kLnRegChunks = 4;     // 8-value chunks per lane held in registers
+constexpr int kLnCtasPerSm = 2;
+constexpr int kLnFlushRows = 16384;  // rows after which 16-bit counters are flushed
 
 __device__ __forceinline__ void ln_store(__nv_bfloat16* __restrict__ yr, const float* __restrict__ gb, int C,
                                          int c, float (&f)[8], float mean, float rstd) {
@@ -28,6 +39,172 @@ __device__ __forceinline__ void ln_store(__nv_bfloat16* __restrict__ yr, const f
     f[k] = v;
   }
   *reinterpret_cast<uint4*>(yr + c * 8) = pack8(f);
+}
+
+template <int NCH>
+__global__ void __launch_bounds__(kVitThreads, kLnCtasPerSm)
+    ln_rows_kernel(const __nv_bfloat16* __restrict__ x, int64_t R, int C, const float* __restrict__ gb, int gb_vec,
+                   float eps, __nv_bfloat16* __restrict__ y, OccDev o_param, int emit) {
+  const OccDev o = o_param;
+  __shared__ uint32_t s_cnt[NCH * 256];
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (kVitThreads / 32);
+  const int64_t w = (int64_t)blockIdx.x * (kVitThreads / 32) + (threadIdx.x >> 5);
+  const int64_t r0 = w * R / warps, r1 = (w + 1) * R / warps;
+  const int chunks = C / 8;
+  const float inv_c = 1.f / (float)C;
+  if (emit)
+    for (int c = threadIdx.x; c < NCH * 256; c += kVitThreads) s_cnt[c] = 0u;
+  pdl_wait();
+  pdl_trigger();
+  uint4 u[NCH];
+  auto load = [&](int64_t r) {
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      const int c = lane + 32 * i;
+      u[i] = c < chunks ? *reinterpret_cast<const uint4*>(x + r * C + c * 8) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  if (r0 < r1) load(r0);
+  float gam[NCH][8], bet[NCH][8];
+#pragma unroll
+  for (int i = 0; i < NCH; ++i) {
+    const int c = lane + 32 * i;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      gam[i][k] = 1.f;
+      bet[i][k] = 0.f;
+    }
+    if (gb && c < chunks) {
+      if (gb_vec) {
+#pragma unroll
+        for (int k = 0; k < 8; k += 4) {
+          const float4 g4 = *reinterpret_cast<const float4*>(gb + c * 8 + k);
+          const float4 b4 = *reinterpret_cast<const float4*>(gb + C + c * 8 + k);
+          gam[i][k] = g4.x; gam[i][k + 1] = g4.y; gam[i][k + 2] = g4.z; gam[i][k + 3] = g4.w;
+          bet[i][k] = b4.x; bet[i][k + 1] = b4.y; bet[i][k + 2] = b4.z; bet[i][k + 3] = b4.w;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          gam[i][k] = gb[c * 8 + k];
+          bet[i][k] = gb[C + c * 8 + k];
+        }
+      }
+    }
+  }
+  uint32_t cnt[NCH][4];  // non-zeros per column, 16-bit halves
+  uint32_t blk[NCH];     // this lane's 8 columns of the current 128-row block
+#pragma unroll
+  for (int i = 0; i < NCH; ++i) {
+    cnt[i][0] = cnt[i][1] = cnt[i][2] = cnt[i][3] = 0u;
+    blk[i] = 0u;
+  }
+  auto flush_cnt = [&]() {
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      const int c = (lane + 32 * i) * 8;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (cnt[i][k] & 0xFFFFu) atomicAdd(&s_cnt[c + 2 * k], cnt[i][k] & 0xFFFFu);
+        if (cnt[i][k] >> 16) atomicAdd(&s_cnt[c + 2 * k + 1], cnt[i][k] >> 16);
+        cnt[i][k] = 0u;
+      }
+    }
+  };
+  auto flush_blk = [&](int64_t b) {  // four lanes' masks are one 32-column word
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      uint32_t m = blk[i] << (8 * (lane & 3));
+      m |= __shfl_xor_sync(0xffffffffu, m, 1);
+      m |= __shfl_xor_sync(0xffffffffu, m, 2);
+      if ((lane & 3) == 0 && m) atomicOr(&o.blk_mask[b * o.C32 + ((lane + 32 * i) >> 2)], m);
+      blk[i] = 0u;
+    }
+  };
+  int since = 0;
+  for (int64_t r = r0; r < r1; ++r) {
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      float f[8];
+      unpack8(u[i], f);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s += f[k];
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+    const float mean = s * inv_c;
+    float q = 0.f;
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      if (lane + 32 * i < chunks) {
+        float f[8];
+        unpack8(u[i], f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) q = fmaf(f[k] - mean, f[k] - mean, q);
+      }
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) q += __shfl_xor_sync(0xffffffffu, q, d);
+    const float rstd = rsqrtf(q * inv_c + eps);
+    unsigned long long rowbits = 0ull;
+    uint4 v[NCH];
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) v[i] = u[i];
+    if (r + 1 < r1) load(r + 1);
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      const int c = lane + 32 * i;
+      uint32_t m8 = 0u;
+      if (c < chunks) {
+        float f[8];
+        unpack8(v[i], f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) f[k] = fmaf((f[k] - mean) * rstd, gam[i][k], bet[i][k]);
+        const uint4 out = pack8(f);
+        *reinterpret_cast<uint4*>(y + r * C + c * 8) = out;
+        if (emit) {
+          const uint32_t n0 = nz_pairs(out.x), n1 = nz_pairs(out.y), n2 = nz_pairs(out.z), n3 = nz_pairs(out.w);
+          cnt[i][0] += n0;
+          cnt[i][1] += n1;
+          cnt[i][2] += n2;
+          cnt[i][3] += n3;
+          const uint32_t t = n0 | (n1 << 2) | (n2 << 4) | (n3 << 6);  // even columns low, odd ones 16 up
+          m8 = (t | (t >> 15)) & 0xFFu;
+          blk[i] |= m8;
+        }
+      }
+      if (emit) {
+        // eight lanes' 64 columns are one bit of the row's word
+        const uint32_t any = __ballot_sync(0xffffffffu, m8 != 0u);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if ((any >> (8 * k)) & 0xFFu) rowbits |= 1ull << (4 * i + k);
+      }
+    }
+    if (emit) {
+      if (lane == 0) o.row_bm[r] = rowbits;  // (C <= 1024: one word per row)
+      if (((r + 1) & 127) == 0 || r + 1 == r1) flush_blk(r >> 7);
+      if (++since == kLnFlushRows) {
+        flush_cnt();
+        since = 0;
+      }
+    }
+  }
+  if (!emit) return;
+  flush_cnt();
+  __syncthreads();
+  unsigned long long total = 0ull;
+  for (int c0 = 0; c0 < C; c0 += kVitThreads) {  // (whole warps: a warp's 32 columns are half a tile)
+    const int c = c0 + threadIdx.x;
+    const uint32_t n = c < C ? s_cnt[c] : 0u;
+    if (n) atomicAdd(&o.col_nnz[c], n);
+    const uint32_t sum = __reduce_add_sync(0xffffffffu, n);
+    total += sum;
+    if (lane == 0 && sum) atomicAdd(&o.tile_nnz[c >> 6], sum);
+  }
+  if (lane == 0 && total) atomicAdd(o.nnz, total);
 }
 
 __global__ void __launch_bounds__(kVitThreads) layernorm_kernel(const __nv_bfloat16* __restrict__ x,
@@ -43,48 +220,6 @@ __global__ void __launch_bounds__(kVitThreads) layernorm_kernel(const __nv_bfloa
   for (int64_t r = (int64_t)blockIdx.x * (kVitThreads / 32) + (threadIdx.x >> 5); r < R; r += warps) {
     const __nv_bfloat16* xr = x + r * C;
     __nv_bfloat16* yr = y + r * C;
-    if (chunks <= 32 * kLnRegChunks) {
-      uint4 u[kLnRegChunks];
-#pragma unroll
-      for (int i = 0; i < kLnRegChunks; ++i) {
-        const int c = lane + 32 * i;
-        u[i] = c < chunks ? *reinterpret_cast<const uint4*>(xr + c * 8) : make_uint4(0u, 0u, 0u, 0u);
-      }
-      float s = 0.f;
-#pragma unroll
-      for (int i = 0; i < kLnRegChunks; ++i) {
-        float f[8];
-        unpack8(u[i], f);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) s += f[k];
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      const float mean = s * inv_c;
-      float q = 0.f;
-#pragma unroll
-      for (int i = 0; i < kLnRegChunks; ++i) {
-        if (lane + 32 * i < chunks) {
-          float f[8];
-          unpack8(u[i], f);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) q = fmaf(f[k] - mean, f[k] - mean, q);
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-      const float rstd = rsqrtf(q * inv_c + eps);
-#pragma unroll
-      for (int i = 0; i < kLnRegChunks; ++i) {
-        const int c = lane + 32 * i;
-        if (c < chunks) {
-          float f[8];
-          unpack8(u[i], f);
-          ln_store(yr, gb, C, c, f, mean, rstd);
-        }
-      }
-      continue;
-    }
     float s = 0.f;
     for (int c = lane; c < chunks; c += 32) {
       float f[8];
@@ -116,22 +251,32 @@ __global__ void __launch_bounds__(kVitThreads) layernorm_kernel(const __nv_bfloa
 // ---------------------------------------------------------------------------
 // Multi-head self-attention on the tensor cores (mma.sync m16n8k16, bf16 in,
 // fp32 accumulate), flash-attention style.  Input rows (one per token) hold
-// q | k | v, each heads x HD values.  One CTA per (image, head): the head's K
-// and V rows are copied once into shared memory by cp.async (row pitch HD + 8
-// elements, so the 8 rows of a fragment load fall in distinct banks; rows past
-// T up to the next multiple of 16 zero-filled), then the 4 warps take the
-// 16-query tiles in turn.  When the (image, head) pairs are fewer than the
-// resident CTAs, each pair's query tiles are split over gridDim.y CTAs (each
-// stages K and V itself).  A warp walks the keys in blocks of 64: S = Q K^T
-// (Q fragments in registers, K fragments read as pairs of consecutive
-// dimensions), an online softmax per query row (running maximum and sum,
-// rescaling the output), and O += P V with P taken straight from the S
-// accumulators (their layout is the A-operand layout of the next MMA) and the
-// V fragments read by ldmatrix.trans from the row-major V.  Key tiles wholly
-// at or past T are not computed.  O / sum is stored as bf16.
-constexpr int kAttnThreads = 128;  // 4 warps
+// q | k | v, each heads x HD values.  A CTA of 7 warps takes 7 16-query tiles of
+// one (image, head): the head's K and V rows are copied once into shared memory
+// by cp.async (row pitch HD + 8 elements, so the 8 rows of a fragment load fall
+// in distinct banks; rows past T up to the next multiple of 16 zero-filled),
+// then every warp does its tile.  (One CTA of 4 warps per (image, head), each
+// warp three or four tiles in turn, left 12 warps per SM and a last round half
+// empty: [32,197,12x64] 34 us.)  A warp walks the keys in blocks of 64: S = Q K^T
+// (Q fragments in registers, K fragments by ldmatrix), an online softmax per
+// query row (running maximum and sum, rescaling the output), and O += P V with P
+// taken straight from the S accumulators (their layout is the A-operand layout
+// of the next MMA) and the V fragments read by ldmatrix.trans from the row-major
+// V.  Key tiles wholly at or past T are not computed.  O / sum is stored as bf16,
+// and the output's occupancy is emitted: row bits by quads, the block-column
+// masks of a 16-query tile (rows of one 128-row block) by shuffles, column
+// counts in 16-bit register halves.
+constexpr int kAttnWarps = 7;
+constexpr int kAttnThreads = 32 * kAttnWarps;
 constexpr int kAttnMaxT = 512;
 constexpr int kAttnKB = 64;        // keys per block
+
+// 2^x; results below the normal range are zero (they are probabilities)
+__device__ __forceinline__ float exp2_ftz(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                                uint32_t b1) {
@@ -152,14 +297,28 @@ __device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t& r0, uint3
                : "memory");
 }
 
+// the same without the transposition, and two matrices
+__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void ldsm_x2(uint32_t addr, uint32_t& r0, uint32_t& r1) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr) : "memory");
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 template <int HD>
-__global__ void __launch_bounds__(kAttnThreads, 3) attention_kernel(const __nv_bfloat16* __restrict__ qkv, int T,
-                                                                    int heads, __nv_bfloat16* __restrict__ y) {
+__global__ void __launch_bounds__(kAttnThreads, 2)
+    attention_kernel(const __nv_bfloat16* __restrict__ qkv, int T, int heads, __nv_bfloat16* __restrict__ y,
+                     OccDev o_param, int emit) {
+  const OccDev occ = o_param;
+  __shared__ uint32_t s_cnt[HD];
   extern __shared__ __align__(16) uint8_t smem[];
   constexpr int KP = HD + 8;  // row pitch of K and V (elements)
   const int T16 = (T + 15) & ~15;
@@ -168,6 +327,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attention_kernel(const __nv_b
   const int n = blockIdx.x / heads, h = blockIdx.x - (blockIdx.x / heads) * heads;
   const int D = heads * HD, row3 = 3 * D;
   const __nv_bfloat16* base = qkv + (int64_t)n * T * row3;
+  if (threadIdx.x < HD) s_cnt[threadIdx.x] = 0u;
   pdl_wait();
   pdl_trigger();
   // K and V rows of the head: 16-byte copies, all in flight at once
@@ -189,10 +349,15 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attention_kernel(const __nv_b
   // 8-15), (keys 8-15, dims 8-15) -> b0, b1 of one 8-dimension n-tile, then
   // b0, b1 of the next
   const uint32_t v_lane = smem_u32(sV) + (uint32_t)(((lane & 15) * KP + (lane >> 4) * 8) * 2);
+  // K fragments of 8 keys: matrices (dims 0-7, 8-15) of one k-step, then of the next
+  const uint32_t k_lane = smem_u32(sK) + (uint32_t)(((lane & 7) * KP + (lane >> 3) * 8) * 2);
   const int qtn = (T + 15) >> 4;  // 16-query tiles
   const int per = (qtn + (int)gridDim.y - 1) / (int)gridDim.y;
   const int qt_end = min(qtn, ((int)blockIdx.y + 1) * per);
-  for (int qt = (int)blockIdx.y * per + warp; qt < qt_end; qt += 4) {
+  uint32_t cnt[HD / 8];  // non-zeros of columns 8 j + 2 tq, + 1 (16-bit halves)
+#pragma unroll
+  for (int j = 0; j < HD / 8; ++j) cnt[j] = 0u;
+  for (int qt = (int)blockIdx.y * per + warp; qt < qt_end; qt += kAttnWarps) {
     const int q0 = qt * 16;
     // Q fragments (A operand, rows g and g + 8, HD / 16 k-steps), zero past T
     uint32_t qa[HD / 16][4];
@@ -220,12 +385,19 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attention_kernel(const __nv_b
       for (int nt = 0; nt < kAttnKB / 8; ++nt) {
         s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
         if (kb + nt * 8 < T) {  // uniform across the warp
-          const __nv_bfloat16* kr = sK + (kb + nt * 8 + g) * KP + 2 * tq;
+          const uint32_t ka = k_lane + (uint32_t)((kb + nt * 8) * KP * 2);
+          if constexpr (HD >= 32) {
 #pragma unroll
-          for (int kk = 0; kk < HD / 16; ++kk) {
-            const uint32_t b0 = *reinterpret_cast<const uint32_t*>(kr + kk * 16);
-            const uint32_t b1 = *reinterpret_cast<const uint32_t*>(kr + kk * 16 + 8);
-            mma_bf16_16816(s[nt], qa[kk], b0, b1);
+            for (int kk = 0; kk < HD / 16; kk += 2) {
+              uint32_t b0, b1, b2, b3;
+              ldsm_x4(ka + (uint32_t)(kk * 32), b0, b1, b2, b3);
+              mma_bf16_16816(s[nt], qa[kk], b0, b1);
+              mma_bf16_16816(s[nt], qa[kk + 1], b2, b3);
+            }
+          } else {
+            uint32_t b0, b1;
+            ldsm_x2(ka, b0, b1);
+            mma_bf16_16816(s[nt], qa[0], b0, b1);
           }
         }
       }
@@ -250,15 +422,20 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attention_kernel(const __nv_b
       bm1 = fmaxf(bm1, __shfl_xor_sync(0xffffffffu, bm1, 1));
       bm1 = fmaxf(bm1, __shfl_xor_sync(0xffffffffu, bm1, 2));
       const float nm0 = fmaxf(m0, bm0), nm1 = fmaxf(m1, bm1);
-      const float c0 = exp2f((m0 - nm0) * sl2), c1 = exp2f((m1 - nm1) * sl2);
+      const float c0 = exp2_ftz((m0 - nm0) * sl2), c1 = exp2_ftz((m1 - nm1) * sl2);
       m0 = nm0;
       m1 = nm1;
       float rs0 = 0.f, rs1 = 0.f;
       uint32_t pa[kAttnKB / 16][4];  // P as A fragments of the P V MMAs
 #pragma unroll
       for (int nt = 0; nt < kAttnKB / 8; ++nt) {
-        const float p0 = exp2f((s[nt][0] - nm0) * sl2), p1 = exp2f((s[nt][1] - nm0) * sl2);
-        const float p2 = exp2f((s[nt][2] - nm1) * sl2), p3 = exp2f((s[nt][3] - nm1) * sl2);
+        float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
+        if (kb + nt * 8 < T) {  // uniform across the warp
+          p0 = exp2_ftz((s[nt][0] - nm0) * sl2);
+          p1 = exp2_ftz((s[nt][1] - nm0) * sl2);
+          p2 = exp2_ftz((s[nt][2] - nm1) * sl2);
+          p3 = exp2_ftz((s[nt][3] - nm1) * sl2);
+        }
         rs0 += p0 + p1;
         rs1 += p2 + p3;
         pa[nt >> 1][(nt & 1) * 2 + 0] = pack_bf16x2(p0, p1);
@@ -296,13 +473,70 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attention_kernel(const __nv_b
     l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
     const float i0 = 1.f / l0, i1 = 1.f / l1;
     const int r0 = q0 + g, r1 = q0 + g + 8;
+    const int64_t g0 = (int64_t)n * T + r0, g1 = (int64_t)n * T + r1;  // output rows
+    unsigned long long nz0 = 0ull, nz1 = 0ull;  // non-zero columns of rows r0, r1 among this lane's
 #pragma unroll
     for (int j = 0; j < HD / 8; ++j) {
       const int c = h * HD + j * 8 + 2 * tq;
-      if (r0 < T)
-        *reinterpret_cast<uint32_t*>(y + ((int64_t)n * T + r0) * D + c) = pack_bf16x2(o[j][0] * i0, o[j][1] * i0);
-      if (r1 < T)
-        *reinterpret_cast<uint32_t*>(y + ((int64_t)n * T + r1) * D + c) = pack_bf16x2(o[j][2] * i1, o[j][3] * i1);
+      const uint32_t w0 = pack_bf16x2(o[j][0] * i0, o[j][1] * i0), w1 = pack_bf16x2(o[j][2] * i1, o[j][3] * i1);
+      if (r0 < T) *reinterpret_cast<uint32_t*>(y + g0 * D + c) = w0;
+      if (r1 < T) *reinterpret_cast<uint32_t*>(y + g1 * D + c) = w1;
+      if (emit) {
+        const uint32_t n0 = r0 < T ? nz_pairs(w0) : 0u, n1 = r1 < T ? nz_pairs(w1) : 0u;
+        cnt[j] += n0 + n1;
+        nz0 |= (unsigned long long)((n0 | (n0 >> 15)) & 3u) << (8 * j + 2 * tq);
+        nz1 |= (unsigned long long)((n1 | (n1 >> 15)) & 3u) << (8 * j + 2 * tq);
+      }
+    }
+    if (emit) {
+      // a quad holds a row's HD columns
+#pragma unroll
+      for (int d = 1; d <= 2; d <<= 1) {
+        nz0 |= __shfl_xor_sync(0xffffffffu, nz0, d);
+        nz1 |= __shfl_xor_sync(0xffffffffu, nz1, d);
+      }
+      const int tile = (h * HD) >> 6;
+      const unsigned long long bit = 1ull << (tile & 63);
+      if (tq == 0 && nz0) atomicOr(&occ.row_bm[g0 * occ.W64 + (tile >> 6)], bit);
+      if (tq == 0 && nz1) atomicOr(&occ.row_bm[g1 * occ.W64 + (tile >> 6)], bit);
+      // block-column words: HD columns from h HD on
+      auto mask_out = [&](unsigned long long m, int64_t b) {
+        const int c = h * HD, sh = c & 31;
+        const uint32_t lo = (uint32_t)m << sh, hi = HD > 32 ? (uint32_t)(m >> 32) : 0u;  // (HD = 64: sh = 0)
+        if (lo) atomicOr(&occ.blk_mask[b * occ.C32 + (c >> 5)], lo);
+        if (hi) atomicOr(&occ.blk_mask[b * occ.C32 + (c >> 5) + 1], hi);
+      };
+      const int64_t t0 = (int64_t)n * T + q0;
+      if ((t0 >> 7) == ((t0 + 15) >> 7)) {  // the tile's rows share a 128-row block
+        unsigned long long m = nz0 | nz1;
+#pragma unroll
+        for (int d = 4; d <= 16; d <<= 1) m |= __shfl_xor_sync(0xffffffffu, m, d);
+        if (lane == 0) mask_out(m, t0 >> 7);
+      } else if (tq == 0) {
+        if (nz0) mask_out(nz0, g0 >> 7);
+        if (nz1) mask_out(nz1, g1 >> 7);
+      }
+    }
+  }
+  if (!emit) return;
+#pragma unroll
+  for (int j = 0; j < HD / 8; ++j) {  // (at most 512 rows: no carry between the halves)
+    uint32_t v = cnt[j];
+#pragma unroll
+    for (int d = 4; d <= 16; d <<= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    if (g == 0) {
+      if (v & 0xFFFFu) atomicAdd(&s_cnt[8 * j + 2 * tq], v & 0xFFFFu);
+      if (v >> 16) atomicAdd(&s_cnt[8 * j + 2 * tq + 1], v >> 16);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 64) {  // (HD columns: whole warps, or half of one)
+    const uint32_t v = threadIdx.x < HD ? s_cnt[threadIdx.x] : 0u;
+    if (v) atomicAdd(&occ.col_nnz[h * HD + threadIdx.x], v);
+    const uint32_t sum = __reduce_add_sync(0xffffffffu, v);
+    if (lane == 0 && sum) {
+      atomicAdd(&occ.tile_nnz[(h * HD) >> 6], sum);
+      atomicAdd(occ.nnz, (unsigned long long)sum);
     }
   }
 }
@@ -368,42 +602,54 @@ namespace {
 
 template <int HD>
 cudaError_t launch_attention_hd(const __nv_bfloat16* qkv, int N, int T, int heads, __nv_bfloat16* y,
-                                cudaStream_t s) {
+                                const OccDev& o, int emit, cudaStream_t s) {
   const size_t smem = attention_smem(T, HD);
   if (smem > 40 * 1024) {
     cudaError_t e = smem_optin(reinterpret_cast<const void*>(attention_kernel<HD>), smem);
     if (e != cudaSuccess) return e;
   }
-  // split the query tiles while the (image, head) pairs leave resident CTA
-  // slots (3 per SM) empty, down to one tile per warp
-  const int pairs = N * heads;
-  const int qsplit_max = ((T + 15) / 16 + 3) / 4;
-  int qsplit = 3 * device_sm_count() / pairs;
-  qsplit = qsplit < 1 ? 1 : (qsplit > qsplit_max ? qsplit_max : qsplit);
-  dim3 grid((unsigned)pairs, (unsigned)qsplit);
-  return launch_kernel(attention_kernel<HD>, grid, dim3(kAttnThreads), smem, s, qkv, T, heads, y);
+  // a query tile per warp
+  const int qsplit = ((T + 15) / 16 + kAttnWarps - 1) / kAttnWarps;
+  return launch_kernel(attention_kernel<HD>, dim3((unsigned)(N * heads), (unsigned)qsplit), dim3(kAttnThreads), smem, s,
+                       qkv, T, heads, y, o, emit);
 }
 
 }  // namespace
 
 cudaError_t launch_attention(const __nv_bfloat16* qkv, int N, int T, int heads, int hd, __nv_bfloat16* y,
-                             cudaStream_t s) {
+                             const OccDev& o, int emit, cudaStream_t s) {
   if (N <= 0 || T <= 0) return cudaSuccess;
   if (T > kAttnMaxT || heads <= 0) return cudaErrorInvalidValue;
   switch (hd) {
-    case 16: return launch_attention_hd<16>(qkv, N, T, heads, y, s);
-    case 32: return launch_attention_hd<32>(qkv, N, T, heads, y, s);
-    case 64: return launch_attention_hd<64>(qkv, N, T, heads, y, s);
+    case 16: return launch_attention_hd<16>(qkv, N, T, heads, y, o, emit, s);
+    case 32: return launch_attention_hd<32>(qkv, N, T, heads, y, o, emit, s);
+    case 64: return launch_attention_hd<64>(qkv, N, T, heads, y, o, emit, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
+bool layernorm_emits(int C) { return C <= 8 * 32 * kLnRegChunks; }
+
 cudaError_t launch_layernorm(const __nv_bfloat16* x, int64_t R, int C, const float* gb, float eps,
-                             __nv_bfloat16* y, cudaStream_t s) {
+                             __nv_bfloat16* y, const OccDev& o, int emit, cudaStream_t s) {
   if (R <= 0) return cudaSuccess;
   if (C % 8) return cudaErrorInvalidValue;
-  return launch_kernel(layernorm_kernel, dim3(grid_for(R, kVitThreads / 32)), dim3(kVitThreads), 0, s, x, R,
-                       C, gb, eps, y);
+  if (!layernorm_emits(C)) {
+    if (emit) return cudaErrorInvalidValue;
+    return launch_kernel(layernorm_kernel, dim3(grid_for(R, kVitThreads / 32)), dim3(kVitThreads), 0, s, x, R, C, gb,
+                         eps, y);
+  }
+  // a warp per row up to the resident warps, then runs of rows
+  const int64_t ctas = (R + kVitThreads / 32 - 1) / (kVitThreads / 32);
+  const int64_t cap = (int64_t)kLnCtasPerSm * device_sm_count();
+  const dim3 grid((unsigned)(ctas < cap ? ctas : cap));
+  const int vec = (reinterpret_cast<uintptr_t>(gb) & 15u) == 0;  // (C % 8 == 0: beta's rows too)
+  switch ((C + 255) / 256) {
+    case 1: return launch_kernel(ln_rows_kernel<1>, grid, dim3(kVitThreads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
+    case 2: return launch_kernel(ln_rows_kernel<2>, grid, dim3(kVitThreads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
+    case 3: return launch_kernel(ln_rows_kernel<3>, grid, dim3(kVitThreads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
+    default: return launch_kernel(ln_rows_kernel<4>, grid, dim3(kVitThreads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
+  }
 }
 
 cudaError_t launch_tokens(const __nv_bfloat16* x, int N, int P, int D, const __nv_bfloat16* cls,

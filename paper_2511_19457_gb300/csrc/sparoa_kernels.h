@@ -179,12 +179,15 @@ cudaError_t launch_fcsmall(const FcSkipArgs& a, cudaStream_t s);
 // Vision-transformer operators (k_vit.cu)
 // ----------------------------------------------------------------------------
 // y[r, :] = LN(x[r, :]) over C (C % 8 == 0); gb fp32 [2][C] gamma, beta or NULL.
+// emit (only where layernorm_emits(C)): also y's occupancy into `o`, whose row
+// bitmaps are written whole and whose other fields must be zero on entry.
+bool layernorm_emits(int C);
 cudaError_t launch_layernorm(const __nv_bfloat16* x, int64_t R, int C, const float* gb, float eps,
-                             __nv_bfloat16* y, cudaStream_t s);
+                             __nv_bfloat16* y, const OccDev& o, int emit, cudaStream_t s);
 // qkv [N, T, 3 D] (q | k | v per token, D = heads * hd) -> y [N, T, D];
-// T <= 512, hd 16, 32 or 64.
+// T <= 512, hd 16, 32 or 64; emit: also y's occupancy into the cleared block `o`.
 cudaError_t launch_attention(const __nv_bfloat16* qkv, int N, int T, int heads, int hd, __nv_bfloat16* y,
-                             cudaStream_t s);
+                             const OccDev& o, int emit, cudaStream_t s);
 size_t attention_smem(int T, int hd);
 // x [N, P, D] -> y [N, 1 + P, D]: class token row, then the patches; + pos [1 + P][D].
 cudaError_t launch_tokens(const __nv_bfloat16* x, int N, int P, int D, const __nv_bfloat16* cls,

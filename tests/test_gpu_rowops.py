@@ -1,0 +1,89 @@
+"""Layer norm, attention and global average pooling at the edges of their work
+splits: runs of rows around 128-row blocks, rows of one to five register chunks,
+parameters off a 16-byte boundary, query tiles around a CTA's seven and around
+block seams, pooling by clusters of 1 to 8 CTAs; occupancy bit for bit.  Values:
+bf16 output rounding 2^-9 (attention: the probabilities' too), fp32 sums."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as orc
+from paper_2511_19457_gb300 import synth
+from tests._parity import assert_close, assert_occ_equal
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sp():
+    from paper_2511_19457_gb300 import sparoa
+    return sparoa
+
+
+@pytest.fixture(scope="module")
+def ctx(sp):
+    c = sp.Context(0)
+    yield c
+    c.close()
+
+
+def _bits(shape, seed, zero_p=0.3):
+    g = torch.Generator().manual_seed(seed)
+    v = torch.randn(*shape, generator=g)
+    v[torch.rand(*shape, generator=g) < zero_p] = 0.0
+    return synth.to_bf16_bits(v)
+
+
+@pytest.mark.parametrize("R,C", [(1, 8), (127, 64), (129, 256), (5000, 264), (6304, 768), (2500, 1024), (300, 1032),
+                                 (20001, 200)])
+@pytest.mark.parametrize("params", ["none", "aligned", "off"])
+def test_layernorm(sp, ctx, R, C, params):
+    xb = _bits((R, C), R + C)
+    xb.reshape(R, C)[R // 2] = 0  # a constant row
+    gb = None
+    if params != "none":
+        g = torch.Generator().manual_seed(C)
+        gb = np.stack([1 + 0.1 * torch.randn(C, generator=g).numpy(), np.zeros(C)]).astype(np.float32)
+        gb[:, ::3] = 0.0  # whole columns of zeros
+    t = None
+    if gb is not None:
+        buf = torch.zeros(2 * C + 1, dtype=torch.float32, device="cuda")
+        t = buf[1:] if params == "off" else buf[:-1]
+        t.copy_(torch.from_numpy(gb).reshape(-1))
+    y = torch.full((R, C), float("nan"), dtype=torch.bfloat16, device="cuda")
+    yo = sp.OccupancyBuffer(R, C)
+    yo.buf.fill_(0x77)
+    sp.sparoa_layernorm(ctx, sp.bits_to_device(xb).view(R, C), y, gamma_beta=t, y_occ=yo)
+    yb = sp.device_to_bits(y)
+    assert_occ_equal(yo.to_host(), orc.stats(yb.reshape(-1), R, C), f"layernorm {R}x{C}")
+    assert_close(y.float().cpu().numpy(), orc.layernorm(xb, R, C, gb, 1e-6), what=f"layernorm {R}x{C}")
+
+
+@pytest.mark.parametrize("N,T,heads,hd", [(1, 1, 1, 64), (3, 16, 2, 64), (2, 112, 3, 64), (5, 113, 2, 32), (2, 128, 4, 16),
+                                          (3, 129, 1, 64), (2, 225, 5, 32), (1, 512, 2, 64), (2, 197, 12, 64)])
+@pytest.mark.parametrize("emit", [True, False])
+def test_attention(sp, ctx, N, T, heads, hd, emit):
+    D = heads * hd
+    qb = _bits((N, T, 3 * D), T + D, 0.0)
+    q = qb.reshape(N, T, 3 * D)
+    q[:, :, 2 * D: 2 * D + 3] = 0  # three zero columns of v
+    y = torch.full((N, T, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+    yo = sp.OccupancyBuffer(N * T, D) if emit else None
+    if emit:
+        yo.buf.fill_(0x11)
+    sp.sparoa_attention(ctx, sp.bits_to_device(qb).view(N, T, 3 * D), y, heads, y_occ=yo)
+    if emit:
+        assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), N * T, D), "attention")
+    assert_close(y.float().cpu().numpy(), orc.attention(qb, N, T, heads, hd), what=f"attention {N} {T} {heads} {hd}")
+
+
+@pytest.mark.parametrize("N,H,W,C", [(1, 127, 1, 8), (1, 128, 1, 64), (2, 37, 41, 72), (32, 56, 56, 64), (1, 224, 224, 16),
+                                     (150, 20, 20, 128), (3, 7, 7, 1280)])
+def test_avgpool(sp, ctx, N, H, W, C):
+    xb = _bits((N, H, W, C), H + C)
+    xb.reshape(N, H, W, C)[..., ::5] = 0
+    y = torch.empty(N, C, dtype=torch.bfloat16, device="cuda")
+    yo = sp.OccupancyBuffer(N, C)
+    sp.sparoa_avgpool_global(ctx, sp.bits_to_device(xb).view(N, H, W, C), y, y_occ=yo)
+    assert_close(y.float().cpu().numpy(), orc.avgpool_global(xb, N, H, W, C), what="avgpool")
+    assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), N, C), "avgpool")
