@@ -541,6 +541,7 @@ struct ConvPlan {
   // the epilogue's parameters and the conv (IgemmArgs::early)
   int early = 0;
   int early_w = 0;  // the same of w and the epilogue's parameters (IgemmArgs::early_w)
+  StemGeo stem;     // the kernel builds its A tiles from stem.x (1 x 1 conv over kh * seg channels)
 };
 
 sparoa_status run_conv(sparoa_ctx* ctx, const ConvPlan& c) {
@@ -578,6 +579,7 @@ sparoa_status run_conv(sparoa_ctx* ctx, const ConvPlan& c) {
   a.fault = ctx->fault == 1 ? kFaultSkipFirstAccCommit : 0;
   a.early = c.early;
   a.early_w = c.early_w;
+  a.stem = c.stem;
   if (!pointwise && conv3_supported(a)) {
     SP_CUDA(launch_conv3(a, ctx->stream));
     return SPAROA_OK;
@@ -1045,7 +1047,23 @@ sparoa_status sparoa_conv2d(sparoa_ctx* ctx, const void* x, int64_t N, int64_t H
       c.w = w;
       int ckh = kh, ckw = kw, cstride = stride, cpad = pad;
       bool cols = false;
-      if (im2col_applies((int)C_in, kh, kw, groups, (int)W, pad)) {
+      if (stem_plan(static_cast<const __nv_bfloat16*>(x), N, (int)H, (int)W, (int)C_in, (int)C_out, kh, kw, stride, pad,
+                    &c.stem)) {
+        // a narrow stem as a GEMM whose A tiles the kernel builds from x; its
+        // weights with each kernel row padded to seg columns
+        const int seg = c.stem.seg;
+        SP_TRY(ensure(ctx, ctx->pad_w, (size_t)(C_out * kh * seg * 2)));
+        SP_CUDA(launch_pad_channels(static_cast<const __nv_bfloat16*>(w), C_out * kh, kw * (int)C_in, seg,
+                                    static_cast<__nv_bfloat16*>(ctx->pad_w.p), ctx->stream));
+        c.w = ctx->pad_w.p;
+        c.H = Ho;
+        c.W = Wo;
+        c.Cin = kh * seg;
+        c.Cp = c.Cin;
+        ckh = ckw = cstride = 1;
+        cpad = 0;
+        cols = true;
+      } else if (im2col_applies((int)C_in, kh, kw, groups, (int)W, pad)) {
         // a narrow stem as a GEMM of its im2col rows (a 1 x 1 conv over Kp channels)
         const int Kp = im2col_width((int)C_in, kh, kw);
         SP_TRY(ensure(ctx, ctx->pad_x, (size_t)(N * Ho * Wo * Kp * 2)));
@@ -1084,7 +1102,7 @@ sparoa_status sparoa_conv2d(sparoa_ctx* ctx, const void* x, int64_t N, int64_t H
       c.ep = to_dev(ep);
       c.y = y;
       c.xo = xo;
-      if (cols) {  // the im2col rows have no occupancy: every K block is kept
+      if (cols) {  // the windows' rows have no occupancy: every K block is kept
         c.xo.blk_mask = nullptr;
         c.xo.row_bm = nullptr;
       }
@@ -1235,6 +1253,7 @@ struct Aux {
   size_t padx = 0, padw = 0, fcocc = 0;
   int64_t cp = 0;
   bool cols = false;  // narrow stem as a GEMM of its im2col rows (im2col_applies)
+  bool stem = false;  // ... whose A tiles the kernel builds (stem_plan)
   bool fc_view = false;
 };
 struct GraphPlan {
@@ -1273,7 +1292,11 @@ sparoa_status plan_graph(sparoa_ctx* ctx, const sparoa_op* ops, int32_t n_ops, i
                op.c_out};
         if (out.h <= 0 || out.w <= 0)
           return fail(ctx, SPAROA_ERR_INVALID_ARG, "run_graph: op %d empty output", i);
-        if (!dw && im2col_applies(op.c_in, op.kh, op.kw, op.groups, (int)in.w, op.pad)) {
+        StemGeo sg;
+        if (!dw && stem_plan(nullptr, in.n, (int)in.h, (int)in.w, op.c_in, op.c_out, op.kh, op.kw, op.stride, op.pad, &sg)) {
+          aux[(size_t)i].stem = true;
+          aux[(size_t)i].cp = op.kh * sg.seg;
+        } else if (!dw && im2col_applies(op.c_in, op.kh, op.kw, op.groups, (int)in.w, op.pad)) {
           aux[(size_t)i].cols = true;
           aux[(size_t)i].cp = im2col_width(op.c_in, op.kh, op.kw);
         } else if (!dw && op.c_in % 8) {
@@ -1365,7 +1388,10 @@ sparoa_status plan_graph(sparoa_ctx* ctx, const sparoa_op* ops, int32_t n_ops, i
     off += align_up((size_t)(vals[v].n * vals[v].h * vals[v].w * vals[v].c) * 2);
   }
   for (int i = 0; i < n_ops; ++i) {
-    if (aux[(size_t)i].cols) {
+    if (aux[(size_t)i].stem) {
+      aux[(size_t)i].padw = off;
+      off += align_up((size_t)(ops[i].c_out * aux[(size_t)i].cp) * 2);
+    } else if (aux[(size_t)i].cols) {
       const Val& out = vals[(size_t)i + 1];
       aux[(size_t)i].padx = off;
       off += align_up((size_t)(out.n * out.h * out.w * aux[(size_t)i].cp) * 2);
@@ -1489,8 +1515,19 @@ sparoa_status sparoa_run_graph(sparoa_ctx* ctx, const sparoa_op* ops, int32_t n_
         c.Cp = aux[(size_t)i].cp ? aux[(size_t)i].cp : in.c;
         c.x = act(op.input);
         c.w = op.weight;
-        const bool cols = aux[(size_t)i].cols;
-        if (cols) {  // a narrow stem as a GEMM of its im2col rows (a 1 x 1 conv over Kp channels)
+        const bool cols = aux[(size_t)i].cols || aux[(size_t)i].stem;
+        if (aux[(size_t)i].stem) {  // a narrow stem as a GEMM whose A tiles the kernel builds
+          if (!stem_plan(static_cast<const __nv_bfloat16*>(c.x), in.n, (int)in.h, (int)in.w, op.c_in, op.c_out, op.kh,
+                         op.kw, op.stride, op.pad, &c.stem))
+            return fail(ctx, SPAROA_ERR_UNSUPPORTED, "run_graph: op %d stem", i);
+          void* pw = base + aux[(size_t)i].padw;
+          SP_CUDA(launch_pad_channels(static_cast<const __nv_bfloat16*>(op.weight), (int64_t)op.c_out * op.kh,
+                                      op.kw * op.c_in, c.stem.seg, static_cast<__nv_bfloat16*>(pw), ctx->stream));
+          c.w = pw;
+          c.H = out.h;
+          c.W = out.w;
+          c.Cin = c.Cp;
+        } else if (cols) {  // a narrow stem as a GEMM of its im2col rows (a 1 x 1 conv over Kp channels)
           void* px = base + aux[(size_t)i].padx;
           void* pw = base + aux[(size_t)i].padw;
           SP_CUDA(launch_im2col(static_cast<const __nv_bfloat16*>(c.x), (int)in.n, (int)in.h, (int)in.w, (int)in.c,
@@ -1524,7 +1561,7 @@ sparoa_status sparoa_run_graph(sparoa_ctx* ctx, const sparoa_op* ops, int32_t n_
         c.ep = ep;
         c.y = act(i + 1);
         c.xo = xo;
-        if (cols) {  // the im2col rows have no occupancy: every K block is kept
+        if (cols) {  // the windows' rows have no occupancy: every K block is kept
           c.xo.blk_mask = nullptr;
           c.xo.row_bm = nullptr;
         }

@@ -15,8 +15,12 @@
 //           one 4-D TMA box {BK channels, bw, bh, bn} of the NHWC input at the
 //           shifted, strided origin (element strides = conv stride) is the A
 //           tile; out-of-range coordinates read zeros, which is the padding.
-//   mode 1  convolution, any C % 8 == 0 (the RGB stem): 128 consecutive output
-//           pixels, gathered by 128 producer threads with cp.async.
+//   mode 1  convolution, any C % 8 == 0: 128 consecutive output pixels,
+//           gathered by 128 producer threads with cp.async.
+//   stem    C < 8 (the RGB input), N <= 64: 128 consecutive output pixels, built
+//           in shared memory from the input rows ([32,224,224,3] 7x7/2 -> 64 with
+//           statistics and occupancy: 103 -> 60 us a call; im2col rows in memory
+//           cost 44 us to write and 26 us to read back).
 // K advances in BK-wide blocks: BK = 64 with the 128-byte swizzle (four
 // tcgen05.mma of K = 16 per stage) or BK = 32 with the 64-byte swizzle.
 //
@@ -61,29 +65,35 @@ namespace sparoa {
 namespace {
 
 constexpr int kMaxSplit = 4;  // K split: at most this many units per output tile
-constexpr int kEpiWarp0 = 4;  // first epilogue warp
 // Warp roles.  The general kernel: 4 producer warps (all 128 threads gather in
 // mode 1), 8 epilogue warps (two per TMEM lane quarter), the MMA warp.  The
 // lean ones: 3 producer warps, the MMA warp, 16 epilogue warps -- 5 warps per
 // scheduler, which leaves 96 registers a thread (a 21st warp would leave 80 and
-// spill).
-template <int LEAN>
+// spill).  Stems, whose producers build the A tiles: 7 producer warps, the MMA
+// warp, 8 epilogue warps.
+template <int LEAN, bool STEM = false>
 struct Warps {
-  static constexpr int kProd = LEAN ? 3 : 4;
-  static constexpr int kEpi = LEAN ? 16 : 8;
+  static constexpr int kProd = STEM ? 7 : LEAN ? 3 : 4;
+  static constexpr int kEpi = LEAN && !STEM ? 16 : 8;
   static constexpr int kEpiThreads = 32 * kEpi;
-  static constexpr int kMma = LEAN ? 3 : kEpiWarp0 + kEpi;
-  static constexpr int kThreads = 32 * (LEAN ? 20 : 13);
+  static constexpr int kEpi0 = STEM ? 8 : 4;  // first epilogue warp (a multiple of 4: its lane quarter)
+  static constexpr int kMma = STEM ? 7 : LEAN ? 3 : kEpi0 + kEpi;
+  static constexpr int kThreads = 32 * (STEM ? 16 : LEAN ? 20 : 13);
 };
 constexpr int kMaxKWords = 128;  // K-block occupancy bits: up to 4096 blocks
 constexpr int kMaxTaps = 64;
 constexpr int kStgBytes = 2 * 128 * 128;  // output staging: 32 rows x 64 bytes per epilogue warp (two each in the general kernel)
 constexpr int kWarpStgBytes = 32 * 64;
-constexpr int kMaxAccCols = 4096;     // per-CTA column counters (output occupancy)
+constexpr int kMaxAccColsGemm = 4096;  // per-CTA column counters (output occupancy)
+constexpr int kMaxStemRows = 48;      // input rows staged per tile (stem)
+constexpr int kStemRowBytes = 24 * 1024;  // ... and their bytes, per buffer
 
-template <int BN, int BK>
+// STEM: a stage is the whole A tile (three 64-wide K blocks), two of them; the
+// weights' three K blocks stay; two buffers of staged input rows follow.
+template <int BN, int BK, bool STEM = false>
 struct Cfg {
-  static constexpr int kAStage = kBM * BK * 2;
+  static constexpr int kMaxAccCols = STEM ? 64 : kMaxAccColsGemm;
+  static constexpr int kAStage = (STEM ? 3 : 1) * kBM * BK * 2;
   static constexpr int kBStage = BN * BK * 2;
   static constexpr int kStageBytes = kAStage + kBStage;
   // Stage ring: about 200 KB of shared memory in all; a deeper ring made the
@@ -101,11 +111,11 @@ struct Cfg {
   static constexpr int kBudget =
       BN == 192 ? 227 * 1024 - kFixed : 200 * 1024 - kStgBytes - 6 * 1024 - kMaxAccCols * 4;
   static constexpr int kStagesRaw = kBudget / kStageBytes;
-  static constexpr int kStages = kStagesRaw > 12 ? 12 : kStagesRaw;
+  static constexpr int kStages = STEM ? 2 : kStagesRaw > 12 ? 12 : kStagesRaw;
   static constexpr int kLag = kStages - 2;  // cp.async stages in flight (mode 1)
   static constexpr int kAOff = 0;
   static constexpr int kBOff = kAOff + kStages * kAStage;
-  static constexpr int kStgOff = kBOff + kStages * kBStage;          // 1024-aligned
+  static constexpr int kStgOff = kBOff + (STEM ? 3 : kStages) * kBStage;  // 1024-aligned
   static constexpr int kBarOff = kStgOff + kStgBytes;
   static constexpr int kNumBars = 2 * kStages + 10;                  // full, empty, accf[4], acce[4], drain, resident B
   static constexpr int kFlagOff = kBarOff + kNumBars * 8;
@@ -119,7 +129,11 @@ struct Cfg {
   // [16 warps][BN / 32 blocks][3 planes][32] bit-sliced column counts (lean, BN <= 128)
   static constexpr int kPlaneOff = (kBlkOff + (BN / 32) * 4 + 15) & ~15;
   static constexpr int kPlaneBytes = BN <= 128 ? 16 * (BN / 32) * 3 * 128 : 0;
-  static constexpr int kBytes = kPlaneOff + kPlaneBytes + 16;
+  // staged input rows [2][kStemRowBytes], per-tile tables [2]: row origins, pixel offsets
+  static constexpr int kStemOff = (kPlaneOff + kPlaneBytes + 127) & ~127;
+  static constexpr int kStemTabOff = kStemOff + 2 * kStemRowBytes;
+  static constexpr int kStemTab = kMaxStemRows * 4 + kBM * 4;
+  static constexpr int kBytes = STEM ? kStemTabOff + 2 * kStemTab : kPlaneOff + kPlaneBytes + 16;
   static constexpr int kSmem = kBytes + 1024;  // slack for 1024-byte alignment
   // TMEM: accumulator b starts at column b * kAccCols (BN rounded up to a
   // power of two, so each starts on a power-of-two column); the allocation
@@ -243,16 +257,23 @@ template <bool B>
 struct BoolConst {
   static constexpr bool value = B;
 };
+template <int I>
+struct IntConst {
+  static constexpr int value = I;
+};
 
-template <int BN, int BK, int LEAN>
-__global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
+template <int BN, int BK, int LEAN, bool STEM>
+__global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
     igemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmA32,
                  const __grid_constant__ CUtensorMap tmB32, const IgemmArgs P) {
-  using C = Cfg<BN, BK>;
-  constexpr int kEpiThreads = Warps<LEAN>::kEpiThreads;
-  constexpr int kMmaWarp = Warps<LEAN>::kMma;
-  constexpr int kProd = Warps<LEAN>::kProd, kProdThreads = 32 * kProd;
+  using C = Cfg<BN, BK, STEM>;
+  constexpr int kMaxAccCols = C::kMaxAccCols;
+  using Wp = Warps<LEAN, STEM>;
+  constexpr int kEpiThreads = Wp::kEpiThreads;
+  constexpr int kMmaWarp = Wp::kMma;
+  constexpr int kProd = Wp::kProd, kProdThreads = 32 * kProd;
+  constexpr int kEpiWarp0 = Wp::kEpi0, kEpiThread0 = 32 * kEpiWarp0;
   // accumulators in tensor memory: tiles in flight between the MMAs and the epilogue
   constexpr int kAcc = LEAN && BN <= 128 ? 4 : 2;
   constexpr uint32_t kTmemCols = kAcc * C::kAccCols;
@@ -261,6 +282,7 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
   // producers only (mode 0 or 2), no K split, bf16 output (the host launches
   // them only then)
   if (LEAN) __builtin_assume(p.conv != 1);
+  if (STEM) __builtin_assume(p.conv == 0);
   const EpiDev ep = P.ep;
   const int act = P.ep.act;
   const __nv_bfloat16* const residual = LEAN == 1 ? nullptr : P.ep.residual;
@@ -321,7 +343,8 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
   // take every 4th tile each; with two (192- and 256-wide tiles), and where the
   // CTA has one tile, they share a tile's 32-column blocks.  ncw: warps that
   // share a quarter of a tile.
-  const int ncw = kAcc == 2 || units <= (int)gridDim.x ? 4 : 1;
+  constexpr int kQw = Wp::kEpi / 4;  // epilogue warps per lane quarter
+  const int ncw = kAcc == 2 || units <= (int)gridDim.x ? kQw : 1;
 
   if (!LEAN && P.dense_only) {
     // launched next to the fused small-FC kernel, which handles the zero-skip
@@ -334,7 +357,7 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
   }
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
-      mbar_init(bar_full + 8 * s, (!LEAN && p.conv == 1) ? 129u : 1u);
+      mbar_init(bar_full + 8 * s, STEM ? (uint32_t)kProd : (!LEAN && p.conv == 1) ? 129u : 1u);
       mbar_init(bar_empty + 8 * s, 1u);
     }
     for (int b = 0; b < kAcc; ++b) {
@@ -345,9 +368,9 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
     mbar_init(bar_resb, 1u);
     *s_abort = 0;
     fence_mbar_init();
-    if (p.conv != 1) prefetch_tmap(&tmA);
+    if (p.conv != 1 && !STEM) prefetch_tmap(&tmA);
     prefetch_tmap(&tmB);
-    if (p.conv == 0 && BK == 64) {
+    if (p.conv == 0 && BK == 64 && !STEM) {
       prefetch_tmap(&tmA32);
       prefetch_tmap(&tmB32);
     }
@@ -356,10 +379,10 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
   if (warp == kMmaWarp) tmem_alloc(smem_u32(s_tmem), kTmemCols);
   const bool epi_warp = warp >= kEpiWarp0 && (LEAN || warp < kMmaWarp);
   if (acc_smem && epi_warp)
-    for (int c = threadIdx.x - 128; c < p.N; c += kEpiThreads) s_acc[c] = 0u;
+    for (int c = threadIdx.x - kEpiThread0; c < p.N; c += kEpiThreads) s_acc[c] = 0u;
   if (!LEAN && epi_warp) {
-    for (int i = threadIdx.x - 128; i < kBM; i += kEpiThreads) s_rowbm[i] = 0ull;
-    for (int i = threadIdx.x - 128; i < BN / 32; i += kEpiThreads) s_blk[i] = 0u;
+    for (int i = threadIdx.x - kEpiThread0; i < kBM; i += kEpiThreads) s_rowbm[i] = 0ull;
+    for (int i = threadIdx.x - kEpiThread0; i < BN / 32; i += kEpiThreads) s_blk[i] = 0u;
   }
   // The producers' first work unit is laid out before the grid dependency
   // wait: no memory is read, and under programmatic dependent launch this
@@ -376,7 +399,7 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
   // with dense_only the zero-skip kernel of this launch runs instead
   const bool run = !(!LEAN && P.dense_only && path == 2);
   if (run) record_path(P.disp, path);
-  const bool skip = (path == 2);
+  const bool skip = !STEM && path == 2;  // (a stem's tiles hold every K block)
   // zero-skip GEMM with 64-wide K blocks: stages hold two occupied 32-column
   // groups each (compacted), loaded as 32-column boxes with the 64-byte swizzle
   const bool compact = skip && p.conv == 0 && BK == 64 && kgroups <= kMaxKWords * 32 && in_blk != nullptr;
@@ -386,13 +409,148 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
   // ... and, on the dense path, a K range that fits the ring: its B blocks are
   // loaded once and stay, and the ring carries A alone (a 1x1 expansion
   // [32,112,112,16] -> 96 spent 11 of 53 us on reloading its 12 KB of weights per tile)
-  const bool resident_b = LEAN && !skip && fixed_cols && kblocks <= S && units > (int)gridDim.x;
+  const bool resident_b =
+      STEM || (LEAN && !skip && fixed_cols && kblocks <= S && units > (int)gridDim.x);
 
   if (!run) {
     // nothing to do; fall through to the common exit (TMEM is freed there)
   } else if (warp < kProd) {
     // ------------------------------------------------------------------ producers
-    if (LEAN && !skip) {
+    if constexpr (STEM) {
+      // The A tiles of a stem: K column kr * seg + e of pixel (n, oh, ow) is
+      // element e of the kw * C window of input row oh * stride - pad + kr, which
+      // is contiguous in NHWC.  A tile's input rows are staged by cp.async (the
+      // next tile's while this one is built), as the 16-byte chunks that hold
+      // them, so that row v starts at lead + (its misalignment); columns outside
+      // the image are zeros around the data, rows outside are zero rows.  One
+      // lane builds one pixel's window of one kernel row: words by a funnel
+      // shift (a window may start on an odd element), 16-byte chunks out.  All
+      // seven warps do both in turn: with the staging left to one warp the tile
+      // waited for it (71 us against 62 on [32,224,224,3] 7x7/2).
+      const StemGeo G = P.stem;
+      const int tid = threadIdx.x;
+      uint8_t* const rowbuf = smem + C::kStemOff;
+      const int row_elems = G.W * G.C;
+      const int wlen = G.kw * G.C, sc = G.stride * G.C, pad_c = G.pad * G.C;
+      const int nseg = G.seg >> 3;
+      const uint32_t xmis = (uint32_t)((reinterpret_cast<uintptr_t>(G.x) >> 1) & 7);  // elements past a 16-byte boundary
+      if (warp == 0 && elect_one()) {
+        mbar_arrive_expect_tx(bar_resb, (uint32_t)(kblocks * C::kBStage));
+        for (int kb = 0; kb < kblocks; ++kb) tma_load_2d(sB + kb * C::kBStage, &tmB, bar_resb, kb * BK, 0);
+      }
+      // zeros everywhere: the margins stay, and the K columns past kh * seg
+      for (int i = tid; i < 2 * kStemRowBytes / 16; i += kProdThreads)
+        reinterpret_cast<uint4*>(rowbuf)[i] = make_uint4(0u, 0u, 0u, 0u);
+      for (int i = tid; i < S * C::kAStage / 16; i += kProdThreads)
+        reinterpret_cast<uint4*>(smem + C::kAOff)[i] = make_uint4(0u, 0u, 0u, 0u);
+      named_bar_sync(1, kProdThreads);
+      const int chunks = (row_elems + 14) >> 3;  // of a row, whatever its misalignment
+      // requests the rows of tile u into buffer b (a warp a row) and writes its tables
+      auto stage_rows = [&](int u, int b) {
+        int* const s_row = reinterpret_cast<int*>(smem + C::kStemTabOff + b * C::kStemTab);  // window origin of row v
+        uint32_t* const s_pix = reinterpret_cast<uint32_t*>(s_row + kMaxStemRows);
+        const int m0 = u * kBM;
+        const int m1 = m0 + kBM < p.M ? m0 + kBM : p.M;
+        const int g0 = (int)__umulhi((uint32_t)m0, G.wo_mul) >> G.wo_shift, ow0 = m0 - g0 * G.Wo;  // m0 / Wo
+        const int span = (int)(__umulhi((uint32_t)(ow0 + m1 - m0 - 1), G.wo_mul) >> G.wo_shift) + 1;  // output rows of the tile
+        const int n0 = (int)__umulhi((uint32_t)g0, G.ho_mul) >> G.ho_shift, oh0 = g0 - n0 * G.Ho;
+        const int ka = G.Ho - oh0 < span ? G.Ho - oh0 : span;  // ... of them in image n0
+        const int rows_a = G.kh + (ka - 1) * G.stride;
+        const int rows = rows_a + (span > ka ? G.kh + (span - ka - 1) * G.stride : 0);
+        const uint32_t dst0 = smem_u32(rowbuf + b * kStemRowBytes);
+        for (int v = warp; v < rows; v += kProd) {
+          const bool second = v >= rows_a;
+          const int ih = second ? v - rows_a - G.pad : oh0 * G.stride - G.pad + v;
+          const bool live = ih >= 0 && ih < G.H;
+          const int64_t e0 = ((int64_t)(n0 + (second ? 1 : 0)) * G.H + (live ? ih : 0)) * row_elems;  // element of x
+          const int mis = (int)((uint32_t)e0 + xmis) & 7;
+          const __nv_bfloat16* src = G.x + e0 - mis;
+          const uint32_t dst = dst0 + (uint32_t)((v * G.pitch + G.lead) * 2);
+          const int end = live ? mis + row_elems : 0;  // elements from the first chunk's start
+          for (int c = lane; c < chunks; c += 32) {
+            const int left = end - 8 * c;
+            cp_async_16(dst + 16u * c, left > 0 ? src + 8 * c : src, left >= 8 ? 16u : left > 0 ? (uint32_t)(2 * left) : 0u);
+          }
+          if (lane == 0) s_row[v] = v * G.pitch + G.lead + (live ? mis : 0) - pad_c;
+        }
+        if (tid < kBM) {
+          const int at = ow0 + (m0 + tid < m1 ? tid : m1 - 1 - m0);
+          const int k = (int)__umulhi((uint32_t)at, G.wo_mul) >> G.wo_shift, ow = at - k * G.Wo;
+          s_pix[tid] = ((uint32_t)(k < ka ? k * G.stride : rows_a + (k - ka) * G.stride) << 24) | (uint32_t)(ow * sc);
+        }
+      };
+      // what a window's last chunk keeps of its four words
+      uint32_t keep[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int have = wlen - (8 * (nseg - 1) + 2 * i);
+        keep[i] = have >= 2 ? 0xFFFFFFFFu : have == 1 ? 0xFFFFu : 0u;
+      }
+      int it = 0;
+      bool ok = true;
+      if ((int)blockIdx.x < units) stage_rows(blockIdx.x, 0);
+      cp_async_commit();
+      for (int u = blockIdx.x; u < units; u += gridDim.x, ++it) {
+        const int b = it & 1, slot = it & 1;
+        if (u + (int)gridDim.x < units) stage_rows(u + gridDim.x, b ^ 1);
+        cp_async_commit();
+        cp_async_wait<1>();
+        named_bar_sync(1, kProdThreads);  // this tile's rows and tables are complete
+        const int* const s_row = reinterpret_cast<const int*>(smem + C::kStemTabOff + b * C::kStemTab);
+        const uint32_t* const s_pix = reinterpret_cast<const uint32_t*>(s_row + kMaxStemRows);
+        if (G.ragged && G.pad > 0) {
+          // the chunks brought in neighbours' columns besides the row: zeros in
+          // the pad * C columns either side that windows read
+          uint16_t* const rows16 = reinterpret_cast<uint16_t*>(rowbuf + b * kStemRowBytes);
+          for (int v = warp; v < G.rows; v += kProd)
+            for (int k = lane; k < 2 * pad_c; k += 32) {
+              const int at = s_row[v] + (k < pad_c ? k : row_elems + k);  // (s_row: pad_c before the data)
+              if (at >= v * G.pitch && at < (v + 1) * G.pitch) rows16[at] = 0;  // (rows this tile has not: anything)
+            }
+          named_bar_sync(1, kProdThreads);
+        }
+        if (it >= S)
+          ok = ok && mbar_wait_warp(bar_empty + 8 * slot, (uint32_t)(((it >> 1) & 1) ^ 1), err, s_abort, kErrTimeoutEmpty, wlim);
+        if (ok) {
+          const uint32_t* const words = reinterpret_cast<const uint32_t*>(rowbuf + b * kStemRowBytes);
+          const uint32_t a0 = sA + slot * C::kAStage;
+          auto build = [&](auto nseg_c) {
+            constexpr int NS = decltype(nseg_c)::value;
+#pragma unroll 4
+            for (int unit = warp; unit < 4 * G.kh; unit += kProd) {
+              const int rr = (unit & 3) * 32 + lane, kr = unit >> 2;
+              const uint32_t px = s_pix[rr];
+              const int e = s_row[(px >> 24) + kr] + (int)(px & 0xFFFFFFu);
+              const uint32_t* src = words + (e >> 1);
+              const uint32_t sh = (uint32_t)(e & 1) * 16u;
+              uint32_t w[4 * NS + 1];
+#pragma unroll
+              for (int i = 0; i <= 4 * NS; ++i) w[i] = src[i];
+#pragma unroll
+              for (int i = 0; i < 4 * NS; ++i) {
+                w[i] = __funnelshift_r(w[i], w[i + 1], sh);
+                if (i >= 4 * (NS - 1)) w[i] &= keep[i & 3];
+              }
+#pragma unroll
+              for (int q = 0; q < NS; ++q) {
+                const int kc = kr * NS + q;  // 16-byte chunk of the K axis
+                sts_u4(a0 + (uint32_t)((kc >> 3) * (kBM * BK * 2)) + swz_offset<BK>(rr, kc & 7),
+                       make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]));
+              }
+            }
+          };
+          if (nseg == 3) build(IntConst<3>{});
+          else if (nseg == 2) build(IntConst<2>{});
+          else build(IntConst<1>{});
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_full + 8 * slot);
+        }
+        named_bar_sync(1, kProdThreads);  // buffer b and its tables are free for the tile after next
+      }
+      cp_async_wait<0>();
+      if (tid == 0) *s_issued = 0;  // (no TMA copies into the ring)
+    } else if (LEAN && !skip) {
       // Dense path: one converged warp, one elected lane issues.  The tiles'
       // origins (a few integer divisions each) are computed for 32 tiles at a
       // time, one per lane.
@@ -764,7 +922,25 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
         break;
       tc_fence_after();
       const uint32_t d = tmem + (uint32_t)b * C::kAccCols;
-      if (!skip) {
+      if constexpr (STEM) {
+        // the whole A tile is one stage
+        const int nks = (p.Ktot + 15) / 16;
+        ok = mbar_wait_warp(bar_full + 8 * slot, ph, err, s_abort, kErrTimeoutFull, wlim);
+        if (ok) {
+          tc_fence_after();
+          if (el) {
+            tc_mma_bf16(d, ad, bd0, idesc, 0u);
+#pragma unroll
+            for (int k = 1; k < 12; ++k)
+              if (k < nks)
+                tc_mma_bf16(d, ad + (uint64_t)((k >> 2) * (kBM * BK * 2 / 16) + 2 * (k & 3)),
+                            bd0 + (uint64_t)((k >> 2) * (C::kBStage / 16) + 2 * (k & 3)), idesc, 1u);
+            tc_commit(bar_empty + 8 * slot);
+          }
+          __syncwarp();
+          next();
+        }
+      } else if (!skip) {
         // every K block of the unit
         const int ks = KS == 1 ? 0 : u - (u / KS) * KS;
         const int n = KS == 1 ? kblocks : (ks + 1) * kblocks / KS - ks * kblocks / KS;
@@ -829,9 +1005,9 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
     const int r = q * 32 + lane;
     const int lane_col = lane < 16 ? 2 * lane : 2 * lane - 31;  // column of bit `lane` in nz_mask32's order
     const int ew = warp - kEpiWarp0;
-    const int slots = 4 / ncw;             // tiles in work at a time
-    const int slot = (ew >> 2) & (slots - 1);
-    const int cw = (ew >> 2) / slots;      // this warp's 32-column blocks: cw, cw + ncw, ...
+    const int slots = ncw == 1 ? kQw : 1;            // tiles in work at a time
+    const int slot = ncw == 1 ? ew >> 2 : 0;
+    const int cw = ncw == 1 ? 0 : ew >> 2;           // this warp's 32-column blocks: cw, cw + ncw, ...
     int sw_ = 0, sh_ = 0, sn_ = 0;
     if (p.conv == 2) {
       const int rho = q * 32;
@@ -846,7 +1022,7 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
     float* const own = s_scale + 2 * BN + ew * 64;  // this warp's block: scale[32], shift[32]
     if (affine && fixed_cols) {
       const int n0 = ((int)blockIdx.x % nt) * BN;
-      for (int c = threadIdx.x - 128; c < BN; c += kEpiThreads) {
+      for (int c = threadIdx.x - kEpiThread0; c < BN; c += kEpiThreads) {
         float sc = 1.f, sh = 0.f;
         if (n0 + c < p.N) epi_affine(ep, p.N, n0 + c, sc, sh);
         s_scale[c] = sc;
@@ -1026,7 +1202,7 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
       named_bar_sync(2, kEpiThreads);
       unsigned long long total = 0ull;
       for (int c0 = 0; c0 < p.N; c0 += kEpiThreads) {
-        const int c = c0 + (int)threadIdx.x - 128;
+        const int c = c0 + (int)threadIdx.x - kEpiThread0;
         const uint32_t cnt = c < p.N ? s_acc[c] : 0u;
         if (cnt) atomicAdd(&o.col_nnz[c], cnt);
         uint32_t sum = cnt;
@@ -1050,7 +1226,7 @@ __global__ void __launch_bounds__(Warps<LEAN>::kThreads, 1)
     const int hf = (warp - 4) >> 2;    // which 32 columns of each 64-column group
     const int ew = warp - 4;           // epilogue warp index
     const int r = q * 32 + lane;       // tile row
-    const int et = threadIdx.x - 128;  // 0..kEpiThreads-1
+    const int et = threadIdx.x - kEpiThread0;  // 0..kEpiThreads-1
     const bool vec = (p.N % 8) == 0;
     const bool affine = ep.bias != nullptr || ep.bn != nullptr;  // else the column affine is 1, 0
     // this warp's 32-row sub-box of the tile: {32 channels, bw', bh', bn'} for
@@ -1465,17 +1641,17 @@ bool make_tmap_nhwc(CUtensorMap* m, const void* base, int n, int h, int w, int c
 
 namespace {
 
-template <int BN, int BK, int LEAN>
+template <int BN, int BK, int LEAN, bool STEM = false>
 cudaError_t launch_cfg(const IgemmArgs& a, const CUtensorMap& tA, const CUtensorMap& tB,
                        const CUtensorMap& tY, const CUtensorMap& tA32, const CUtensorMap& tB32,
                        int64_t tiles, cudaStream_t s) {
   cudaError_t e0 =
-      smem_optin(reinterpret_cast<const void*>(igemm_kernel<BN, BK, LEAN>), (size_t)Cfg<BN, BK>::kSmem);
+      smem_optin(reinterpret_cast<const void*>(igemm_kernel<BN, BK, LEAN, STEM>), (size_t)Cfg<BN, BK, STEM>::kSmem);
   if (e0 != cudaSuccess) return e0;
   const int64_t units = tiles * (a.ksplit > 1 ? a.ksplit : 1);
   const int64_t grid = units < device_sm_count() ? units : device_sm_count();
-  cudaError_t e = launch_kernel(igemm_kernel<BN, BK, LEAN>, dim3((unsigned)grid), dim3(Warps<LEAN>::kThreads),
-                                (size_t)Cfg<BN, BK>::kSmem, s, tA, tB, tY, tA32, tB32, a);
+  cudaError_t e = launch_kernel(igemm_kernel<BN, BK, LEAN, STEM>, dim3((unsigned)grid), dim3(Warps<LEAN, STEM>::kThreads),
+                                (size_t)Cfg<BN, BK, STEM>::kSmem, s, tA, tB, tY, tA32, tB32, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -1574,9 +1750,64 @@ void choose_tiles(const IgemmArgs& a, int64_t mtiles, int* bn_out, int* ks_out) 
   *ks_out = ks;
 }
 
+// n / d = umulhi(n, mul) >> shift for 0 <= n < 2^31 (Granlund and Montgomery,
+// "Division by invariant integers using multiplication", 1994: with 2^l >= d,
+// mul = ceil(2^(31 + l) / d) < 2^32 and the product's excess stays below 2^(31+l)/d).
+static void div_magic(uint32_t d /* >= 2 */, uint32_t* mul, uint32_t* shift) {
+  uint32_t l = 0;
+  while ((1u << l) < d) ++l;
+  const uint64_t num = (uint64_t)1 << (31 + l);
+  *mul = (uint32_t)((num + d - 1) / d);
+  *shift = l - 1;
+}
+
+bool stem_plan(const __nv_bfloat16* x, int64_t n, int H, int W, int C, int N, int kh, int kw, int stride, int pad,
+               StemGeo* g) {
+  StemGeo q;
+  q.x = x;
+  q.H = H;
+  q.W = W;
+  q.C = C;
+  q.kh = kh;
+  q.kw = kw;
+  q.stride = stride;
+  q.pad = pad;
+  q.Ho = (H + 2 * pad - kh) / stride + 1;
+  q.Wo = (W + 2 * pad - kw) / stride + 1;
+  if (C >= 8 || kh * kw <= 1 || N > 64 || N % 8 || n <= 0) return false;
+  // a window of a kernel row fits 24 K columns, the whole window three K blocks
+  if (kw * C > 24 || pad >= kw || pad >= kh) return false;
+  q.seg = (kw * C + 7) / 8 * 8;
+  if (kh * q.seg > 192) return false;
+  // a tile's 128 pixels lie in at most two images
+  if ((int64_t)q.Ho * q.Wo < kBM || (int64_t)n * q.Ho * q.Wo > ((int64_t)1 << 31) - 1 - kBM) return false;
+  const int span = 1 + (kBM - 1 + q.Wo - 1) / q.Wo;
+  const int one = kh + (span - 1) * stride, two = 2 * kh + (span - 2) * stride;
+  q.rows = one > two ? one : two;
+  q.lead = (pad * C + 1 + 7) / 8 * 8;
+  const int need = q.lead + 7 + (W * C > (q.Wo - 1) * stride * C ? W * C : (q.Wo - 1) * stride * C) + q.seg + 10;
+  q.pitch = (need + 7) / 8 * 8;
+  if (q.rows > kMaxStemRows || (int64_t)q.rows * q.pitch * 2 > kStemRowBytes || (int64_t)W * stride * C >= (1 << 23)) return false;
+  if (q.Wo < 2 || q.Ho < 2) return false;  // (a divisor of 1 has no 32-bit multiplier)
+  div_magic((uint32_t)q.Wo, &q.wo_mul, &q.wo_shift);
+  div_magic((uint32_t)q.Ho, &q.ho_mul, &q.ho_shift);
+  q.ragged = (reinterpret_cast<uintptr_t>(x) & 15u) != 0 || (W * C) % 8 != 0;
+  *g = q;
+  return true;
+}
+
 cudaError_t launch_igemm(const IgemmArgs& a_in, cudaStream_t s) {
   IgemmArgs a = a_in;
   if (a.M <= 0 || a.N <= 0) return cudaSuccess;
+  if (a.stem.x) {
+    CUtensorMap tB, tY;
+    if (!make_tmap_2d(&tB, a.w, (uint64_t)a.N, (uint64_t)a.Ktot, 64, 64) ||
+        !make_tmap_2d(&tY, a.y, (uint64_t)a.M, (uint64_t)a.N, 32, 32))
+      return cudaErrorInvalidValue;
+    const int64_t tiles = ((int64_t)a.M + kBM - 1) / kBM;
+    return a.ep.residual ? launch_cfg<64, 64, 2, true>(a, tB, tB, tY, tB, tB, tiles, s)
+                         : launch_cfg<64, 64, 1, true>(a, tB, tB, tY, tB, tB, tiles, s);
+  }
   if (a.conv == 2 && (a.Cp % 32 != 0 || a.bw * a.bh * a.bn != 128)) return cudaErrorInvalidValue;
   const int64_t mtiles =
       a.conv == 2 ? (int64_t)((a.Nimg + a.bn - 1) / a.bn) * a.th * a.tw : (a.M + kBM - 1) / kBM;

@@ -65,6 +65,20 @@ cudaError_t launch_clear(const ClearArgs& a, cudaStream_t s);
 // ----------------------------------------------------------------------------
 // Implicit-GEMM tensor-core kernel (dense path and zero-skip path)
 // ----------------------------------------------------------------------------
+// A convolution with few input channels (the RGB stem) whose A tiles the kernel
+// builds itself from the input rows (stem_plan): conv = 0, Ktot = kh * seg, w
+// [N][kh][seg] with each kernel row's kw * C weights zero-padded to seg.
+struct StemGeo {
+  const __nv_bfloat16* x = nullptr;  // NHWC, any alignment; null: not a stem
+  int H = 0, W = 0, C = 0, Ho = 0, Wo = 0, kh = 0, kw = 0, stride = 1, pad = 0;
+  int seg = 0;    // K columns per kernel row: 8, 16 or 24
+  int rows = 0;   // input rows staged per tile, at most
+  int lead = 0;   // staged row: zero columns before the data (a multiple of 8) ...
+  int pitch = 0;  // ... and its length (a multiple of 8)
+  uint32_t wo_mul = 0, wo_shift = 0, ho_mul = 0, ho_shift = 0;  // n / Wo, n / Ho = umulhi(n, mul) >> shift
+  int ragged = 0; // 1: some row of x does not start on a 16-byte boundary
+};
+
 struct IgemmArgs {
   // Output y[M, N] (conv: M = images * Ho * Wo output pixels, N = C_out).
   int M = 0, N = 0;
@@ -102,6 +116,7 @@ struct IgemmArgs {
   int early = 0;
   // 1: the same for w and the epilogue's parameters only
   int early_w = 0;
+  StemGeo stem;
   // split K (set by launch_igemm from the scratch offered here): fp32 partial
   // tiles [tiles][ksplit][128][BN] in `ws` (ws_bytes), one zeroed arrival
   // counter per output tile in `ws_cnt` (ws_cnt_len), left zero again
@@ -123,6 +138,11 @@ bool make_tmap_2d(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols
                   uint32_t box_rows);
 bool make_tmap_nhwc(CUtensorMap* m, const void* base, int n, int h, int w, int c, int box_c, int bw, int bh,
                     int bn, int stride);
+
+// Fills in a.stem (all but the weights) for a convolution of x [n, H, W, C] with
+// N output channels; false where the shape is not for it.
+bool stem_plan(const __nv_bfloat16* x, int64_t n, int H, int W, int C, int N, int kh, int kw, int stride, int pad,
+               StemGeo* g);
 
 // One 128 x 64 output tile per cluster of up to 8 CTAs that share its K range
 // (k_onetile.cu).  onetile_split: the cluster size for K blocks of `bk`, 0
