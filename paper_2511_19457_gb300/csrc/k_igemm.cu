@@ -399,10 +399,12 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
   // with dense_only the zero-skip kernel of this launch runs instead
   const bool run = !(!LEAN && P.dense_only && path == 2);
   if (run) record_path(P.disp, path);
-  const bool skip = !STEM && path == 2;  // (a stem's tiles hold every K block)
+  // (nothing can be left out of a stem's tiles, a GEMM with one K block or an
+  // input without block masks)
+  const bool skip = !STEM && path == 2 && !(p.conv == 0 && (kblocks == 1 || in_blk == nullptr));
   // zero-skip GEMM with 64-wide K blocks: stages hold two occupied 32-column
   // groups each (compacted), loaded as 32-column boxes with the 64-byte swizzle
-  const bool compact = skip && p.conv == 0 && BK == 64 && kgroups <= kMaxKWords * 32 && in_blk != nullptr;
+  const bool compact = skip && p.conv == 0;  // (kblocks > 1: BK = 64)
 
   // every tile of the CTA has the same columns
   const bool fixed_cols = nt == 1 || (int)gridDim.x % nt == 0 || units <= (int)gridDim.x;
@@ -550,7 +552,73 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
       }
       cp_async_wait<0>();
       if (tid == 0) *s_issued = 0;  // (no TMA copies into the ring)
-    } else if (LEAN && !skip) {
+    } else if (compact) {
+      // Zero-skip GEMM: the converged warp walks the tile's 128-row block of the
+      // input's masks, 32 column groups a step (one word a lane, the next step's
+      // words loaded ahead, across tiles), and issues the occupied groups in
+      // pairs.  A stage is held back until the next occupied group or the tile's
+      // end is known, so that the last one can be marked; a tile with none runs
+      // group 0 (all zero) so that its accumulator is written.
+      if (warp == 0) {
+        const bool el = elect_one();
+        int it = 0, slot = 0;
+        uint32_t ph = 0u;
+        bool ok = true;
+        auto issue = [&](int ga, int gb, int m0, int n0, bool last) {
+          ok = ok && (it < S || mbar_wait_warp(bar_empty + 8 * slot, ph ^ 1u, err, s_abort, kErrTimeoutEmpty, wlim));
+          if (!ok) return;
+          if (el) {
+            const uint32_t fb = bar_full + 8 * slot;
+            const int nh = gb >= 0 ? 2 : 1;
+            stage_last[slot] = (last ? 1 : 0) | (nh == 1 ? 2 : 0);
+            mbar_arrive_expect_tx(fb, (uint32_t)(nh * (kBM * 64 + BN * 64)));
+            tma_load_2d(sA + slot * C::kAStage, &tmA32, fb, ga * 32, m0);
+            tma_load_2d(sB + slot * C::kBStage, &tmB32, fb, ga * 32, n0);
+            if (nh == 2) {
+              tma_load_2d(sA + slot * C::kAStage + kBM * 64, &tmA32, fb, gb * 32, m0);
+              tma_load_2d(sB + slot * C::kBStage + BN * 64, &tmB32, fb, gb * 32, n0);
+            }
+          }
+          __syncwarp();
+          ++it;
+          if (++slot == S) {
+            slot = 0;
+            ph ^= 1u;
+          }
+        };
+        auto word_at = [&](int u, int c) -> uint32_t {  // group 32 c + lane of tile u's block
+          if (u >= units) return 0u;
+          const int mi = nt == 1 ? u : u / nt;
+          const int gi = c * 32 + lane;
+          return gi < kgroups ? in_blk[(int64_t)mi * in_C32 + gi] : 0u;
+        };
+        const int steps = (kgroups + 31) / 32;
+        uint32_t ahead = word_at(blockIdx.x, 0);
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+          const int mi = nt == 1 ? u : u / nt;
+          const int m0 = mi * kBM, n0 = (u - mi * nt) * BN;
+          int ga = -1, gb = -1;  // the stage held back
+          for (int c = 0; c < steps; ++c) {
+            uint32_t bits = __ballot_sync(0xffffffffu, ahead != 0u);
+            ahead = c + 1 < steps ? word_at(u, c + 1) : word_at(u + (int)gridDim.x, 0);
+            for (; bits; bits &= bits - 1u) {
+              const int gi = c * 32 + __ffs(bits) - 1;
+              if (ga < 0) {
+                ga = gi;
+              } else if (gb < 0) {
+                gb = gi;
+              } else {
+                issue(ga, gb, m0, n0, false);
+                ga = gi;
+                gb = -1;
+              }
+            }
+          }
+          issue(ga < 0 ? 0 : ga, gb, m0, n0, true);
+        }
+        if (lane == 0) *s_issued = it;  // stages this CTA filled (TMA copies issued)
+      }
+    } else if (p.conv != 1 && !skip) {
       // Dense path: one converged warp, one elected lane issues.  The tiles'
       // origins (a few integer divisions each) are computed for 32 tiles at a
       // time, one per lane.
@@ -613,11 +681,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
     int it = 0;        // stages filled so far (ring position)
     int pending = 0;   // mode 1: filled stages whose A arrivals are still owed
     bool ok = true;
-    // dense TMA modes: thread 0 issues everything, the other producer threads
-    // have no part in the loop (their tile geometry would only take issue
-    // slots from the epilogue warps on the same schedulers)
-    const bool lone = !skip && p.conv != 1;
-    for (int u = (lone && r != 0) ? units : (int)blockIdx.x; u < units; u += gridDim.x) {
+    for (int u = blockIdx.x; u < units; u += gridDim.x) {
       if (u != (int)blockIdx.x) ug = unit_geo(p, u, KS, kblocks, nt, BN, BK, r);
       const int kb0 = ug.kb0, kb1 = ug.kb1;
       const TileGeo g = ug.g;
@@ -627,93 +691,62 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
       if (skip) {
         // ---- occupied K blocks of this tile
         named_bar_sync(1, kProdThreads);  // thread 0 is done with the previous tile's bits
-        if (compact) {
-          // occupied 32-column groups of this unit's K range in the tile's
-          // 128-row block: one bit per group
-          const int g0 = 2 * kb0, g1 = 2 * kb1 < kgroups ? 2 * kb1 : kgroups;
-          const uint32_t* words = in_blk + (int64_t)(g.m0 >> 7) * in_C32;
-          for (int w0 = 0; w0 < kgroups && w0 < kMaxKWords * 32; w0 += kProdThreads) {
-            const int gi = w0 + r;
-            const bool occ = gi >= g0 && gi < g1 && words[gi] != 0u;
-            const uint32_t bits = __ballot_sync(0xffffffffu, occ);
-            if (lane == 0 && (w0 >> 5) + warp < kMaxKWords) s_kbits[(w0 >> 5) + warp] = bits;
+        if (r < kMaxTaps) s_tap[r] = 0ull;
+        named_bar_sync(1, kProdThreads);
+        const int taps = p.kh * p.kw < kMaxTaps ? p.kh * p.kw : kMaxTaps;
+        // (with 96 producer threads warp 0 takes the last 32 rows as well)
+        for (int row = r; row < kBM; row += kProdThreads) {
+          bool rv = rvalid;
+          int ri = img, ry = oh, rx = ow;
+          if (row != r) tile_row(p, g, row, rv, ri, ry, rx);
+          for (int t0 = 0; t0 < taps; t0 += 8) {
+            unsigned long long wv[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {  // issue 8 taps' loads before reducing any
+              const int tp = t0 + u;
+              const int ih = ry * p.stride - p.pad + tp / p.kw;
+              const int iw = rx * p.stride - p.pad + tp % p.kw;
+              wv[u] = 0ull;
+              if (in_rowbm && tp < taps && rv && ih >= 0 && ih < p.H && iw >= 0 && iw < p.W)
+                wv[u] = in_rowbm[(((int64_t)ri * p.H + ih) * p.W + iw) * in_W64];
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+              unsigned long long w = wv[u];
+#pragma unroll
+              for (int s = 16; s > 0; s >>= 1) w |= __shfl_xor_sync(0xffffffffu, w, s);
+              if (lane == 0 && w) atomicOr(&s_tap[t0 + u], w);
+            }
           }
-        } else if (p.conv == 0) {
-          for (int w0 = 0; w0 < kblocks && w0 < kMaxKWords * 32; w0 += kProdThreads) {
-            const int kb = w0 + r;
-            // a K block covers BK / 32 words of the 128-row block-column mask
-            // (an input without block masks, such as the im2col rows of a
-            // narrow stem, keeps every block)
-            bool occ = false;
-            if (kb < kblocks && in_blk == nullptr) {
+        }
+        named_bar_sync(1, kProdThreads);
+        // no per-tap masks (too many taps, wide rows, or an input given without
+        // row bitmaps): keep every block
+        const bool many = p.kh * p.kw > kMaxTaps || in_W64 > 1 || in_rowbm == nullptr;
+        for (int w0 = 0; w0 < kblocks && w0 < kMaxKWords * 32; w0 += kProdThreads) {
+          const int kb = w0 + r;
+          bool occ = false;
+          if (kb < kblocks) {
+            if (many) {
               occ = true;
-            } else if (kb < kblocks) {
-              const uint32_t* words = in_blk + (int64_t)(g.m0 >> 7) * in_C32;
-              occ = words[kb * (BK / 32)] != 0u;
-              if (BK == 64 && kb * 2 + 1 < in_C32) occ |= words[kb * 2 + 1] != 0u;
-            }
-            const uint32_t bits = __ballot_sync(0xffffffffu, occ);
-            if (lane == 0 && (w0 >> 5) + warp < kMaxKWords) s_kbits[(w0 >> 5) + warp] = bits;
-          }
-        } else {
-          if (r < kMaxTaps) s_tap[r] = 0ull;
-          named_bar_sync(1, kProdThreads);
-          const int taps = p.kh * p.kw < kMaxTaps ? p.kh * p.kw : kMaxTaps;
-          // (with 96 producer threads warp 0 takes the last 32 rows as well)
-          for (int row = r; row < kBM; row += kProdThreads) {
-            bool rv = rvalid;
-            int ri = img, ry = oh, rx = ow;
-            if (row != r) tile_row(p, g, row, rv, ri, ry, rx);
-            for (int t0 = 0; t0 < taps; t0 += 8) {
-              unsigned long long wv[8];
+            } else {
 #pragma unroll
-              for (int u = 0; u < 8; ++u) {  // issue 8 taps' loads before reducing any
-                const int tp = t0 + u;
-                const int ih = ry * p.stride - p.pad + tp / p.kw;
-                const int iw = rx * p.stride - p.pad + tp % p.kw;
-                wv[u] = 0ull;
-                if (in_rowbm && tp < taps && rv && ih >= 0 && ih < p.H && iw >= 0 && iw < p.W)
-                  wv[u] = in_rowbm[(((int64_t)ri * p.H + ih) * p.W + iw) * in_W64];
-              }
-#pragma unroll
-              for (int u = 0; u < 8; ++u) {
-                unsigned long long w = wv[u];
-#pragma unroll
-                for (int s = 16; s > 0; s >>= 1) w |= __shfl_xor_sync(0xffffffffu, w, s);
-                if (lane == 0 && w) atomicOr(&s_tap[t0 + u], w);
+              for (int j = 0; j < BK / 8; ++j) {
+                const int flat = kb * BK + 8 * j;
+                if (flat >= p.Ktot) break;
+                const int tp = flat / p.Cp;
+                const int c = flat - tp * p.Cp;
+                occ |= ((s_tap[tp] >> (c >> 6)) & 1ull) != 0ull;
               }
             }
           }
-          named_bar_sync(1, kProdThreads);
-          // no per-tap masks (too many taps, wide rows, or an input given without
-          // row bitmaps): keep every block
-          const bool many = p.kh * p.kw > kMaxTaps || in_W64 > 1 || in_rowbm == nullptr;
-          for (int w0 = 0; w0 < kblocks && w0 < kMaxKWords * 32; w0 += kProdThreads) {
-            const int kb = w0 + r;
-            bool occ = false;
-            if (kb < kblocks) {
-              if (many) {
-                occ = true;
-              } else {
-#pragma unroll
-                for (int j = 0; j < BK / 8; ++j) {
-                  const int flat = kb * BK + 8 * j;
-                  if (flat >= p.Ktot) break;
-                  const int tp = flat / p.Cp;
-                  const int c = flat - tp * p.Cp;
-                  occ |= ((s_tap[tp] >> (c >> 6)) & 1ull) != 0ull;
-                }
-              }
-            }
-            const uint32_t bits = __ballot_sync(0xffffffffu, occ);
-            if (lane == 0 && (w0 >> 5) + warp < kMaxKWords) s_kbits[(w0 >> 5) + warp] = bits;
-          }
+          const uint32_t bits = __ballot_sync(0xffffffffu, occ);
+          if (lane == 0 && (w0 >> 5) + warp < kMaxKWords) s_kbits[(w0 >> 5) + warp] = bits;
         }
         named_bar_sync(1, kProdThreads);
         // last occupied block of this unit's K range; a range with none still
         // runs its first block (whose data is all zero)
         last = kb0;
-        if (compact) last = kb1 - 1;  // unused: the compacted loop tracks its own last stage
         for (int kb = kb1 - 1; kb > kb0; --kb) {
           if (kb >= kMaxKWords * 32 || ((s_kbits[kb >> 5] >> (kb & 31)) & 1u)) {
             last = kb;
@@ -722,58 +755,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
         }
       }
       if (!ok) continue;  // keep the skip-mask barriers in step; issue nothing more
-      if (compact) {
-        if (r == 0) {
-          // pairs of occupied groups in increasing order; an odd last group
-          // takes a stage alone; a unit with none runs group g0 (all zero) so
-          // that its accumulator is written
-          const int g0 = 2 * kb0, g1 = 2 * kb1 < kgroups ? 2 * kb1 : kgroups;
-          int cnt = 0;
-          for (int wd = g0 >> 5; wd <= (g1 - 1) >> 5; ++wd) cnt += __popc(s_kbits[wd]);
-          const int nst = cnt ? (cnt + 1) / 2 : 1;
-          int slot = it % S;
-          uint32_t ph = (uint32_t)((it / S) & 1);
-          int st = 0, pend = -1;
-          auto issue = [&](int ga, int gb) -> bool {
-            if (it >= S && !mbar_wait(bar_empty + 8 * slot, ph ^ 1u, err, s_abort, kErrTimeoutEmpty, wlim)) return false;
-            const uint32_t fb = bar_full + 8 * slot;
-            const int nh = gb >= 0 ? 2 : 1;
-            stage_last[slot] = (st == nst - 1 ? 1 : 0) | (nh == 1 ? 2 : 0);
-            mbar_arrive_expect_tx(fb, (uint32_t)(nh * (kBM * 64 + BN * 64)));
-            tma_load_2d(sA + slot * C::kAStage, &tmA32, fb, ga * 32, g.m0);
-            tma_load_2d(sB + slot * C::kBStage, &tmB32, fb, ga * 32, g.n0);
-            if (nh == 2) {
-              tma_load_2d(sA + slot * C::kAStage + kBM * 64, &tmA32, fb, gb * 32, g.m0);
-              tma_load_2d(sB + slot * C::kBStage + BN * 64, &tmB32, fb, gb * 32, g.n0);
-            }
-            ++st;
-            ++it;
-            if (++slot == S) {
-              slot = 0;
-              ph ^= 1u;
-            }
-            return true;
-          };
-          if (cnt == 0) {
-            ok = issue(g0, -1);
-          } else {
-            for (int wd = g0 >> 5; wd <= (g1 - 1) >> 5 && ok; ++wd) {
-              uint32_t bits = s_kbits[wd];
-              while (bits && ok) {
-                const int gi = wd * 32 + __ffs(bits) - 1;
-                bits &= bits - 1u;
-                if (pend < 0) {
-                  pend = gi;
-                } else {
-                  ok = issue(pend, gi);
-                  pend = -1;
-                }
-              }
-            }
-            if (ok && pend >= 0) ok = issue(pend, -1);
-          }
-        }
-      } else if (LEAN || p.conv != 1) {
+      if (LEAN || p.conv != 1) {
         if (r == 0) {
           // The issuing lane is slow at anything but issuing: ring slot, phase
           // and the (tap, channel block) of each K block advance incrementally,
