@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
       // Zero-skip GEMM: the converged warp walks the tile's 128-row block of the
       // input's masks, 32 column groups a step (one word a lane, the next step's
       // words loaded ahead, across tiles), and issues the occupied groups in
-      // pairs.  A stage is held back until the next occupied group or the tile's
+      // pairs (an aligned pair as one 64-wide K block).  A stage is held back until the next occupied group or the tile's
       // end is known, so that the last one can be marked; a tile with none runs
       // group 0 (all zero) so that its accumulator is written.
       if (warp == 0) {
@@ -570,13 +570,19 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
           if (el) {
             const uint32_t fb = bar_full + 8 * slot;
             const int nh = gb >= 0 ? 2 : 1;
-            stage_last[slot] = (last ? 1 : 0) | (nh == 1 ? 2 : 0);
+            const bool whole = gb == ga + 1 && (ga & 1) == 0;  // a 64-wide K block: one box of 128-byte rows
+            stage_last[slot] = (last ? 1 : 0) | (nh == 1 ? 2 : 0) | (whole ? 4 : 0);
             mbar_arrive_expect_tx(fb, (uint32_t)(nh * (kBM * 64 + BN * 64)));
-            tma_load_2d(sA + slot * C::kAStage, &tmA32, fb, ga * 32, m0);
-            tma_load_2d(sB + slot * C::kBStage, &tmB32, fb, ga * 32, n0);
-            if (nh == 2) {
-              tma_load_2d(sA + slot * C::kAStage + kBM * 64, &tmA32, fb, gb * 32, m0);
-              tma_load_2d(sB + slot * C::kBStage + BN * 64, &tmB32, fb, gb * 32, n0);
+            if (whole) {
+              tma_load_2d(sA + slot * C::kAStage, &tmA, fb, ga * 32, m0);
+              tma_load_2d(sB + slot * C::kBStage, &tmB, fb, ga * 32, n0);
+            } else {
+              tma_load_2d(sA + slot * C::kAStage, &tmA32, fb, ga * 32, m0);
+              tma_load_2d(sB + slot * C::kBStage, &tmB32, fb, ga * 32, n0);
+              if (nh == 2) {
+                tma_load_2d(sA + slot * C::kAStage + kBM * 64, &tmA32, fb, gb * 32, m0);
+                tma_load_2d(sB + slot * C::kBStage + BN * 64, &tmB32, fb, gb * 32, n0);
+              }
             }
           }
           __syncwarp();
@@ -941,7 +947,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
           const int sflags = stage_last[slot];
           last = (sflags & 1) != 0;
           if (el) {
-            if (compact) {
+            if (compact && !(sflags & 4)) {
               // one or two 32-column groups, each 128 (A) / BN (B) rows of 64
               // bytes with the 64-byte swizzle: two k-steps of 16 per group
               const uint32_t a = sA + slot * C::kAStage, bb = sB + slot * C::kBStage;
