@@ -23,11 +23,12 @@ constexpr int kVitThreads = 256;
 // beta, and the output's occupancy is emitted on the way: row bitmap words whole
 // (one word per row), block-column masks ORed over the run's rows of a 128-row
 // block, column counts in 16-bit register halves, added up in shared memory once
-// per CTA.  [6304, 768] with occupancy: 14.1 us + 9.5 us for a clear and a
-// statistics pass before (gamma and beta were re-read, value by value, for every
-// row).  Longer rows (layernorm_kernel) are re-read for each of the three steps.
+// per CTA.  [6304, 768]: 4.7 us, with occupancy and its clear 10.3 us (14.1 us and
+// 9.5 us more for a clear and a statistics pass before: gamma and beta were
+// re-read, value by value, for every row).  Longer rows (layernorm_kernel) are
+// re-read for each of the three steps.
 constexpr int kLnRegChunks = 4;     // 8-value chunks per lane held in registers
-constexpr int kLnCtasPerSm = 2;
+constexpr int kLnThreads = 512;     // at most: one CTA per SM, whose column counts reach global memory once
 constexpr int kLnFlushRows = 16384;  // rows after which 16-bit counters are flushed
 
 __device__ __forceinline__ void ln_store(__nv_bfloat16* __restrict__ yr, const float* __restrict__ gb, int C,
@@ -42,19 +43,19 @@ __device__ __forceinline__ void ln_store(__nv_bfloat16* __restrict__ yr, const f
 }
 
 template <int NCH>
-__global__ void __launch_bounds__(kVitThreads, kLnCtasPerSm)
+__global__ void __launch_bounds__(kLnThreads, 1)
     ln_rows_kernel(const __nv_bfloat16* __restrict__ x, int64_t R, int C, const float* __restrict__ gb, int gb_vec,
                    float eps, __nv_bfloat16* __restrict__ y, OccDev o_param, int emit) {
   const OccDev o = o_param;
-  __shared__ uint32_t s_cnt[NCH * 256];
+  __shared__ uint32_t s_cnt[NCH * 256];  // column 8 (32 i + lane) + k at (8 i + k) * 32 + lane
   const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (kVitThreads / 32);
-  const int64_t w = (int64_t)blockIdx.x * (kVitThreads / 32) + (threadIdx.x >> 5);
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
+  const int64_t w = (int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   const int64_t r0 = w * R / warps, r1 = (w + 1) * R / warps;
   const int chunks = C / 8;
   const float inv_c = 1.f / (float)C;
   if (emit)
-    for (int c = threadIdx.x; c < NCH * 256; c += kVitThreads) s_cnt[c] = 0u;
+    for (int c = threadIdx.x; c < NCH * 256; c += blockDim.x) s_cnt[c] = 0u;
   pdl_wait();
   pdl_trigger();
   uint4 u[NCH];
@@ -103,11 +104,10 @@ __global__ void __launch_bounds__(kVitThreads, kLnCtasPerSm)
   auto flush_cnt = [&]() {
 #pragma unroll
     for (int i = 0; i < NCH; ++i) {
-      const int c = (lane + 32 * i) * 8;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        if (cnt[i][k] & 0xFFFFu) atomicAdd(&s_cnt[c + 2 * k], cnt[i][k] & 0xFFFFu);
-        if (cnt[i][k] >> 16) atomicAdd(&s_cnt[c + 2 * k + 1], cnt[i][k] >> 16);
+        if (cnt[i][k] & 0xFFFFu) atomicAdd(&s_cnt[(i * 8 + 2 * k) * 32 + lane], cnt[i][k] & 0xFFFFu);
+        if (cnt[i][k] >> 16) atomicAdd(&s_cnt[(i * 8 + 2 * k + 1) * 32 + lane], cnt[i][k] >> 16);
         cnt[i][k] = 0u;
       }
     }
@@ -196,9 +196,9 @@ __global__ void __launch_bounds__(kVitThreads, kLnCtasPerSm)
   flush_cnt();
   __syncthreads();
   unsigned long long total = 0ull;
-  for (int c0 = 0; c0 < C; c0 += kVitThreads) {  // (whole warps: a warp's 32 columns are half a tile)
+  for (int c0 = 0; c0 < C; c0 += blockDim.x) {  // (whole warps: a warp's 32 columns are half a tile)
     const int c = c0 + threadIdx.x;
-    const uint32_t n = c < C ? s_cnt[c] : 0u;
+    const uint32_t n = c < C ? s_cnt[((c >> 8) * 8 + (c & 7)) * 32 + ((c >> 3) & 31)] : 0u;
     if (n) atomicAdd(&o.col_nnz[c], n);
     const uint32_t sum = __reduce_add_sync(0xffffffffu, n);
     total += sum;
@@ -639,16 +639,18 @@ cudaError_t launch_layernorm(const __nv_bfloat16* x, int64_t R, int C, const flo
     return launch_kernel(layernorm_kernel, dim3(grid_for(R, kVitThreads / 32)), dim3(kVitThreads), 0, s, x, R, C, gb,
                          eps, y);
   }
-  // a warp per row up to the resident warps, then runs of rows
-  const int64_t ctas = (R + kVitThreads / 32 - 1) / (kVitThreads / 32);
-  const int64_t cap = (int64_t)kLnCtasPerSm * device_sm_count();
+  // a warp per row up to the resident warps, then runs of rows; 16 warps a CTA
+  // once they fill the SMs (fewer CTAs add their column counts up in global memory)
+  const int threads = R >= 8 * (int64_t)device_sm_count() ? kLnThreads : 256;
+  const int64_t ctas = (R + threads / 32 - 1) / (threads / 32);
+  const int64_t cap = (int64_t)device_sm_count();
   const dim3 grid((unsigned)(ctas < cap ? ctas : cap));
   const int vec = (reinterpret_cast<uintptr_t>(gb) & 15u) == 0;  // (C % 8 == 0: beta's rows too)
   switch ((C + 255) / 256) {
-    case 1: return launch_kernel(ln_rows_kernel<1>, grid, dim3(kVitThreads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
-    case 2: return launch_kernel(ln_rows_kernel<2>, grid, dim3(kVitThreads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
-    case 3: return launch_kernel(ln_rows_kernel<3>, grid, dim3(kVitThreads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
-    default: return launch_kernel(ln_rows_kernel<4>, grid, dim3(kVitThreads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
+    case 1: return launch_kernel(ln_rows_kernel<1>, grid, dim3((unsigned)threads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
+    case 2: return launch_kernel(ln_rows_kernel<2>, grid, dim3((unsigned)threads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
+    case 3: return launch_kernel(ln_rows_kernel<3>, grid, dim3((unsigned)threads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
+    default: return launch_kernel(ln_rows_kernel<4>, grid, dim3((unsigned)threads), 0, s, x, R, C, gb, vec, eps, y, o, emit);
   }
 }
 
