@@ -257,19 +257,27 @@ __global__ void __launch_bounds__(kVitThreads) layernorm_kernel(const __nv_bfloa
 // in distinct banks; rows past T up to the next multiple of 16 zero-filled),
 // then every warp does its tile.  (One CTA of 4 warps per (image, head), each
 // warp three or four tiles in turn, left 12 warps per SM and a last round half
-// empty: [32,197,12x64] 34 us.)  A warp walks the keys in blocks of 64: S = Q K^T
+// empty: [32,197,12x64] 34 us.)  A warp walks the keys in blocks of 32: S = Q K^T
 // (Q fragments in registers, K fragments by ldmatrix), an online softmax per
 // query row (running maximum and sum, rescaling the output), and O += P V with P
 // taken straight from the S accumulators (their layout is the A-operand layout
 // of the next MMA) and the V fragments read by ldmatrix.trans from the row-major
 // V.  Key tiles wholly at or past T are not computed.  O / sum is stored as bf16,
-// and the output's occupancy is emitted: row bits by quads, the block-column
-// masks of a 16-query tile (rows of one 128-row block) by shuffles, column
-// counts in 16-bit register halves.
+// and the output's occupancy is emitted from one non-zero bit per value: row
+// bits by votes, block-column masks by warp OR, column counts by a transposition
+// of the warp's 32 x 32 bits.
+//
+// Bound by latency: 14 warps an SM against chains of MMAs, shuffles and
+// exponentials.  So a whole block of keys has no branches (the ones around each 8
+// keys kept the MMAs of different keys from overlapping) and the first queries
+// are loaded beside K and V.  Blocks of 32 keys rather than 64 fit 128 registers.
+// [32,197,12x64] without / with occupancy 28.9 / 34.7 -> 21.9 / 25.7 us (64-key
+// blocks 24.4 / 31.3), [8,512,12x64] 48.8 / 54.4 -> 33.6 / 36.9 us; the occupancy
+// took 64-bit masks by shuffles and 16 counters a lane before.
 constexpr int kAttnWarps = 7;
 constexpr int kAttnThreads = 32 * kAttnWarps;
 constexpr int kAttnMaxT = 512;
-constexpr int kAttnKB = 64;        // keys per block
+constexpr int kAttnKB = 32;        // keys per block
 
 // 2^x; results below the normal range are zero (they are probabilities)
 __device__ __forceinline__ float exp2_ftz(float x) {
@@ -280,8 +288,7 @@ __device__ __forceinline__ float exp2_ftz(float x) {
 
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                                uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
       "{%8, %9}, {%0, %1, %2, %3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
@@ -313,6 +320,11 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
+template <bool B>
+struct BoolConst {
+  static constexpr bool value = B;
+};
+
 template <int HD>
 __global__ void __launch_bounds__(kAttnThreads, 2)
     attention_kernel(const __nv_bfloat16* __restrict__ qkv, int T, int heads, __nv_bfloat16* __restrict__ y,
@@ -339,10 +351,29 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     cp_async_16(smem_u32(sV + t * KP + c * 8), src + 2 * D, live ? 16u : 0u);
   }
   cp_async_commit();
-  cp_async_wait<0>();
-  __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, tq = lane & 3;
+  const int qtn = (T + 15) >> 4;  // 16-query tiles
+  const int per = (qtn + (int)gridDim.y - 1) / (int)gridDim.y;
+  const int qt0 = (int)blockIdx.y * per + warp, qt_end = min(qtn, ((int)blockIdx.y + 1) * per);
+  // Q fragments (A operand, rows g and g + 8, HD / 16 k-steps), zero past T
+  uint32_t qa[HD / 16][4];
+  auto load_q = [&](int q0) {
+    const int r0 = q0 + g, r1 = q0 + g + 8;
+    const __nv_bfloat16* p0 = base + (int64_t)(r0 < T ? r0 : 0) * row3 + h * HD;
+    const __nv_bfloat16* p1 = base + (int64_t)(r1 < T ? r1 : 0) * row3 + h * HD;
+#pragma unroll
+    for (int kk = 0; kk < HD / 16; ++kk) {
+      const int c = kk * 16 + 2 * tq;
+      qa[kk][0] = r0 < T ? *reinterpret_cast<const uint32_t*>(p0 + c) : 0u;
+      qa[kk][1] = r1 < T ? *reinterpret_cast<const uint32_t*>(p1 + c) : 0u;
+      qa[kk][2] = r0 < T ? *reinterpret_cast<const uint32_t*>(p0 + c + 8) : 0u;
+      qa[kk][3] = r1 < T ? *reinterpret_cast<const uint32_t*>(p1 + c + 8) : 0u;
+    }
+  };
+  if (qt0 < qt_end) load_q(qt0 * 16);  // the first tile's queries arrive beside K and V
+  cp_async_wait<0>();
+  __syncthreads();
   const float sl2 = rsqrtf((float)HD) * 1.4426950408889634f;  // 1/sqrt(HD) * log2(e)
   // ldmatrix.trans lane address within a (16 keys x 16 dimensions) V block:
   // matrices (keys 0-7, dims 0-7), (keys 8-15, dims 0-7), (keys 0-7, dims
@@ -351,58 +382,51 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   const uint32_t v_lane = smem_u32(sV) + (uint32_t)(((lane & 15) * KP + (lane >> 4) * 8) * 2);
   // K fragments of 8 keys: matrices (dims 0-7, 8-15) of one k-step, then of the next
   const uint32_t k_lane = smem_u32(sK) + (uint32_t)(((lane & 7) * KP + (lane >> 3) * 8) * 2);
-  const int qtn = (T + 15) >> 4;  // 16-query tiles
-  const int per = (qtn + (int)gridDim.y - 1) / (int)gridDim.y;
-  const int qt_end = min(qtn, ((int)blockIdx.y + 1) * per);
-  uint32_t cnt[HD / 8];  // non-zeros of columns 8 j + 2 tq, + 1 (16-bit halves)
-#pragma unroll
-  for (int j = 0; j < HD / 8; ++j) cnt[j] = 0u;
-  for (int qt = (int)blockIdx.y * per + warp; qt < qt_end; qt += kAttnWarps) {
+  uint32_t cnt = 0u;  // byte i: non-zeros of column 8 (lane & 7) + 2 i + (lane >> 4) in the rows of half (lane >> 3) & 1
+  for (int qt = qt0; qt < qt_end; qt += kAttnWarps) {
     const int q0 = qt * 16;
-    // Q fragments (A operand, rows g and g + 8, HD / 16 k-steps), zero past T
-    uint32_t qa[HD / 16][4];
-    {
-      const int r0 = q0 + g, r1 = q0 + g + 8;
-      const __nv_bfloat16* p0 = base + (int64_t)(r0 < T ? r0 : 0) * row3 + h * HD;
-      const __nv_bfloat16* p1 = base + (int64_t)(r1 < T ? r1 : 0) * row3 + h * HD;
-#pragma unroll
-      for (int kk = 0; kk < HD / 16; ++kk) {
-        const int c = kk * 16 + 2 * tq;
-        qa[kk][0] = r0 < T ? *reinterpret_cast<const uint32_t*>(p0 + c) : 0u;
-        qa[kk][1] = r1 < T ? *reinterpret_cast<const uint32_t*>(p1 + c) : 0u;
-        qa[kk][2] = r0 < T ? *reinterpret_cast<const uint32_t*>(p0 + c + 8) : 0u;
-        qa[kk][3] = r1 < T ? *reinterpret_cast<const uint32_t*>(p1 + c + 8) : 0u;
-      }
-    }
+    if (qt != qt0) load_q(q0);
     float o[HD / 8][4];
 #pragma unroll
     for (int j = 0; j < HD / 8; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
     float m0 = -3.0e38f, m1 = -3.0e38f, l0 = 0.f, l1 = 0.f;  // rows g, g + 8
-    for (int kb = 0; kb < T; kb += kAttnKB) {
-      // S = Q K^T for up to 64 keys: 8 n-tiles of 8 keys
+    // one block of keys; all of its keys are below T if FULL, so that nothing in it
+    // branches and the MMAs of independent key tiles overlap
+    auto block = [&](auto full, int kb) {
+      constexpr bool FULL = decltype(full)::value;
+      // S = Q K^T, n-tiles of 8 keys
       float s[kAttnKB / 8][4];
 #pragma unroll
-      for (int nt = 0; nt < kAttnKB / 8; ++nt) {
-        s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
-        if (kb + nt * 8 < T) {  // uniform across the warp
-          const uint32_t ka = k_lane + (uint32_t)((kb + nt * 8) * KP * 2);
+      for (int nt = 0; nt < kAttnKB / 8; ++nt) s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
+      constexpr int G = FULL ? 4 : 1;  // n-tiles at a time
+#pragma unroll
+      for (int n0 = 0; n0 < kAttnKB / 8; n0 += G) {
+        if (FULL || kb + n0 * 8 < T) {  // uniform across the warp
+          const uint32_t ka = k_lane + (uint32_t)((kb + n0 * 8) * KP * 2);
           if constexpr (HD >= 32) {
 #pragma unroll
             for (int kk = 0; kk < HD / 16; kk += 2) {
-              uint32_t b0, b1, b2, b3;
-              ldsm_x4(ka + (uint32_t)(kk * 32), b0, b1, b2, b3);
-              mma_bf16_16816(s[nt], qa[kk], b0, b1);
-              mma_bf16_16816(s[nt], qa[kk + 1], b2, b3);
+              uint32_t b[G][4];
+#pragma unroll
+              for (int i = 0; i < G; ++i)
+                ldsm_x4(ka + (uint32_t)(i * 8 * KP * 2 + kk * 32), b[i][0], b[i][1], b[i][2], b[i][3]);
+#pragma unroll
+              for (int i = 0; i < G; ++i) mma_bf16_16816(s[n0 + i], qa[kk], b[i][0], b[i][1]);
+#pragma unroll
+              for (int i = 0; i < G; ++i) mma_bf16_16816(s[n0 + i], qa[kk + 1], b[i][2], b[i][3]);
             }
           } else {
-            uint32_t b0, b1;
-            ldsm_x2(ka, b0, b1);
-            mma_bf16_16816(s[nt], qa[0], b0, b1);
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+              uint32_t b0, b1;
+              ldsm_x2(ka + (uint32_t)(i * 8 * KP * 2), b0, b1);
+              mma_bf16_16816(s[n0 + i], qa[0], b0, b1);
+            }
           }
         }
       }
       // keys past T do not take part
-      if (kb + kAttnKB > T) {
+      if (!FULL) {
 #pragma unroll
         for (int nt = 0; nt < kAttnKB / 8; ++nt) {
           const int key = kb + nt * 8 + 2 * tq;
@@ -418,23 +442,27 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
         bm1 = fmaxf(bm1, fmaxf(s[nt][2], s[nt][3]));
       }
       bm0 = fmaxf(bm0, __shfl_xor_sync(0xffffffffu, bm0, 1));
-      bm0 = fmaxf(bm0, __shfl_xor_sync(0xffffffffu, bm0, 2));
       bm1 = fmaxf(bm1, __shfl_xor_sync(0xffffffffu, bm1, 1));
+      bm0 = fmaxf(bm0, __shfl_xor_sync(0xffffffffu, bm0, 2));
       bm1 = fmaxf(bm1, __shfl_xor_sync(0xffffffffu, bm1, 2));
       const float nm0 = fmaxf(m0, bm0), nm1 = fmaxf(m1, bm1);
       const float c0 = exp2_ftz((m0 - nm0) * sl2), c1 = exp2_ftz((m1 - nm1) * sl2);
       m0 = nm0;
       m1 = nm1;
+      const float t0 = -nm0 * sl2, t1 = -nm1 * sl2;
+      const f2_t sc2 = f2(sl2, sl2), t02 = f2(t0, t0), t12 = f2(t1, t1);
       float rs0 = 0.f, rs1 = 0.f;
       uint32_t pa[kAttnKB / 16][4];  // P as A fragments of the P V MMAs
 #pragma unroll
       for (int nt = 0; nt < kAttnKB / 8; ++nt) {
         float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
-        if (kb + nt * 8 < T) {  // uniform across the warp
-          p0 = exp2_ftz((s[nt][0] - nm0) * sl2);
-          p1 = exp2_ftz((s[nt][1] - nm0) * sl2);
-          p2 = exp2_ftz((s[nt][2] - nm1) * sl2);
-          p3 = exp2_ftz((s[nt][3] - nm1) * sl2);
+        if (FULL || kb + nt * 8 < T) {  // uniform across the warp
+          f2_split(ffma2(f2(s[nt][0], s[nt][1]), sc2, t02), p0, p1);
+          f2_split(ffma2(f2(s[nt][2], s[nt][3]), sc2, t12), p2, p3);
+          p0 = exp2_ftz(p0);
+          p1 = exp2_ftz(p1);
+          p2 = exp2_ftz(p2);
+          p3 = exp2_ftz(p3);
         }
         rs0 += p0 + p1;
         rs1 += p2 + p3;
@@ -454,7 +482,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       // n-tiles per ldmatrix
 #pragma unroll
       for (int kk = 0; kk < kAttnKB / 16; ++kk) {
-        if (kb + kk * 16 < T) {  // uniform across the warp
+        if (FULL || kb + kk * 16 < T) {  // uniform across the warp
           const uint32_t va = v_lane + (uint32_t)((kb + kk * 16) * KP * 2);
 #pragma unroll
           for (int j = 0; j < HD / 8; j += 2) {
@@ -465,7 +493,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
           }
         }
       }
-    }
+    };
+    int kb = 0;
+    for (; kb + kAttnKB <= T; kb += kAttnKB) block(BoolConst<true>{}, kb);
+    if (kb < T) block(BoolConst<false>{}, kb);
     // row sums over the quad, then O / sum
     l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
     l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
@@ -474,59 +505,59 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     const float i0 = 1.f / l0, i1 = 1.f / l1;
     const int r0 = q0 + g, r1 = q0 + g + 8;
     const int64_t g0 = (int64_t)n * T + r0, g1 = (int64_t)n * T + r1;  // output rows
-    unsigned long long nz0 = 0ull, nz1 = 0ull;  // non-zero columns of rows r0, r1 among this lane's
+    // which of this lane's values are non-zero: bit j column 8 j + 2 tq, bit 16 + j
+    // the one after it, of rows r0 and r1
+    uint32_t nz0 = 0u, nz1 = 0u;
+    const __nv_bfloat162 zero2 = __floats2bfloat162_rn(0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < HD / 8; ++j) {
       const int c = h * HD + j * 8 + 2 * tq;
-      const uint32_t w0 = pack_bf16x2(o[j][0] * i0, o[j][1] * i0), w1 = pack_bf16x2(o[j][2] * i1, o[j][3] * i1);
-      if (r0 < T) *reinterpret_cast<uint32_t*>(y + g0 * D + c) = w0;
-      if (r1 < T) *reinterpret_cast<uint32_t*>(y + g1 * D + c) = w1;
-      if (emit) {
-        const uint32_t n0 = r0 < T ? nz_pairs(w0) : 0u, n1 = r1 < T ? nz_pairs(w1) : 0u;
-        cnt[j] += n0 + n1;
-        nz0 |= (unsigned long long)((n0 | (n0 >> 15)) & 3u) << (8 * j + 2 * tq);
-        nz1 |= (unsigned long long)((n1 | (n1 >> 15)) & 3u) << (8 * j + 2 * tq);
-      }
+      const __nv_bfloat162 w0 = __floats2bfloat162_rn(o[j][0] * i0, o[j][1] * i0);
+      const __nv_bfloat162 w1 = __floats2bfloat162_rn(o[j][2] * i1, o[j][3] * i1);
+      if (r0 < T) *reinterpret_cast<__nv_bfloat162*>(y + g0 * D + c) = w0;
+      if (r1 < T) *reinterpret_cast<__nv_bfloat162*>(y + g1 * D + c) = w1;
+      nz0 |= __hneu2_mask(w0, zero2) & (0x00010001u << j);
+      nz1 |= __hneu2_mask(w1, zero2) & (0x00010001u << j);
     }
     if (emit) {
-      // a quad holds a row's HD columns
-#pragma unroll
-      for (int d = 1; d <= 2; d <<= 1) {
-        nz0 |= __shfl_xor_sync(0xffffffffu, nz0, d);
-        nz1 |= __shfl_xor_sync(0xffffffffu, nz1, d);
-      }
+      if (r0 >= T) nz0 = 0u;
+      if (r1 >= T) nz1 = 0u;
+      // row bits: a quad holds a row's HD columns
+      const uint32_t any0 = __ballot_sync(0xffffffffu, nz0 != 0u), any1 = __ballot_sync(0xffffffffu, nz1 != 0u);
       const int tile = (h * HD) >> 6;
       const unsigned long long bit = 1ull << (tile & 63);
-      if (tq == 0 && nz0) atomicOr(&occ.row_bm[g0 * occ.W64 + (tile >> 6)], bit);
-      if (tq == 0 && nz1) atomicOr(&occ.row_bm[g1 * occ.W64 + (tile >> 6)], bit);
-      // block-column words: HD columns from h HD on
-      auto mask_out = [&](unsigned long long m, int64_t b) {
-        const int c = h * HD, sh = c & 31;
-        const uint32_t lo = (uint32_t)m << sh, hi = HD > 32 ? (uint32_t)(m >> 32) : 0u;  // (HD = 64: sh = 0)
-        if (lo) atomicOr(&occ.blk_mask[b * occ.C32 + (c >> 5)], lo);
-        if (hi) atomicOr(&occ.blk_mask[b * occ.C32 + (c >> 5) + 1], hi);
+      if (tq == 0 && ((any0 >> (4 * g)) & 15u)) atomicOr(&occ.row_bm[g0 * occ.W64 + (tile >> 6)], bit);
+      if (tq == 0 && ((any1 >> (4 * g)) & 15u)) atomicOr(&occ.row_bm[g1 * occ.W64 + (tile >> 6)], bit);
+      // block-column words (HD columns from h HD on) of the one or two 128-row
+      // blocks that the tile's rows lie in
+      auto mask_out = [&](uint32_t v, int64_t b) {
+        // four bits to the low bits of four bytes: (x * (1 + 2^7 + 2^14 + 2^21)) & 0x01010101
+        auto spread = [](uint32_t x) { return ((x & 15u) * 0x00204081u) & 0x01010101u; };
+        const int c = h * HD, sh = c & 31;  // (HD = 64: sh = 0)
+        const uint32_t lo = __reduce_or_sync(0xffffffffu, (spread(v) | (spread(v >> 16) << 1)) << (2 * tq)) << sh;
+        if (lane == 0 && lo) atomicOr(&occ.blk_mask[b * occ.C32 + (c >> 5)], lo);
+        if constexpr (HD > 32) {
+          const uint32_t hi = __reduce_or_sync(0xffffffffu, (spread(v >> 4) | (spread(v >> 20) << 1)) << (2 * tq));
+          if (lane == 0 && hi) atomicOr(&occ.blk_mask[b * occ.C32 + (c >> 5) + 1], hi);
+        }
       };
-      const int64_t t0 = (int64_t)n * T + q0;
-      if ((t0 >> 7) == ((t0 + 15) >> 7)) {  // the tile's rows share a 128-row block
-        unsigned long long m = nz0 | nz1;
+      const int64_t b0 = ((int64_t)n * T + q0) >> 7;
+      const bool in0 = (g0 >> 7) == b0, in1 = (g1 >> 7) == b0;
+      mask_out((in0 ? nz0 : 0u) | (in1 ? nz1 : 0u), b0);
+      if ((((int64_t)n * T + q0 + 15) >> 7) != b0) mask_out((in0 ? 0u : nz0) | (in1 ? 0u : nz1), b0 + 1);
+      // column counts: rows r1's bits beside r0's, transposed over the warp
+      const uint32_t x = warp_transpose32(nz0 | (nz1 << 8));
 #pragma unroll
-        for (int d = 4; d <= 16; d <<= 1) m |= __shfl_xor_sync(0xffffffffu, m, d);
-        if (lane == 0) mask_out(m, t0 >> 7);
-      } else if (tq == 0) {
-        if (nz0) mask_out(nz0, g0 >> 7);
-        if (nz1) mask_out(nz1, g1 >> 7);
-      }
+      for (int i = 0; i < 4; ++i) cnt += (uint32_t)__popc(x & (0x11111111u << i)) << (8 * i);
     }
   }
   if (!emit) return;
+  cnt += __shfl_xor_sync(0xffffffffu, cnt, 8);  // (at most 5 tiles of 16 rows: bytes do not overflow)
+  if ((lane & 8) == 0 && (lane & 7) < HD / 8) {
 #pragma unroll
-  for (int j = 0; j < HD / 8; ++j) {  // (at most 512 rows: no carry between the halves)
-    uint32_t v = cnt[j];
-#pragma unroll
-    for (int d = 4; d <= 16; d <<= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-    if (g == 0) {
-      if (v & 0xFFFFu) atomicAdd(&s_cnt[8 * j + 2 * tq], v & 0xFFFFu);
-      if (v >> 16) atomicAdd(&s_cnt[8 * j + 2 * tq + 1], v >> 16);
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t v = (cnt >> (8 * i)) & 0xFFu;
+      if (v) atomicAdd(&s_cnt[8 * (lane & 7) + 2 * i + (lane >> 4)], v);
     }
   }
   __syncthreads();

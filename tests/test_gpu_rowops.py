@@ -77,6 +77,28 @@ def test_attention(sp, ctx, N, T, heads, hd, emit):
     assert_close(y.float().cpu().numpy(), orc.attention(qb, N, T, heads, hd), what=f"attention {N} {T} {heads} {hd}")
 
 
+@pytest.mark.parametrize("T", [31, 32, 33, 63, 64, 65, 96, 257])
+@pytest.mark.parametrize("hd", [16, 32, 64])
+def test_attention_key_blocks(sp, ctx, T, hd):
+    """Whole and partial blocks of 32 keys, scores far apart (the maxima move from
+    block to block), and images whose output is zero next to others in a block of rows."""
+    N, heads = 4, 3
+    D = heads * hd
+    g = torch.Generator().manual_seed(T * hd)
+    v = torch.randn(N, T, 3 * D, generator=g)
+    v[:, :, :D] *= 6.0
+    v[1, :, 2 * D:] = 0.0
+    v[3, :, 2 * D + hd: 2 * D + 2 * hd] = 0.0  # one head
+    qb = synth.to_bf16_bits(v)
+    y = torch.full((N, T, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+    yo = sp.OccupancyBuffer(N * T, D)
+    yo.buf.fill_(0x11)
+    sp.sparoa_attention(ctx, sp.bits_to_device(qb).view(N, T, 3 * D), y, heads, y_occ=yo)
+    assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), N * T, D), "attention")
+    # (bf16 probabilities, 2^-9 of a value below 5)
+    assert_close(y.float().cpu().numpy(), orc.attention(qb, N, T, heads, hd), what=f"attention {T} {hd}")
+
+
 @pytest.mark.parametrize("N,H,W,C", [(1, 127, 1, 8), (1, 128, 1, 64), (2, 37, 41, 72), (32, 56, 56, 64), (1, 224, 224, 16),
                                      (150, 20, 20, 128), (3, 7, 7, 1280)])
 def test_avgpool(sp, ctx, N, H, W, C):
