@@ -898,11 +898,17 @@ __global__ void __launch_bounds__(256) stats_narrow_kernel(const __nv_bfloat16* 
       cnt[c] += (uint32_t)__popcll(mc);
       chbits |= (mc != 0ull ? 1u : 0u) << c;
     }
-    if (g < groups) {
-      const int64_t r0 = g * 8;
+    // row words: bit p of a lane's byte is row p of its group; a store takes 32
+    // consecutive rows, from four lanes (each lane storing its own 8 rows touched
+    // four times the sectors: [1605632, 3] 10.2 us with its clear, now 5.6)
+    uint32_t rows = 0u;
 #pragma unroll
-      for (int p = 0; p < 8; ++p)
-        if (r0 + p < R) o.row_bm[r0 + p] = ((m >> (p * C)) & ((1ull << C) - 1ull)) ? 1ull : 0ull;
+    for (int p = 0; p < 8; ++p) rows |= (((m >> (p * C)) & ((1ull << C) - 1ull)) != 0ull ? 1u : 0u) << p;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const uint32_t byte = __shfl_sync(0xffffffffu, rows, 4 * k + (lane >> 3));
+      const int64_t r = g0 * 8 + 32 * k + lane;
+      if (r < R) o.row_bm[r] = (byte >> (lane & 7)) & 1u;
     }
     // block masks: lanes 0-15 and 16-31 are the blocks g0 / 16 and g0 / 16 + 1
     const uint32_t blo = __reduce_or_sync(0xffffffffu, lane < 16 ? chbits : 0u);
