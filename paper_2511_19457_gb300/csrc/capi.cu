@@ -1063,7 +1063,7 @@ sparoa_status sparoa_conv2d(sparoa_ctx* ctx, const void* x, int64_t N, int64_t H
         ckh = ckw = cstride = 1;
         cpad = 0;
         cols = true;
-      } else if (im2col_applies((int)C_in, kh, kw, groups, (int)W, pad)) {
+      } else if (im2col_applies((int)C_in, kh, kw, groups, (int)W, stride, pad)) {
         // a narrow stem as a GEMM of its im2col rows (a 1 x 1 conv over Kp channels)
         const int Kp = im2col_width((int)C_in, kh, kw);
         SP_TRY(ensure(ctx, ctx->pad_x, (size_t)(N * Ho * Wo * Kp * 2)));
@@ -1296,7 +1296,7 @@ sparoa_status plan_graph(sparoa_ctx* ctx, const sparoa_op* ops, int32_t n_ops, i
         if (!dw && stem_plan(nullptr, in.n, (int)in.h, (int)in.w, op.c_in, op.c_out, op.kh, op.kw, op.stride, op.pad, &sg)) {
           aux[(size_t)i].stem = true;
           aux[(size_t)i].cp = op.kh * sg.seg;
-        } else if (!dw && im2col_applies(op.c_in, op.kh, op.kw, op.groups, (int)in.w, op.pad)) {
+        } else if (!dw && im2col_applies(op.c_in, op.kh, op.kw, op.groups, (int)in.w, op.stride, op.pad)) {
           aux[(size_t)i].cols = true;
           aux[(size_t)i].cp = im2col_width(op.c_in, op.kh, op.kw);
         } else if (!dw && op.c_in % 8) {

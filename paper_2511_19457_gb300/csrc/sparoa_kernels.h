@@ -236,9 +236,9 @@ cudaError_t launch_stats(const __nv_bfloat16* x, int64_t R, int C, const OccDev&
 // im2col for a convolution with few input channels (k_tiles.cu): x [N, H, W,
 // C] -> xc [N Ho Wo, Kp], each row the [kh][kw][C] window of one output pixel,
 // zero-padded to Kp = im2col_width(C, kh, kw) (see im2col_kernel); for groups
-// == 1, C < 8, kh kw > 1 and small enough windows (im2col_applies).
+// == 1, C < 8, kh kw > 1 and small enough or separate windows (im2col_applies).
 int im2col_width(int C, int kh, int kw);
-bool im2col_applies(int C, int kh, int kw, int groups, int W, int P);
+bool im2col_applies(int C, int kh, int kw, int groups, int W, int S, int P);
 cudaError_t launch_im2col(const __nv_bfloat16* x, int N, int H, int W, int C, int kh, int kw, int S, int P,
                           __nv_bfloat16* xc, cudaStream_t s);
 

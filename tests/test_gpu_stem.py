@@ -66,3 +66,27 @@ def test_infinity_stays_in_its_windows(sp, ctx):
     sp.sparoa_conv2d(ctx, x, w, y, stride=2, pad=3)
     ref = torch.nn.functional.conv2d(x.float().permute(0, 3, 1, 2), w.float().permute(0, 3, 1, 2), stride=2, padding=3)
     assert torch.equal(torch.isfinite(y), torch.isfinite(ref.permute(0, 2, 3, 1)))
+
+
+@pytest.mark.parametrize("B,H,W,C,Co,k,stride", [
+    (2, 64, 48, 3, 64, 16, 16), (1, 70, 61, 3, 768, 14, 14),  # images that are not whole patches
+    (3, 40, 45, 4, 40, 13, 15),                              # gaps between the windows
+    (9, 50, 50, 3, 72, 25, 25),                              # 1875 values a window
+    (2, 54, 54, 3, 64, 27, 27),                              # 2187: past the limit
+    (5, 16, 16, 7, 128, 16, 16)])                            # one window an image
+@pytest.mark.parametrize("force", [1, 2])
+def test_patch_embedding(sp, ctx, B, H, W, C, Co, k, stride, force):
+    """windows of more than 512 values that do not overlap"""
+    d = synth.conv_layer(seed=H + W, N=B, H=H, W=W, Cin=C, Cout=Co, k=k, stride=stride, pad=0, bn="random")
+    Ho, Wo = (H - k) // stride + 1, (W - k) // stride + 1
+    R = B * Ho * Wo
+    y = torch.full((B, Ho, Wo, Co), float("nan"), dtype=torch.bfloat16, device="cuda")
+    yo = sp.OccupancyBuffer(R, Co)
+    yo.buf.fill_(0x3C)
+    st = sp.sparoa_conv2d(ctx, sp.bits_to_device(d["x"]).view(B, H, W, C), sp.bits_to_device(d["w"]).view(Co, k, k, C), y,
+                          stride=stride, pad=0, bn=torch.from_numpy(d["bn"]).cuda(), act=1,
+                          thr=sp.thresholds(force_path=force), y_occ=yo, host=True)
+    assert st.path == force and st.nnz == orc.stats(d["x"], B * H * W, C).nnz
+    ref = orc.conv2d(d["x"], B, H, W, C, d["w"], Co, k, k, stride, 0, bn=d["bn"], act=1)
+    assert_close(y.float().cpu().numpy(), ref, what="patches")
+    assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), R, Co), "patches")
