@@ -1713,6 +1713,7 @@ void choose_tiles(const IgemmArgs& a, int64_t mtiles, int* bn_out, int* ks_out) 
   if (bn == 128) {
     int64_t best = ((tiles + sms - 1) / sms) * (128 + 128);
     for (int cand = 192; cand <= 256 && cand < a.N + 64; cand += 64) {
+      if (cand == 192 && a.N > 4096) continue;  // a tile's columns lie in one word of the row bitmap
       const int64_t t = mtiles * ((a.N + cand - 1) / cand);
       const int64_t cost = ((t + sms - 1) / sms) * (128 + cand);
       if (cost < best) {

@@ -52,3 +52,23 @@ def test_pointwise(sp, ctx, B, H, W, C, Co, stride, act, res, force):
     assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), R, Co), "occupancy")
     ref = orc.conv2d(d["x"], B, H, W, C, d["w"], Co, 1, 1, stride, 0, bn=d["bn"], residual_bits=rb, act=act)
     assert_close(y.float().cpu().numpy(), np.asarray(ref).reshape(y.shape), what="pointwise")
+
+
+@pytest.mark.parametrize("M,N", [(1576, 6144), (130, 4104), (4000, 8200)])
+def test_more_than_one_row_word(sp, ctx, M, N):
+    """outputs of more than 4096 columns: every row has several bitmap words, and no
+    tile's columns may lie in two"""
+    g = torch.Generator().manual_seed(M)
+    x = torch.randn(M, 64, generator=g)
+    w = torch.randn(N, 64, generator=g)
+    w[4032:4096] = 0.0  # the last 64 columns of the first word, and the first of the second
+    w[4160:4200] = 0.0
+    xb, wb = synth.to_bf16_bits(x), synth.to_bf16_bits(w)
+    y = torch.full((M, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+    xo, yo = sp.OccupancyBuffer(M, 64), sp.OccupancyBuffer(M, N)
+    yo.buf.fill_(0x5A)
+    xd, wd = sp.bits_to_device(xb).view(M, 64), sp.bits_to_device(wb).view(N, 64)
+    sp.sparoa_op_stats(ctx, xd, (M, 64), occ=xo)
+    sp.sparoa_gemm(ctx, xd, wd, y, x_occ=xo, y_occ=yo, thr=sp.thresholds(force_path=1))
+    assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), M, N), "occupancy")
+    assert_close(y.float().cpu().numpy(), (xd.double() @ wd.double().T).cpu().numpy(), what="gemm")
