@@ -1651,6 +1651,12 @@ cudaError_t launch_bn(const IgemmArgs& a, int bn, int bk, const CUtensorMap& tA,
   if (bk == 64) {
     switch (bn) {
       case 64: return launch_cfg<64, 64, LEAN>(a, tA, tB, tY, tA32, tB32, tiles, s);
+      case 96:
+        if constexpr (LEAN) return launch_cfg<96, 64, LEAN>(a, tA, tB, tY, tA32, tB32, tiles, s);
+        return cudaErrorInvalidValue;  // (choose_tiles: lean kernels only)
+      case 160:
+        if constexpr (LEAN) return launch_cfg<160, 64, LEAN>(a, tA, tB, tY, tA32, tB32, tiles, s);
+        return cudaErrorInvalidValue;
       case 128: return launch_cfg<128, 64, LEAN>(a, tA, tB, tY, tA32, tB32, tiles, s);
       case 192: return launch_cfg<192, 64, LEAN>(a, tA, tB, tY, tA32, tB32, tiles, s);
       default: return launch_cfg<256, 64, LEAN>(a, tA, tB, tY, tA32, tB32, tiles, s);
@@ -1693,11 +1699,14 @@ void choose_spatial_tile(IgemmArgs& a) {
 // N tile and K split.  The main loop is bound by shared-memory traffic: a
 // K block of a 128 x BN tile is written by TMA and read back by the MMAs,
 // (128 + BN) rows each way, so a tile costs about (128 + BN) per K block and
-// the tiles take ceil(tiles / SMs) rounds over the SMs.  Of 128, 192 and 256
-// wide tiles the cheapest total wins, ties going to the narrower (a shorter
-// epilogue); 64 wide ones when 128 wide tiles would fill under half of the
-// SMs.  On GB300, GEMMs with M 1024..8192, K 768..3072 and N 768..3072 follow
-// this ordering.  K blocks are 64 wide (128-byte swizzle) wherever the
+// the tiles take ceil(tiles / SMs) rounds over the SMs.  Of 96, 128, 160, 192
+// and 256 wide tiles the cheapest total wins, ties going to 128 and then to the
+// narrower (a shorter epilogue); 64 wide ones when 128 wide tiles would fill under
+// half of the SMs.  On GB300, GEMMs with M 1024..8192, K 768..3072 and N
+// 768..3072 follow this ordering.  96 and 160: lean kernels with 64-wide K blocks;
+// with weights in L2 they gain little (1576 rows x 3072 columns 11.9 -> 11.5 us),
+// with weights from memory the additional CTAs have
+// more loads in flight (ViT-B/16 at batch 8, 1576 rows: 1175 -> 1139 us).  K blocks are 64 wide (128-byte swizzle) wherever the
 // channel layout allows: 32 wide ones were slower at every tile width.
 // 64-wide tiles that number at most the SMs go to the one-tile-per-cluster
 // kernel (k_onetile.cu), which shares a tile's K range through distributed
@@ -1706,14 +1715,19 @@ void choose_spatial_tile(IgemmArgs& a) {
 // blocks per unit (the tile's last unit reads the other partials alone).
 static int k_block(const IgemmArgs& a) { return (a.conv == 2 ? (a.Cp % 64 == 0) : (a.Ktot > 32)) ? 64 : 32; }
 
-void choose_tiles(const IgemmArgs& a, int64_t mtiles, int* bn_out, int* ks_out) {
+void choose_tiles(const IgemmArgs& a, int64_t mtiles, bool lean, int* bn_out, int* ks_out) {
   const int sms = device_sm_count();
   int bn = a.N > 64 ? 128 : 64;
   int64_t tiles = mtiles * ((a.N + bn - 1) / bn);
-  if (bn == 128) {
+  if (bn == 128 && tiles < sms / 2) {
+    bn = 64;
+    tiles = mtiles * ((a.N + bn - 1) / bn);
+  } else if (bn == 128) {
     int64_t best = ((tiles + sms - 1) / sms) * (128 + 128);
-    for (int cand = 192; cand <= 256 && cand < a.N + 64; cand += 64) {
-      if (cand == 192 && a.N > 4096) continue;  // a tile's columns lie in one word of the row bitmap
+    for (const int cand : {96, 160, 192, 256}) {
+      if (cand >= a.N + 64) break;
+      if (cand != 256 && a.N > 4096) continue;  // a tile's columns lie in one word of the row bitmap
+      if (cand % 64 && !(lean && k_block(a) == 64)) continue;
       const int64_t t = mtiles * ((a.N + cand - 1) / cand);
       const int64_t cost = ((t + sms - 1) / sms) * (128 + cand);
       if (cost < best) {
@@ -1721,10 +1735,6 @@ void choose_tiles(const IgemmArgs& a, int64_t mtiles, int* bn_out, int* ks_out) 
         bn = cand;
         tiles = t;
       }
-    }
-    if (bn == 128 && tiles < sms / 2) {
-      bn = 64;
-      tiles = mtiles * ((a.N + bn - 1) / bn);
     }
   }
   const int bk = k_block(a);
@@ -1801,7 +1811,10 @@ cudaError_t launch_igemm(const IgemmArgs& a_in, cudaStream_t s) {
   const int64_t mtiles =
       a.conv == 2 ? (int64_t)((a.Nimg + a.bn - 1) / a.bn) * a.th * a.tw : (a.M + kBM - 1) / kBM;
   int bn = 64, ks = 1;
-  choose_tiles(a, mtiles, &bn, &ks);
+  const bool lean = a.conv != 1 && !a.y_f32 && !a.dense_only &&
+                    (a.ep.residual == nullptr ||
+                     (a.N % 8 == 0 && (reinterpret_cast<uintptr_t>(a.ep.residual) & 15u) == 0));
+  choose_tiles(a, mtiles, lean, &bn, &ks);
   a.ksplit = ks;
   const int bk = k_block(a);
   if (bn == 64) {
@@ -1843,9 +1856,6 @@ cudaError_t launch_igemm(const IgemmArgs& a_in, cudaStream_t s) {
       return cudaErrorInvalidValue;
   }
   const int64_t tiles = mtiles * ((a.N + bn - 1) / bn);
-  const bool lean = a.conv != 1 && ks == 1 && !a.y_f32 && !a.dense_only &&
-                    (a.ep.residual == nullptr ||
-                     (a.N % 8 == 0 && (reinterpret_cast<uintptr_t>(a.ep.residual) & 15u) == 0));
   if (!lean) return launch_bn<0>(a, bn, bk, tA, tB, tY, tA32, tB32, tiles, s);
   return a.ep.residual ? launch_bn<2>(a, bn, bk, tA, tB, tY, tA32, tB32, tiles, s)
                        : launch_bn<1>(a, bn, bk, tA, tB, tY, tA32, tB32, tiles, s);

@@ -72,3 +72,38 @@ def test_more_than_one_row_word(sp, ctx, M, N):
     sp.sparoa_gemm(ctx, xd, wd, y, x_occ=xo, y_occ=yo, thr=sp.thresholds(force_path=1))
     assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), M, N), "occupancy")
     assert_close(y.float().cpu().numpy(), (xd.double() @ wd.double().T).cpu().numpy(), what="gemm")
+
+
+@pytest.mark.parametrize("M,K,N,act,res", [
+    (1576, 768, 768, 0, True), (1576, 768, 3072, 3, False), (20000, 64, 96, 1, False), (20000, 144, 136, 2, True),
+    (77777, 200, 72, 1, False), (1500, 1000, 760, 1, True), (40000, 96, 152, 0, False)])
+@pytest.mark.parametrize("force", [1, 2])
+def test_tiles_of_96_and_160_columns(sp, ctx, M, K, N, act, res, force):
+    """one and several tiles per CTA, several column tiles, the last one partial"""
+    g = torch.Generator().manual_seed(N)
+    x = torch.randn(M, K, generator=g)
+    x[(torch.rand((M + 127) // 128, (K + 31) // 32, generator=g) < 0.4)
+      .repeat_interleave(128, 0)[:M].repeat_interleave(32, 1)[:, :K]] = 0.0  # whole 128 x 32 blocks
+    w = torch.randn(N, K, generator=g) / K ** 0.5
+    w[N // 3: N // 3 + 40] = 0.0
+    b = torch.randn(N, generator=g)
+    b[N // 3: N // 3 + 40] = 0.0
+    r = torch.randn(M, N, generator=g) * (torch.rand(M, N, generator=g) < 0.5) if res else None
+    xd = sp.bits_to_device(synth.to_bf16_bits(x)).view(M, K)
+    wd = sp.bits_to_device(synth.to_bf16_bits(w)).view(N, K)
+    rd = sp.bits_to_device(synth.to_bf16_bits(r)).view(M, N) if res else None
+    bd = b.cuda()
+    y = torch.full((M, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+    xo, yo = sp.OccupancyBuffer(M, K), sp.OccupancyBuffer(M, N)
+    yo.buf.fill_(0x5A)
+    sp.sparoa_op_stats(ctx, xd, (M, K), occ=xo)
+    sp.sparoa_gemm(ctx, xd, wd, y, bias=bd, act=act, x_occ=xo, y_occ=yo, residual=rd,
+                   thr=sp.thresholds(force_path=force))
+    assert ctx.last_path() == force
+    assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), M, N), "occupancy")
+    v = xd.double() @ wd.double().T + bd.double()
+    if res:
+        v = v + rd.double()
+    v = {0: lambda t: t, 1: torch.relu, 2: lambda t: t.clamp(0, 6),
+         3: lambda t: torch.nn.functional.gelu(t, approximate="tanh")}[act](v)
+    assert_close(y.float().cpu().numpy(), v.cpu().numpy(), what="gemm")
