@@ -393,6 +393,9 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
+  if constexpr (LEAN && !STEM) {
+    if (warp == Wp::kMma) prefetch_weights_l2(P.w, p.N, p.Ktot, lane);
+  }
   pdl_wait();
   pdl_trigger();
   const int path = decide_path(P.disp);
