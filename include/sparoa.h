@@ -296,7 +296,7 @@ sparoa_status sparoa_op_stats(sparoa_ctx *ctx, const void *x, int64_t N, int64_t
  * path: for M <= 128 with W_kn given, a column-compacting kernel that reads
  * only the rows of W_kn whose activation column is occupied; otherwise a
  * tcgen05 GEMM that stages only the 32-wide K blocks occupied in each 128-row
- * block of x.
+ * block of x (with few output tiles 64-wide ones, after the first eight).
  *   W_kn    optional [K][N] copy of W (nullable)
  *   y_dtype SPAROA_BF16 or SPAROA_F32
  *   y_occ   occupancy of y to write (nullable; bf16 y only)

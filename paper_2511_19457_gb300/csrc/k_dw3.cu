@@ -11,7 +11,7 @@
 // accumulators and the 36 weights stay in registers.  Channels go in pairs
 // through packed fp32x2 FMAs, in the order kernel row, then kernel column.
 //
-// Input rows reach shared memory as 4-D TMA boxes {32 channels, IW, S rows, 1}
+// Input rows reach shared memory as 4-D TMA boxes {32 channels, IW, 3 rows (stride 2: 2), 1}
 // (coordinates outside the image read zeros, which is the padding) through a
 // ring of boxes per warp that runs on across items.
 //
@@ -24,8 +24,8 @@
 // 28.7 / 40.2 and 23.6 / 29.8 us.
 //
 // Occupancy: a warp's slice is one 32-channel word of the 128-row block masks,
-// which gather in registers until the rows leave the block; row bits are voted
-// per pixel; column counts are 16-bit halves per lane, summed per item into
+// which gather in registers until the rows leave the block; row bits are ORed over
+// a pixel's lanes; column counts are 16-bit halves per lane, summed per item into
 // shared memory and once per CTA into global memory.
 #include <cuda.h>
 #include <cudaTypedefs.h>

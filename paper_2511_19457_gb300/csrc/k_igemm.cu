@@ -48,7 +48,7 @@
 // that fit the ring.  Measured (GB300, BN + ReLU6 + output occupancy): the 1x1
 // expansion [32,112,112,16] -> 96 53.5 -> 34.5 us (90 MB: 2.6 TB/s; 22.9 without
 // the occupancy), [32,56,56,24] -> 144 35.9 -> 22.9 us, the MLP's up projection
-// [6304,768] x [3072,768] + GELU 48 -> 45 us.  One column block's instructions
+// [6304,768] x [3072,768] + GELU 48 -> 34 us.  One column block's instructions
 // appear once: a second copy (planes of two blocks in registers) cost the wide
 // tiles 10 % in instruction-cache misses.
 #include <cuda.h>
