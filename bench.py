@@ -1229,7 +1229,7 @@ def run_profile(args, rank, local_rank, world, peaks):
         y = torch.empty(32, 112, 112, 96, dtype=torch.bfloat16, device=dev)
         yo = sp.OccupancyBuffer(32 * 112 * 112, 96)
         call = lambda: sp.sparoa_conv2d(ctx, x, w, y, bn=bnp, act=sp.ACT_RELU6, y_occ=yo)
-    elif op == "stem7x7":  # ResNet-18's stem at batch 32: im2col rows, then a GEMM; BN + ReLU
+    elif op == "stem7x7":  # ResNet-18's stem at batch 32, BN + ReLU
         x = act(32, 224, 224, 3, zero_p=0.0)
         w = (torch.randn(64, 7, 7, 3, device=dev, generator=gen) / 12).to(torch.bfloat16)
         bnp = torch.tensor(synth.identity_bn(64), device=dev)

@@ -15,7 +15,7 @@
 // (coordinates outside the image read zeros, which is the padding) through a
 // ring of boxes per warp that runs on across items.
 //
-// Bound by issued instructions (FMAs are less than a third of them), so the rows
+// Bound by instruction issue and latency (FMAs are under a third), so the rows
 // come three to a box (one wait and one request for them), pointers advance by
 // constants and a value is widened once.  [32, 56, 56, 144] stride 1 without / with
 // occupancy 18.5 / 25.8 us, [32, 112, 112, 96] stride 2 17.6 / 23.1 us; CTAs of
