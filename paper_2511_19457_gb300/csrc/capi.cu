@@ -1067,13 +1067,15 @@ sparoa_status sparoa_conv2d(sparoa_ctx* ctx, const void* x, int64_t N, int64_t H
         // a narrow stem as a GEMM of its im2col rows (a 1 x 1 conv over Kp channels)
         const int Kp = im2col_width((int)C_in, kh, kw);
         SP_TRY(ensure(ctx, ctx->pad_x, (size_t)(N * Ho * Wo * Kp * 2)));
-        SP_TRY(ensure(ctx, ctx->pad_w, (size_t)(C_out * Kp * 2)));
         SP_CUDA(launch_im2col(static_cast<const __nv_bfloat16*>(x), (int)N, (int)H, (int)W, (int)C_in, kh, kw,
                               stride, pad, static_cast<__nv_bfloat16*>(ctx->pad_x.p), ctx->stream));
-        SP_CUDA(launch_pad_channels(static_cast<const __nv_bfloat16*>(w), C_out, kh * kw * (int)C_in, Kp,
-                                    static_cast<__nv_bfloat16*>(ctx->pad_w.p), ctx->stream));
         c.x = ctx->pad_x.p;
-        c.w = ctx->pad_w.p;
+        if (Kp != kh * kw * C_in || !aligned16(w)) {  // (else the weights are these rows already)
+          SP_TRY(ensure(ctx, ctx->pad_w, (size_t)(C_out * Kp * 2)));
+          SP_CUDA(launch_pad_channels(static_cast<const __nv_bfloat16*>(w), C_out, kh * kw * (int)C_in, Kp,
+                                      static_cast<__nv_bfloat16*>(ctx->pad_w.p), ctx->stream));
+          c.w = ctx->pad_w.p;
+        }
         c.H = Ho;
         c.W = Wo;
         c.Cin = Kp;
@@ -1532,11 +1534,13 @@ sparoa_status sparoa_run_graph(sparoa_ctx* ctx, const sparoa_op* ops, int32_t n_
           void* pw = base + aux[(size_t)i].padw;
           SP_CUDA(launch_im2col(static_cast<const __nv_bfloat16*>(c.x), (int)in.n, (int)in.h, (int)in.w, (int)in.c,
                                 op.kh, op.kw, op.stride, op.pad, static_cast<__nv_bfloat16*>(px), ctx->stream));
-          SP_CUDA(launch_pad_channels(static_cast<const __nv_bfloat16*>(op.weight), (int64_t)op.c_out,
-                                      op.kh * op.kw * (int)in.c, (int)c.Cp, static_cast<__nv_bfloat16*>(pw),
-                                      ctx->stream));
           c.x = px;
-          c.w = pw;
+          if (c.Cp != op.kh * op.kw * in.c || !aligned16(op.weight)) {  // (else the weights are these rows already)
+            SP_CUDA(launch_pad_channels(static_cast<const __nv_bfloat16*>(op.weight), (int64_t)op.c_out,
+                                        op.kh * op.kw * (int)in.c, (int)c.Cp, static_cast<__nv_bfloat16*>(pw),
+                                        ctx->stream));
+            c.w = pw;
+          }
           c.H = out.h;
           c.W = out.w;
           c.Cin = c.Cp;

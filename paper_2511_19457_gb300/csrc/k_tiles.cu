@@ -1352,7 +1352,7 @@ int im2col_width(int C, int kh, int kw) { return (kh * kw * C + 31) / 32 * 32; }
 // image (patch embeddings): their rows are then no larger than x, against x with
 // its channels padded to 8 and a K as much wider for the gather that loads such
 // windows otherwise (16x16/16 of [8, 224, 224, 3] to 768 channels: K 2048
-// instead of 768, 37.0 us; 18.4 us as a GEMM).  2048: a thread per 16-byte
+// instead of 768, 37.0 us; 16.3 us as a GEMM).  2048: a thread per 16-byte
 // chunk of a row.
 bool im2col_applies(int C, int kh, int kw, int groups, int W, int S, int P) {
   if (groups != 1 || C >= 8 || kh * kw <= 1) return false;
