@@ -58,3 +58,29 @@ def test_depthwise_edges(sp, ctx, N, H, W, C, act, res, s):
     assert_close(y.float().cpu().numpy().astype(np.float64),
                  orc.conv2d(xb, N, H, W, C, wb, C, 3, 3, s, 1, groups=C, bn=bn, residual_bits=rb, act=act), what=what)
     assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), N * Ho * Wo, C), what)
+
+
+@pytest.mark.parametrize("kind", ["dw", "pointwise", "attention"])
+def test_subnormal_outputs_count(sp, ctx, kind):
+    """occupancy counts every bf16 pattern but +-0, subnormal values among them"""
+    C, R = 64, 4 * 9 * 11
+    pat = np.resize(np.array([0x0001, 0x8001, 0x0000, 0x8000, 0x007F, 0x3F80, 0x0010], dtype=np.uint16), R * C)
+    yo = sp.OccupancyBuffer(R, C)
+    yo.buf.fill_(0x77)
+    x = sp.bits_to_device(pat)
+    y = torch.full((R, C), float("nan"), dtype=torch.bfloat16, device="cuda")
+    if kind == "dw":
+        w = torch.zeros(C, 3, 3, 1, dtype=torch.bfloat16, device="cuda")
+        w[:, 1, 1] = 1.0
+        sp.sparoa_conv2d(ctx, x.view(4, 9, 11, C), w, y.view(4, 9, 11, C), stride=1, pad=1, groups=C, y_occ=yo)
+    elif kind == "pointwise":
+        w = torch.eye(C, device="cuda").to(torch.bfloat16).view(C, 1, 1, C).contiguous()
+        sp.sparoa_conv2d(ctx, x.view(4, 9, 11, C), w, y.view(4, 9, 11, C), stride=1, pad=0, y_occ=yo)
+    else:
+        qkv = torch.zeros(R, 1, 3 * C, dtype=torch.bfloat16, device="cuda")  # one token: the output is v
+        qkv[:, 0, 2 * C:] = x.view(R, C)
+        sp.sparoa_attention(ctx, qkv, y.view(R, 1, C), 1, y_occ=yo)
+    yb = sp.device_to_bits(y).reshape(-1)
+    if kind == "dw":
+        assert np.array_equal(yb & 0x7FFF, pat & 0x7FFF)
+    assert_occ_equal(yo.to_host(), orc.stats(yb, R, C), kind)
