@@ -485,7 +485,7 @@ cudaError_t launch_shape(const DwArgs& a, cudaStream_t s) {
   const long long all = (long long)device_sm_count() * Sh::kWarps;
   double best = 0.;
   g.run = 0;
-  for (int c = (a.Ho + kMaxRun - 1) / kMaxRun; c <= a.Ho; ++c) {
+  for (int c = (a.Ho + kMaxRun - 1) / kMaxRun;;) {
     const int run = (a.Ho + c - 1) / c, runs = (a.Ho + run - 1) / run;
     const double cost = (double)((base * runs + all - 1) / all) * (S == 1 ? 3 * Sh::boxes(run) + 1 : run + 3);
     if (g.run == 0 || cost < best) {
@@ -494,6 +494,7 @@ cudaError_t launch_shape(const DwArgs& a, cudaStream_t s) {
       g.runs = runs;
     }
     if (base * runs > 8 * all || run == 1) break;
+    c = (a.Ho + run - 2) / (run - 1);  // the fewest runs that are shorter
   }
   if (base * g.runs >= (1ll << 31)) return cudaErrorInvalidValue;
   g.items = (uint32_t)(base * g.runs);
