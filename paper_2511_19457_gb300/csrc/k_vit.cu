@@ -54,8 +54,10 @@ __global__ void __launch_bounds__(kLnThreads, 1)
   const int64_t r0 = w * R / warps, r1 = (w + 1) * R / warps;
   const int chunks = C / 8;
   const float inv_c = 1.f / (float)C;
-  if (emit)
+  if (emit) {
     for (int c = threadIdx.x; c < NCH * 256; c += blockDim.x) s_cnt[c] = 0u;
+    __syncthreads();  // a warp adds its counts as soon as its own rows are done
+  }
   pdl_wait();
   pdl_trigger();
   uint4 u[NCH];

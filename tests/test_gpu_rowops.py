@@ -109,3 +109,18 @@ def test_avgpool(sp, ctx, N, H, W, C):
     sp.sparoa_avgpool_global(ctx, sp.bits_to_device(xb).view(N, H, W, C), y, y_occ=yo)
     assert_close(y.float().cpu().numpy(), orc.avgpool_global(xb, N, H, W, C), what="avgpool")
     assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), N, C), "avgpool")
+
+
+@pytest.mark.parametrize("R,C", [(7, 1024), (1208, 1024), (1216, 768)])
+def test_layernorm_counts_of_short_runs(sp, ctx, R, C):
+    """One row a warp, so that a warp adds its column counts as early as it can:
+    the same counters after every one of many calls, back to back."""
+    xb = _bits((R, C), R)
+    x = sp.bits_to_device(xb).view(R, C)
+    y = torch.empty(R, C, dtype=torch.bfloat16, device="cuda")
+    occ = [sp.OccupancyBuffer(R, C) for _ in range(64)]
+    for yo in occ:
+        sp.sparoa_layernorm(ctx, x, y, y_occ=yo)
+    want = orc.stats(sp.device_to_bits(y).reshape(-1), R, C)
+    for yo in occ:
+        assert_occ_equal(yo.to_host(), want, f"layernorm {R}x{C}")
