@@ -124,3 +124,26 @@ def test_layernorm_counts_of_short_runs(sp, ctx, R, C):
     want = orc.stats(sp.device_to_bits(y).reshape(-1), R, C)
     for yo in occ:
         assert_occ_equal(yo.to_host(), want, f"layernorm {R}x{C}")
+
+
+@pytest.mark.parametrize("T", [64, 197, 257])
+@pytest.mark.parametrize("hd", [16, 32, 64])
+def test_attention_large_scores(sp, ctx, T, hd):
+    """Scores of 2^22 plus a few units, exact in fp32, whose maximum rises from one
+    block of keys to the next: the weights depend on the differences alone.  Rounding
+    s / sqrt(hd) and its maximum before the difference puts blocks 2^-5 apart
+    (relative Frobenius error of such a softmax on the CPU: 6e-3 to 5e-2); with the
+    difference first the probabilities' and the output's bf16 rounding is left, 2e-3
+    to 2.5e-3."""
+    g = torch.Generator().manual_seed(T + hd)
+    v = torch.randn(1, T, 3 * hd, generator=g)
+    q, k = torch.zeros(T, hd), torch.zeros(T, hd)
+    q[:, 0] = k[:, 0] = 2048.0
+    q[:, 1] = 1.0
+    t = torch.arange(T)
+    k[:, 1] = (2 * (t // 32) + (7 * t) % 5).float()
+    v[0, :, :hd], v[0, :, hd:2 * hd] = q, k
+    qb = synth.to_bf16_bits(v)
+    y = torch.full((1, T, hd), float("nan"), dtype=torch.bfloat16, device="cuda")
+    sp.sparoa_attention(ctx, sp.bits_to_device(qb).view(1, T, 3 * hd), y, 1)
+    assert_close(y.float().cpu().numpy(), orc.attention(qb, 1, T, 1, hd), what=f"attention {T} {hd}")
