@@ -281,13 +281,6 @@ constexpr int kAttnThreads = 32 * kAttnWarps;
 constexpr int kAttnMaxT = 512;
 constexpr int kAttnKB = 32;        // keys per block
 
-// 2^x; results below the normal range are zero (they are probabilities)
-__device__ __forceinline__ float exp2_ftz(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                                uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
@@ -448,7 +441,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       bm0 = fmaxf(bm0, __shfl_xor_sync(0xffffffffu, bm0, 2));
       bm1 = fmaxf(bm1, __shfl_xor_sync(0xffffffffu, bm1, 2));
       const float nm0 = fmaxf(m0, bm0), nm1 = fmaxf(m1, bm1);
-      const float c0 = exp2_ftz((m0 - nm0) * sl2), c1 = exp2_ftz((m1 - nm1) * sl2);
+      const float c0 = exp2f((m0 - nm0) * sl2), c1 = exp2f((m1 - nm1) * sl2);
       m0 = nm0;
       m1 = nm1;
       // exponents (s - max) sl2, the difference first: it is exact for scores near
@@ -464,10 +457,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
         if (FULL || kb + nt * 8 < T) {  // uniform across the warp
           f2_split(fmul2(fadd2(f2(s[nt][0], s[nt][1]), n02), sc2), p0, p1);
           f2_split(fmul2(fadd2(f2(s[nt][2], s[nt][3]), n12), sc2), p2, p3);
-          p0 = exp2_ftz(p0);
-          p1 = exp2_ftz(p1);
-          p2 = exp2_ftz(p2);
-          p3 = exp2_ftz(p3);
+          p0 = exp2f(p0);
+          p1 = exp2f(p1);
+          p2 = exp2f(p2);
+          p3 = exp2f(p3);
         }
         rs0 += p0 + p1;
         rs1 += p2 + p3;

@@ -147,3 +147,24 @@ def test_attention_large_scores(sp, ctx, T, hd):
     y = torch.full((1, T, hd), float("nan"), dtype=torch.bfloat16, device="cuda")
     sp.sparoa_attention(ctx, sp.bits_to_device(qb).view(1, T, 3 * hd), y, 1)
     assert_close(y.float().cpu().numpy(), orc.attention(qb, 1, T, 1, hd), what=f"attention {T} {hd}")
+
+
+@pytest.mark.parametrize("far", [1, 40])
+def test_attention_weights_below_the_normal_range(sp, ctx, far):
+    """Key 0 has a value of 2^125 and a weight of 2^-128.4 (key `far` scores 712 / 8
+    higher, in the same block of keys or in a later one): fp32 and bf16 hold such
+    weights as subnormals, and the output is 2^-3.4.  In the same block the weight
+    is rounded to a multiple of 2^-133: within 2^-134 / 2^-128.4 = 2.1 %."""
+    T, hd = 64, 64
+    v = torch.zeros(1, T, 3 * hd)
+    v[0, :, 0], v[0, :, hd] = 8.0, -1024.0
+    v[0, 0, hd], v[0, far, hd] = 0.0, 89.0
+    v[0, 0, 2 * hd] = 2.0 ** 125
+    qb = synth.to_bf16_bits(v)
+    y = torch.full((1, T, hd), float("nan"), dtype=torch.bfloat16, device="cuda")
+    sp.sparoa_attention(ctx, sp.bits_to_device(qb).view(1, T, 3 * hd), y, 1)
+    want = orc.attention(qb, 1, T, 1, hd).reshape(T, hd)
+    got = y.float().cpu().numpy().reshape(T, hd)
+    assert want[0, 0] > 0.09
+    assert np.abs(got[:, 0] / want[:, 0] - 1).max() <= 0.021 + 2.0 ** -9
+    assert not got[:, 1:].any()
