@@ -1159,49 +1159,29 @@ __global__ void __launch_bounds__(kTileThreads) dwconv_kernel(const DwArgs a_par
 }
 
 // ---------------------------------------------------------------------------
-// Global average pooling [N, HW, C] -> [N, C] (C % 8 == 0): one cluster of 1 to
-// 8 CTAs per (image, 64-channel slice), which share its pixels, so that large
-// maps of few channels fill the chip ([32,56,56,64]: 32 CTAs, 29 us, before;
-// 256 CTAs now).  Lane l of warp w of CTA r sums pixels 32 r + 4 w + l / 8 + 32
-// S k of the 8 channels 8 (l % 8) .. + 7, four loads in flight; the partial sums
-// of a channel meet by shuffles, in shared memory and, in rank order, in the
-// first CTA's, whose threads 0..63 finish one channel each: the mean, its bf16
-// value and the output occupancy (atomics into the cleared block: row bit,
-// column, tile and total counts, block-column mask words).
-__global__ void __launch_bounds__(kTileThreads)
-    avgpool_kernel(const __nv_bfloat16* __restrict__ x, int N, int HW, int C,
-                   __nv_bfloat16* __restrict__ y, OccDev o_param, int emit, int S) {
-  const OccDev o = o_param;
-  __shared__ float s_part[8 * 64];   // [warp][channel of the slice]
-  __shared__ float s_share[8 * 64];  // first CTA: [rank][channel of the slice]
+// Global average pooling [N, HW, C] -> [N, C] (C % 8 == 0), a 64-channel slice of
+// an image at a time.  Lane l of warp w sums pixels 4 w + l / 8 + 32 k of the 8
+// channels 8 (l % 8) .. + 7; the partial sums of a channel meet by shuffles and in
+// shared memory, and threads 0..63 finish one channel each (avgpool_finish): the
+// mean, its bf16 value and the output occupancy (atomics into the cleared block:
+// row bit, column, tile and total counts, block-column mask words).
+//   avgpool_kernel       a CTA per slice: many slices or small maps, few registers
+//                        so that eight CTAs share an SM ([128,7,7,1280] 5.0 us)
+//   avgpool_deep_kernel  slices that leave the SMs room: a cluster of 1 to 8 CTAs
+//                        per slice, rank r starting 32 r pixels on and stepping 32
+//                        S, eight loads in flight a lane; the ranks' sums meet in
+//                        the first CTA's shared memory, in rank order
+//                        ([32,56,56,64] @P1@; [32,56,56,320] @P2@ us)
+__device__ __forceinline__ void avgpool_add(float (&a8)[8], const uint4& u) {
+  float f[8];
+  unpack8(u, f);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) a8[j] += f[j];
+}
+
+// This CTA's pixel sums into s_part[warp][channel of the slice].
+__device__ __forceinline__ void avgpool_meet(float (&a8)[8], float* s_part) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int cg = lane & 7, pq = warp * 4 + (lane >> 3);  // channel group, pixel lane 0..31
-  const int ctn = (C + 63) / 64;
-  const int slice = (int)blockIdx.x / S, rank = (int)blockIdx.x - slice * S;
-  const int n = slice / ctn, ct = slice - n * ctn;
-  const int c0 = ct * 64 + cg * 8;
-  if (S > 1) cluster_arrive();  // (waited for below: every CTA of the cluster has started)
-  pdl_wait();
-  pdl_trigger();
-  float a8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if (c0 < C) {
-    const __nv_bfloat16* p = x + (int64_t)n * HW * C + c0;
-    const int step = 32 * S;
-    for (int q = 32 * rank + pq; q < HW; q += 4 * step) {
-      uint4 u[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        u[i] = q + i * step < HW ? __ldg(reinterpret_cast<const uint4*>(p + (int64_t)(q + i * step) * C))
-                                 : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        float f[8];
-        unpack8(u[i], f);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) a8[j] += f[j];
-      }
-    }
-  }
   // lanes cg, cg + 8, cg + 16, cg + 24 of a warp hold the same channels
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -1213,41 +1193,107 @@ __global__ void __launch_bounds__(kTileThreads)
     for (int j = 0; j < 8; ++j) s_part[warp * 64 + lane * 8 + j] = a8[j];
   }
   __syncthreads();
+}
+
+// Threads 0..63 (two full warps): channel ct * 64 + threadIdx.x of image n, its sum over the pixels.
+__device__ __forceinline__ void avgpool_finish(float sum, int n, int ct, int HW, int C, __nv_bfloat16* y,
+                                               const OccDev& o, int emit) {
+  const int lane = threadIdx.x & 31;
+  const int c = ct * 64 + (int)threadIdx.x;
+  const __nv_bfloat16 b = __float2bfloat16_rn(sum / (float)HW);
+  const bool live = c < C;
+  if (live) y[(int64_t)n * C + c] = b;
+  const bool nz = live && (__bfloat16_as_ushort(b) & 0x7FFFu) != 0u;
+  if (emit) {
+    const uint32_t word = __ballot_sync(0xffffffffu, nz);  // this warp's 32 columns
+    if (nz) atomicAdd(&o.col_nnz[c], 1u);
+    if (lane == 0 && word) {
+      const int w = ct * 2 + (int)(threadIdx.x >> 5);
+      if (w < o.C32) atomicOr(&o.blk_mask[(int64_t)(n >> 7) * o.C32 + w], word);
+      atomicAdd(&o.tile_nnz[ct], (uint32_t)__popc(word));
+      atomicAdd(o.nnz, (unsigned long long)__popc(word));
+      atomicOr(&o.row_bm[(int64_t)n * o.W64 + (ct >> 6)], 1ull << (ct & 63));
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kTileThreads)
+    avgpool_kernel(const __nv_bfloat16* __restrict__ x, int N, int HW, int C,
+                   __nv_bfloat16* __restrict__ y, OccDev o_param, int emit) {
+  const OccDev o = o_param;
+  __shared__ float s_part[8 * 64];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int cg = lane & 7, pq = warp * 4 + (lane >> 3);  // channel group, pixel lane 0..31
+  const int ctn = (C + 63) / 64;
+  const int n = (int)(blockIdx.x / ctn), ct = (int)(blockIdx.x - (blockIdx.x / ctn) * ctn);
+  const int c0 = ct * 64 + cg * 8;
+  pdl_wait();
+  pdl_trigger();
+  float a8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  if (c0 < C) {
+    const __nv_bfloat16* p = x + (int64_t)n * HW * C + c0;
+    for (int q = pq; q < HW; q += 32) avgpool_add(a8, __ldg(reinterpret_cast<const uint4*>(p + (int64_t)q * C)));
+  }
+  avgpool_meet(a8, s_part);
+  if (threadIdx.x < 64) {
+    float sum = 0.f;
+#pragma unroll
+    for (int w = 0; w < kTileThreads / 32; ++w) sum += s_part[w * 64 + threadIdx.x];
+    avgpool_finish(sum, n, ct, HW, C, y, o, emit);
+  }
+}
+
+constexpr int kDeepCtas = 3;  // avgpool_deep_kernel CTAs an SM holds
+
+__global__ void __launch_bounds__(kTileThreads, kDeepCtas)
+    avgpool_deep_kernel(const __nv_bfloat16* __restrict__ x, int N, int HW, int C,
+                        __nv_bfloat16* __restrict__ y, OccDev o_param, int emit, int S) {
+  const OccDev o = o_param;
+  __shared__ float s_part[8 * 64];
+  __shared__ float s_share[8 * 64];  // first CTA: [rank][channel of the slice]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int cg = lane & 7, pq = warp * 4 + (lane >> 3);
+  const int ctn = (C + 63) / 64;
+  const int slice = (int)blockIdx.x / S, rank = (int)blockIdx.x - slice * S;
+  const int n = slice / ctn, ct = slice - n * ctn;
+  const int c0 = ct * 64 + cg * 8;
+  if (S > 1) cluster_arrive();  // (waited for below: every CTA of the cluster has started)
+  pdl_wait();
+  pdl_trigger();
+  float a8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  if (c0 < C) {
+    const __nv_bfloat16* p = x + (int64_t)n * HW * C + c0;
+    const int step = 32 * S;
+    int q = 32 * rank + pq;
+    for (; q < HW - 7 * step; q += 8 * step) {
+      uint4 u[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) u[i] = __ldg(reinterpret_cast<const uint4*>(p + (int64_t)(q + i * step) * C));
+#pragma unroll
+      for (int i = 0; i < 8; ++i) avgpool_add(a8, u[i]);
+    }
+#pragma unroll 4
+    for (; q < HW; q += step) avgpool_add(a8, __ldg(reinterpret_cast<const uint4*>(p + (int64_t)q * C)));
+  }
+  avgpool_meet(a8, s_part);
+  float sum = 0.f;
+  if (threadIdx.x < 64) {
+#pragma unroll
+    for (int w = 0; w < kTileThreads / 32; ++w) sum += s_part[w * 64 + threadIdx.x];
+  }
   if (S > 1) {
     cluster_wait();
-    if (threadIdx.x < 64) {
-      float sum = 0.f;
-#pragma unroll
-      for (int w = 0; w < kTileThreads / 32; ++w) sum += s_part[w * 64 + threadIdx.x];
-      st_cluster_f32(cluster_map(smem_u32(s_share + rank * 64 + threadIdx.x), 0u), sum);
-    }
+    if (threadIdx.x < 64) st_cluster_f32(cluster_map(smem_u32(s_share + rank * 64 + threadIdx.x), 0u), sum);
     __syncwarp();
     cluster_arrive();
     cluster_wait();
     if (rank != 0) return;
-  }
-  if (threadIdx.x < 64) {  // two full warps
-    const int c = ct * 64 + (int)threadIdx.x;
-    const float* part = S > 1 ? s_share : s_part;
-    const int parts = S > 1 ? S : kTileThreads / 32;
-    float sum = 0.f;
-    for (int w = 0; w < parts; ++w) sum += part[w * 64 + threadIdx.x];
-    const __nv_bfloat16 b = __float2bfloat16_rn(sum / (float)HW);
-    const bool live = c < C;
-    if (live) y[(int64_t)n * C + c] = b;
-    const bool nz = live && (__bfloat16_as_ushort(b) & 0x7FFFu) != 0u;
-    if (emit) {
-      const uint32_t word = __ballot_sync(0xffffffffu, nz);  // this warp's 32 columns
-      if (nz) atomicAdd(&o.col_nnz[c], 1u);
-      if (lane == 0 && word) {
-        const int w = ct * 2 + (int)(threadIdx.x >> 5);
-        if (w < o.C32) atomicOr(&o.blk_mask[(int64_t)(n >> 7) * o.C32 + w], word);
-        atomicAdd(&o.tile_nnz[ct], (uint32_t)__popc(word));
-        atomicAdd(o.nnz, (unsigned long long)__popc(word));
-        atomicOr(&o.row_bm[(int64_t)n * o.W64 + (ct >> 6)], 1ull << (ct & 63));
-      }
+    if (threadIdx.x < 64) {
+      sum = 0.f;
+      for (int k = 0; k < S; ++k) sum += s_share[k * 64 + threadIdx.x];
     }
   }
+  if (threadIdx.x < 64) avgpool_finish(sum, n, ct, HW, C, y, o, emit);
 }
 
 // Dynamic shared memory of a tile kernel: the per-CTA column counters.
@@ -1424,14 +1470,16 @@ cudaError_t launch_avgpool(const __nv_bfloat16* x, int N, int HW, int C, __nv_bf
   if (C % 8) return cudaErrorInvalidValue;
   const int64_t ctas = (int64_t)N * ((C + 63) / 64);
   if (ctas >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
-  // CTAs per slice: while two per SM are not reached and each keeps 64 pixels
-  // (two rounds of its pixel lanes; 7x7 maps stay whole)
+  if (HW < 128 || ctas > kDeepCtas * device_sm_count())
+    return launch_kernel(avgpool_kernel, dim3((unsigned)ctas), dim3(kTileThreads), 0, s, x, N, HW, C, y, o, emit);
+  // CTAs per slice: while two per SM are not reached and each keeps 128 pixels
+  // (14x14 maps stay whole: 2.1 us, 2.3 by two)
   int S = 1;
-  while (S < 8 && ctas * S * 2 <= 2 * device_sm_count() && HW >= 64 * S * 2) S *= 2;
+  while (S < 8 && ctas * S * 2 <= 2 * device_sm_count() && HW >= 128 * S * 2) S *= 2;
   if (S == 1)
-    return launch_kernel(avgpool_kernel, dim3((unsigned)ctas), dim3(kTileThreads), 0, s, x, N, HW, C, y, o, emit, 1);
-  return launch_cluster_kernel(avgpool_kernel, dim3((unsigned)(ctas * S)), dim3(kTileThreads), (unsigned)S, 0, s, x, N,
-                               HW, C, y, o, emit, S);
+    return launch_kernel(avgpool_deep_kernel, dim3((unsigned)ctas), dim3(kTileThreads), 0, s, x, N, HW, C, y, o, emit, 1);
+  return launch_cluster_kernel(avgpool_deep_kernel, dim3((unsigned)(ctas * S)), dim3(kTileThreads), (unsigned)S, 0, s, x,
+                               N, HW, C, y, o, emit, S);
 }
 
 cudaError_t launch_bn_act(const __nv_bfloat16* x, int64_t R, int C, const EpiDev& ep,
