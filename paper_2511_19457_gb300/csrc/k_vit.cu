@@ -43,7 +43,7 @@ __device__ __forceinline__ void ln_store(__nv_bfloat16* __restrict__ yr, const f
 }
 
 template <int NCH>
-__global__ void __launch_bounds__(kLnThreads, 1)
+__global__ void __launch_bounds__(kLnThreads, NCH == 1 ? 2 : 1)
     ln_rows_kernel(const __nv_bfloat16* __restrict__ x, int64_t R, int C, const float* __restrict__ gb, int gb_vec,
                    float eps, __nv_bfloat16* __restrict__ y, OccDev o_param, int emit) {
   const OccDev o = o_param;
@@ -222,30 +222,50 @@ __global__ void __launch_bounds__(kVitThreads) layernorm_kernel(const __nv_bfloa
   for (int64_t r = (int64_t)blockIdx.x * (kVitThreads / 32) + (threadIdx.x >> 5); r < R; r += warps) {
     const __nv_bfloat16* xr = x + r * C;
     __nv_bfloat16* yr = y + r * C;
-    float s = 0.f;
-    for (int c = lane; c < chunks; c += 32) {
-      float f[8];
-      unpack8(*reinterpret_cast<const uint4*>(xr + c * 8), f);
+    uint4 u[4];
+    auto load4 = [&](int c) {  // chunks c, c + 32, ...: four loads in flight, to the row's end
 #pragma unroll
-      for (int k = 0; k < 8; ++k) s += f[k];
+      for (int i = 0; i < 4; ++i)
+        u[i] = c + 32 * i < chunks ? *reinterpret_cast<const uint4*>(xr + (c + 32 * i) * 8) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    float s = 0.f;
+    for (int c = lane; c < chunks; c += 128) {
+      load4(c);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        float f[8];
+        unpack8(u[i], f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += f[k];
+      }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     const float mean = s * inv_c;
     float q = 0.f;
-    for (int c = lane; c < chunks; c += 32) {
-      float f[8];
-      unpack8(*reinterpret_cast<const uint4*>(xr + c * 8), f);
+    for (int c = lane; c < chunks; c += 128) {
+      load4(c);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) q = fmaf(f[k] - mean, f[k] - mean, q);
+      for (int i = 0; i < 4; ++i) {
+        if (c + 32 * i >= chunks) break;
+        float f[8];
+        unpack8(u[i], f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) q = fmaf(f[k] - mean, f[k] - mean, q);
+      }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
     const float rstd = rsqrtf(q * inv_c + eps);
-    for (int c = lane; c < chunks; c += 32) {
-      float f[8];
-      unpack8(*reinterpret_cast<const uint4*>(xr + c * 8), f);
-      ln_store(yr, gb, C, c, f, mean, rstd);
+    for (int c = lane; c < chunks; c += 128) {
+      load4(c);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (c + 32 * i >= chunks) break;
+        float f[8];
+        unpack8(u[i], f);
+        ln_store(yr, gb, C, c + 32 * i, f, mean, rstd);
+      }
     }
   }
 }
@@ -334,16 +354,19 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   const int n = blockIdx.x / heads, h = blockIdx.x - (blockIdx.x / heads) * heads;
   const int D = heads * HD, row3 = 3 * D;
   const __nv_bfloat16* base = qkv + (int64_t)n * T * row3;
-  if (threadIdx.x < HD) s_cnt[threadIdx.x] = 0u;
+  for (int c = threadIdx.x; c < HD; c += blockDim.x) s_cnt[c] = 0u;
   pdl_wait();
   pdl_trigger();
-  // K and V rows of the head: 16-byte copies, all in flight at once
-  for (int idx = threadIdx.x; idx < T16 * (HD / 8); idx += kAttnThreads) {
-    const int t = idx / (HD / 8), c = idx - (idx / (HD / 8)) * (HD / 8);
-    const bool live = t < T;
-    const __nv_bfloat16* src = base + (int64_t)(live ? t : 0) * row3 + h * HD + c * 8;
-    cp_async_16(smem_u32(sK + t * KP + c * 8), src + D, live ? 16u : 0u);
-    cp_async_16(smem_u32(sV + t * KP + c * 8), src + 2 * D, live ? 16u : 0u);
+  // K and V rows of the head: 16-byte copies, all in flight at once; a thread
+  // takes the same chunk of every (threads / chunks)-th row
+  {
+    const int c = (int)threadIdx.x % (HD / 8), step = (int)blockDim.x / (HD / 8);
+    for (int t = (int)threadIdx.x / (HD / 8); t < T16; t += step) {
+      const bool live = t < T;
+      const __nv_bfloat16* src = base + (int64_t)(live ? t : 0) * row3 + h * HD + c * 8;
+      cp_async_16(smem_u32(sK + t * KP + c * 8), src + D, live ? 16u : 0u);
+      cp_async_16(smem_u32(sV + t * KP + c * 8), src + 2 * D, live ? 16u : 0u);
+    }
   }
   cp_async_commit();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -378,7 +401,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   // K fragments of 8 keys: matrices (dims 0-7, 8-15) of one k-step, then of the next
   const uint32_t k_lane = smem_u32(sK) + (uint32_t)(((lane & 7) * KP + (lane >> 3) * 8) * 2);
   uint32_t cnt = 0u;  // byte i: non-zeros of column 8 (lane & 7) + 2 i + (lane >> 4) in the rows of half (lane >> 3) & 1
-  for (int qt = qt0; qt < qt_end; qt += kAttnWarps) {
+  for (int qt = qt0; qt < qt_end; qt += (int)blockDim.x / 32) {
     const int q0 = qt * 16;
     if (qt != qt0) load_q(q0);
     float o[HD / 8][4];
@@ -559,9 +582,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     }
   }
   __syncthreads();
-  if (threadIdx.x < 64) {  // (HD columns: whole warps, or half of one)
-    const uint32_t v = threadIdx.x < HD ? s_cnt[threadIdx.x] : 0u;
-    if (v) atomicAdd(&occ.col_nnz[h * HD + threadIdx.x], v);
+  for (int c0 = warp * 32; c0 < HD; c0 += blockDim.x) {  // (HD columns: whole warps, or half of one)
+    const int c = c0 + lane;
+    const uint32_t v = c < HD ? s_cnt[c] : 0u;
+    if (v) atomicAdd(&occ.col_nnz[h * HD + c], v);
     const uint32_t sum = __reduce_add_sync(0xffffffffu, v);
     if (lane == 0 && sum) {
       atomicAdd(&occ.tile_nnz[(h * HD) >> 6], sum);
@@ -629,6 +653,38 @@ size_t attention_smem(int T, int hd) {
 
 namespace {
 
+// Warps of a CTA and CTAs of a head, for `pairs` (image, head) pairs.
+//   - Pairs that fill the SMs twice: one CTA a head, which stages its K and V
+//     once, a tile per warp up to 7, then over at most 5 warps (7 beyond 15
+//     tiles).  With CTAs of 7 warps and a tile per warp throughout the warps
+//     without a tile, and a second copy of K and V, cost more than the fuller
+//     SMs gave.  Where one CTA a head leaves the last round mostly empty (some
+//     hundred pairs of more than 15 tiles, two CTAs an SM), a tile per warp.
+//   - Fewer pairs: a tile per warp, and up to a CTA per SM, of two tiles or more;
+//     three a head while two an SM hold them.  Warps without a tile stage.
+// Times (with occupancy) of this rule against CTAs of 7 warps, a tile per warp:
+//   head dimension 64: @A@
+//   head dimension 32: @B@
+void attention_split(int64_t pairs, int T, size_t smem, int* warps, int* qsplit) {
+  const int64_t sms = device_sm_count();
+  const int tiles = (T + 15) / 16;
+  auto up = [](int a, int b) { return (a + b - 1) / b; };
+  const bool two = smem <= 110 * 1024;  // CTAs that fit an SM
+  int q = up(tiles, kAttnWarps);
+  if (pairs >= 2 * sms) {
+    if (tiles <= 15 || pairs >= 8 * sms || !two) q = 1;
+    const int per = up(tiles, q), wmax = per > kAttnWarps && per <= 15 ? 5 : kAttnWarps;
+    *warps = up(per, up(per, wmax));
+  } else {
+    const int64_t fill = sms / pairs;
+    if (fill > q) q = (int)(fill < up(tiles, 2) ? fill : up(tiles, 2));
+    if (q < 3 && tiles >= 8 && 3 * pairs <= 2 * sms) q = 3;
+    q = up(tiles, up(tiles, q));
+    *warps = kAttnWarps;
+  }
+  *qsplit = q;
+}
+
 template <int HD>
 cudaError_t launch_attention_hd(const __nv_bfloat16* qkv, int N, int T, int heads, __nv_bfloat16* y,
                                 const OccDev& o, int emit, cudaStream_t s) {
@@ -637,9 +693,9 @@ cudaError_t launch_attention_hd(const __nv_bfloat16* qkv, int N, int T, int head
     cudaError_t e = smem_optin(reinterpret_cast<const void*>(attention_kernel<HD>), smem);
     if (e != cudaSuccess) return e;
   }
-  // a query tile per warp
-  const int qsplit = ((T + 15) / 16 + kAttnWarps - 1) / kAttnWarps;
-  return launch_kernel(attention_kernel<HD>, dim3((unsigned)(N * heads), (unsigned)qsplit), dim3(kAttnThreads), smem, s,
+  int warps, qsplit;
+  attention_split((int64_t)N * heads, T, smem, &warps, &qsplit);
+  return launch_kernel(attention_kernel<HD>, dim3((unsigned)(N * heads), (unsigned)qsplit), dim3(32u * warps), smem, s,
                        qkv, T, heads, y, o, emit);
 }
 
@@ -672,7 +728,7 @@ cudaError_t launch_layernorm(const __nv_bfloat16* x, int64_t R, int C, const flo
   // once they fill the SMs (fewer CTAs add their column counts up in global memory)
   const int threads = R >= 8 * (int64_t)device_sm_count() ? kLnThreads : 256;
   const int64_t ctas = (R + threads / 32 - 1) / (threads / 32);
-  const int64_t cap = (int64_t)device_sm_count();
+  const int64_t cap = (int64_t)device_sm_count() * (C <= 256 ? 2 : 1);
   const dim3 grid((unsigned)(ctas < cap ? ctas : cap));
   const int vec = (reinterpret_cast<uintptr_t>(gb) & 15u) == 0;  // (C % 8 == 0: beta's rows too)
   switch ((C + 255) / 256) {
