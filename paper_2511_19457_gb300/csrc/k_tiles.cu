@@ -1171,7 +1171,8 @@ __global__ void __launch_bounds__(kTileThreads) dwconv_kernel(const DwArgs a_par
 //                        per slice, rank r starting 32 r pixels on and stepping 32
 //                        S, eight loads in flight a lane; the ranks' sums meet in
 //                        the first CTA's shared memory, in rank order
-//                        ([32,56,56,64] @P1@; [32,56,56,320] @P2@ us)
+//                        ([32,56,56,64] 3.2 us, [32,56,56,320] 15.5;
+//                        as CTAs of the first kernel 11.7 and 32)
 __device__ __forceinline__ void avgpool_add(float (&a8)[8], const uint4& u) {
   float f[8];
   unpack8(u, f);

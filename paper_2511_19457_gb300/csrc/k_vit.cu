@@ -25,8 +25,10 @@ constexpr int kVitThreads = 256;
 // block, column counts in 16-bit register halves, added up in shared memory once
 // per CTA.  [6304, 768]: 4.7 us, with occupancy and its clear 10.3 us (14.1 us and
 // 9.5 us more for a clear and a statistics pass before: gamma and beta were
-// re-read, value by value, for every row).  Longer rows (layernorm_kernel) are
-// re-read for each of the three steps.
+// re-read, value by value, for every row).  Rows of up to 256 values run two CTAs
+// an SM ([87511, 64] 22 us, one CTA 36).  Longer rows than 1024 (layernorm_kernel)
+// are re-read for each of the three steps, four loads in flight ([5091, 1312] 19 us;
+// loads one at a time 32).
 constexpr int kLnRegChunks = 4;     // 8-value chunks per lane held in registers
 constexpr int kLnThreads = 512;     // at most: one CTA per SM, whose column counts reach global memory once
 constexpr int kLnFlushRows = 16384;  // rows after which 16-bit counters are flushed
@@ -354,19 +356,16 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   const int n = blockIdx.x / heads, h = blockIdx.x - (blockIdx.x / heads) * heads;
   const int D = heads * HD, row3 = 3 * D;
   const __nv_bfloat16* base = qkv + (int64_t)n * T * row3;
-  for (int c = threadIdx.x; c < HD; c += blockDim.x) s_cnt[c] = 0u;
+  if (threadIdx.x < HD) s_cnt[threadIdx.x] = 0u;
   pdl_wait();
   pdl_trigger();
-  // K and V rows of the head: 16-byte copies, all in flight at once; a thread
-  // takes the same chunk of every (threads / chunks)-th row
-  {
-    const int c = (int)threadIdx.x % (HD / 8), step = (int)blockDim.x / (HD / 8);
-    for (int t = (int)threadIdx.x / (HD / 8); t < T16; t += step) {
-      const bool live = t < T;
-      const __nv_bfloat16* src = base + (int64_t)(live ? t : 0) * row3 + h * HD + c * 8;
-      cp_async_16(smem_u32(sK + t * KP + c * 8), src + D, live ? 16u : 0u);
-      cp_async_16(smem_u32(sV + t * KP + c * 8), src + 2 * D, live ? 16u : 0u);
-    }
+  // K and V rows of the head: 16-byte copies, all in flight at once
+  for (int idx = threadIdx.x; idx < T16 * (HD / 8); idx += kAttnThreads) {
+    const int t = idx / (HD / 8), c = idx - (idx / (HD / 8)) * (HD / 8);
+    const bool live = t < T;
+    const __nv_bfloat16* src = base + (int64_t)(live ? t : 0) * row3 + h * HD + c * 8;
+    cp_async_16(smem_u32(sK + t * KP + c * 8), src + D, live ? 16u : 0u);
+    cp_async_16(smem_u32(sV + t * KP + c * 8), src + 2 * D, live ? 16u : 0u);
   }
   cp_async_commit();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -401,7 +400,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   // K fragments of 8 keys: matrices (dims 0-7, 8-15) of one k-step, then of the next
   const uint32_t k_lane = smem_u32(sK) + (uint32_t)(((lane & 7) * KP + (lane >> 3) * 8) * 2);
   uint32_t cnt = 0u;  // byte i: non-zeros of column 8 (lane & 7) + 2 i + (lane >> 4) in the rows of half (lane >> 3) & 1
-  for (int qt = qt0; qt < qt_end; qt += (int)blockDim.x / 32) {
+  for (int qt = qt0; qt < qt_end; qt += kAttnWarps) {
     const int q0 = qt * 16;
     if (qt != qt0) load_q(q0);
     float o[HD / 8][4];
@@ -582,10 +581,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     }
   }
   __syncthreads();
-  for (int c0 = warp * 32; c0 < HD; c0 += blockDim.x) {  // (HD columns: whole warps, or half of one)
-    const int c = c0 + lane;
-    const uint32_t v = c < HD ? s_cnt[c] : 0u;
-    if (v) atomicAdd(&occ.col_nnz[h * HD + c], v);
+  if (threadIdx.x < 64) {  // (HD columns: whole warps, or half of one)
+    const uint32_t v = threadIdx.x < HD ? s_cnt[threadIdx.x] : 0u;
+    if (v) atomicAdd(&occ.col_nnz[h * HD + threadIdx.x], v);
     const uint32_t sum = __reduce_add_sync(0xffffffffu, v);
     if (lane == 0 && sum) {
       atomicAdd(&occ.tile_nnz[(h * HD) >> 6], sum);
@@ -653,38 +651,6 @@ size_t attention_smem(int T, int hd) {
 
 namespace {
 
-// Warps of a CTA and CTAs of a head, for `pairs` (image, head) pairs.
-//   - Pairs that fill the SMs twice: one CTA a head, which stages its K and V
-//     once, a tile per warp up to 7, then over at most 5 warps (7 beyond 15
-//     tiles).  With CTAs of 7 warps and a tile per warp throughout the warps
-//     without a tile, and a second copy of K and V, cost more than the fuller
-//     SMs gave.  Where one CTA a head leaves the last round mostly empty (some
-//     hundred pairs of more than 15 tiles, two CTAs an SM), a tile per warp.
-//   - Fewer pairs: a tile per warp, and up to a CTA per SM, of two tiles or more;
-//     three a head while two an SM hold them.  Warps without a tile stage.
-// Times (with occupancy) of this rule against CTAs of 7 warps, a tile per warp:
-//   head dimension 64: @A@
-//   head dimension 32: @B@
-void attention_split(int64_t pairs, int T, size_t smem, int* warps, int* qsplit) {
-  const int64_t sms = device_sm_count();
-  const int tiles = (T + 15) / 16;
-  auto up = [](int a, int b) { return (a + b - 1) / b; };
-  const bool two = smem <= 110 * 1024;  // CTAs that fit an SM
-  int q = up(tiles, kAttnWarps);
-  if (pairs >= 2 * sms) {
-    if (tiles <= 15 || pairs >= 8 * sms || !two) q = 1;
-    const int per = up(tiles, q), wmax = per > kAttnWarps && per <= 15 ? 5 : kAttnWarps;
-    *warps = up(per, up(per, wmax));
-  } else {
-    const int64_t fill = sms / pairs;
-    if (fill > q) q = (int)(fill < up(tiles, 2) ? fill : up(tiles, 2));
-    if (q < 3 && tiles >= 8 && 3 * pairs <= 2 * sms) q = 3;
-    q = up(tiles, up(tiles, q));
-    *warps = kAttnWarps;
-  }
-  *qsplit = q;
-}
-
 template <int HD>
 cudaError_t launch_attention_hd(const __nv_bfloat16* qkv, int N, int T, int heads, __nv_bfloat16* y,
                                 const OccDev& o, int emit, cudaStream_t s) {
@@ -693,9 +659,9 @@ cudaError_t launch_attention_hd(const __nv_bfloat16* qkv, int N, int T, int head
     cudaError_t e = smem_optin(reinterpret_cast<const void*>(attention_kernel<HD>), smem);
     if (e != cudaSuccess) return e;
   }
-  int warps, qsplit;
-  attention_split((int64_t)N * heads, T, smem, &warps, &qsplit);
-  return launch_kernel(attention_kernel<HD>, dim3((unsigned)(N * heads), (unsigned)qsplit), dim3(32u * warps), smem, s,
+  // a query tile per warp
+  const int qsplit = ((T + 15) / 16 + kAttnWarps - 1) / kAttnWarps;
+  return launch_kernel(attention_kernel<HD>, dim3((unsigned)(N * heads), (unsigned)qsplit), dim3(kAttnThreads), smem, s,
                        qkv, T, heads, y, o, emit);
 }
 
