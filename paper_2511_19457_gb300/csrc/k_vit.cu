@@ -275,13 +275,12 @@ __global__ void __launch_bounds__(kVitThreads) layernorm_kernel(const __nv_bfloa
 // ---------------------------------------------------------------------------
 // Multi-head self-attention on the tensor cores (mma.sync m16n8k16, bf16 in,
 // fp32 accumulate), flash-attention style.  Input rows (one per token) hold
-// q | k | v, each heads x HD values.  A CTA of 7 warps takes 7 16-query tiles of
-// one (image, head): the head's K and V rows are copied once into shared memory
-// by cp.async (row pitch HD + 8 elements, so the 8 rows of a fragment load fall
-// in distinct banks; rows past T up to the next multiple of 16 zero-filled),
-// then every warp does its tile.  (One CTA of 4 warps per (image, head), each
-// warp three or four tiles in turn, left 12 warps per SM and a last round half
-// empty: [32,197,12x64] 34 us.)  A warp walks the keys in blocks of 32: S = Q K^T
+// q | k | v, each heads x HD values.  A CTA of up to 7 warps takes some of the
+// 16-query tiles of one (image, head) (attention_split): the head's K and V rows
+// are copied once into shared memory by cp.async (row pitch HD + 8 elements, so
+// the 8 rows of a fragment load fall in distinct banks; rows past T up to the next
+// multiple of 16 zero-filled), then the warps take the tiles in turn, at most five
+// each.  A warp walks the keys in blocks of 32: S = Q K^T
 // (Q fragments in registers, K fragments by ldmatrix), an online softmax per
 // query row (running maximum and sum, rescaling the output), and O += P V with P
 // taken straight from the S accumulators (their layout is the A-operand layout
@@ -295,11 +294,10 @@ __global__ void __launch_bounds__(kVitThreads) layernorm_kernel(const __nv_bfloa
 // exponentials.  So a whole block of keys has no branches (the ones around each 8
 // keys kept the MMAs of different keys from overlapping) and the first queries
 // are loaded beside K and V.  Blocks of 32 keys rather than 64 fit 128 registers.
-// [32,197,12x64] without / with occupancy 28.9 / 34.7 -> 21.9 / 25.7 us (64-key
-// blocks 24.4 / 31.3), [8,512,12x64] 48.8 / 54.4 -> 33.6 / 36.9 us; the occupancy
-// took 64-bit masks by shuffles and 16 counters a lane before.
+// (64-key blocks, with branches, occupancy by 64-bit masks and 16 counters a lane:
+// [32,197,12x64] with occupancy 39 us, now 28; [8,512,12x64] 76 us, now 42.)
 constexpr int kAttnWarps = 7;
-constexpr int kAttnThreads = 32 * kAttnWarps;
+constexpr int kAttnThreads = 32 * kAttnWarps;  // at most
 constexpr int kAttnMaxT = 512;
 constexpr int kAttnKB = 32;        // keys per block
 
@@ -356,16 +354,19 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   const int n = blockIdx.x / heads, h = blockIdx.x - (blockIdx.x / heads) * heads;
   const int D = heads * HD, row3 = 3 * D;
   const __nv_bfloat16* base = qkv + (int64_t)n * T * row3;
-  if (threadIdx.x < HD) s_cnt[threadIdx.x] = 0u;
+  for (int c = threadIdx.x; c < HD; c += blockDim.x) s_cnt[c] = 0u;
   pdl_wait();
   pdl_trigger();
-  // K and V rows of the head: 16-byte copies, all in flight at once
-  for (int idx = threadIdx.x; idx < T16 * (HD / 8); idx += kAttnThreads) {
-    const int t = idx / (HD / 8), c = idx - (idx / (HD / 8)) * (HD / 8);
-    const bool live = t < T;
-    const __nv_bfloat16* src = base + (int64_t)(live ? t : 0) * row3 + h * HD + c * 8;
-    cp_async_16(smem_u32(sK + t * KP + c * 8), src + D, live ? 16u : 0u);
-    cp_async_16(smem_u32(sV + t * KP + c * 8), src + 2 * D, live ? 16u : 0u);
+  // K and V rows of the head: 16-byte copies, all in flight at once; a thread
+  // takes the same chunk of every (threads / chunks)-th row
+  {
+    const int c = (int)threadIdx.x % (HD / 8), step = (int)blockDim.x / (HD / 8);
+    for (int t = (int)threadIdx.x / (HD / 8); t < T16; t += step) {
+      const bool live = t < T;
+      const __nv_bfloat16* src = base + (int64_t)(live ? t : 0) * row3 + h * HD + c * 8;
+      cp_async_16(smem_u32(sK + t * KP + c * 8), src + D, live ? 16u : 0u);
+      cp_async_16(smem_u32(sV + t * KP + c * 8), src + 2 * D, live ? 16u : 0u);
+    }
   }
   cp_async_commit();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -400,7 +401,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   // K fragments of 8 keys: matrices (dims 0-7, 8-15) of one k-step, then of the next
   const uint32_t k_lane = smem_u32(sK) + (uint32_t)(((lane & 7) * KP + (lane >> 3) * 8) * 2);
   uint32_t cnt = 0u;  // byte i: non-zeros of column 8 (lane & 7) + 2 i + (lane >> 4) in the rows of half (lane >> 3) & 1
-  for (int qt = qt0; qt < qt_end; qt += kAttnWarps) {
+  for (int qt = qt0; qt < qt_end; qt += (int)blockDim.x / 32) {
     const int q0 = qt * 16;
     if (qt != qt0) load_q(q0);
     float o[HD / 8][4];
@@ -581,9 +582,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     }
   }
   __syncthreads();
-  if (threadIdx.x < 64) {  // (HD columns: whole warps, or half of one)
-    const uint32_t v = threadIdx.x < HD ? s_cnt[threadIdx.x] : 0u;
-    if (v) atomicAdd(&occ.col_nnz[h * HD + threadIdx.x], v);
+  for (int c0 = warp * 32; c0 < HD; c0 += blockDim.x) {  // (HD columns: whole warps, or half of one)
+    const int c = c0 + lane;
+    const uint32_t v = c < HD ? s_cnt[c] : 0u;
+    if (v) atomicAdd(&occ.col_nnz[h * HD + c], v);
     const uint32_t sum = __reduce_add_sync(0xffffffffu, v);
     if (lane == 0 && sum) {
       atomicAdd(&occ.tile_nnz[(h * HD) >> 6], sum);
@@ -651,6 +653,41 @@ size_t attention_smem(int T, int hd) {
 
 namespace {
 
+// Warps of a CTA and CTAs of a head, for `pairs` (image, head) pairs.
+//   - Pairs that fill the SMs twice: one CTA a head, which stages its K and V
+//     once, a tile per warp up to 7, then over at most 5 warps (7 beyond 15
+//     tiles).  With CTAs of 7 warps and a tile per warp throughout the warps
+//     without a tile, and a second copy of K and V, cost more than the fuller
+//     SMs gave.  Where one CTA a head leaves the last round mostly empty (some
+//     hundred pairs of more than 15 tiles, two CTAs an SM), a tile per warp.
+//   - Fewer pairs: a tile per warp, and up to a CTA per SM, of two tiles or more;
+//     three a head while two an SM hold them.  Warps without a tile stage.
+// Times with occupancy, us: CTAs of 7 warps with a tile per warp / this rule:
+//   pairs, dimension  T = 16       64         128        197        257       512
+//   12, 64           3.4 / 3.5  4.0 / 3.9  4.9 / 4.8  7.3 / 6.0  8.3 / 6.9  12 / 9.7
+//   384, 64          5.7 / 4.4  7.8 / 6.5   17 / 13    30 / 28    42 / 42  145 / 138
+//   1536, 64          14 / 7.0   24 / 20    54 / 40    89 / 87   147 / 137
+//   1536, 32          13 / 5.4   18 / 14    42 / 28    67 / 61   107 / 97  267 / 254
+void attention_split(int64_t pairs, int T, size_t smem, int* warps, int* qsplit) {
+  const int64_t sms = device_sm_count();
+  const int tiles = (T + 15) / 16;
+  auto up = [](int a, int b) { return (a + b - 1) / b; };
+  const bool two = smem <= 110 * 1024;  // CTAs that fit an SM
+  int q = up(tiles, kAttnWarps);
+  if (pairs >= 2 * sms) {
+    if (tiles <= 15 || pairs >= 8 * sms || !two) q = 1;
+    const int per = up(tiles, q), wmax = per > kAttnWarps && per <= 15 ? 5 : kAttnWarps;
+    *warps = up(per, up(per, wmax));
+  } else {
+    const int64_t fill = sms / pairs;
+    if (fill > q) q = (int)(fill < up(tiles, 2) ? fill : up(tiles, 2));
+    if (q < 3 && tiles >= 8 && 3 * pairs <= 2 * sms) q = 3;
+    q = up(tiles, up(tiles, q));
+    *warps = kAttnWarps;
+  }
+  *qsplit = q;
+}
+
 template <int HD>
 cudaError_t launch_attention_hd(const __nv_bfloat16* qkv, int N, int T, int heads, __nv_bfloat16* y,
                                 const OccDev& o, int emit, cudaStream_t s) {
@@ -659,9 +696,9 @@ cudaError_t launch_attention_hd(const __nv_bfloat16* qkv, int N, int T, int head
     cudaError_t e = smem_optin(reinterpret_cast<const void*>(attention_kernel<HD>), smem);
     if (e != cudaSuccess) return e;
   }
-  // a query tile per warp
-  const int qsplit = ((T + 15) / 16 + kAttnWarps - 1) / kAttnWarps;
-  return launch_kernel(attention_kernel<HD>, dim3((unsigned)(N * heads), (unsigned)qsplit), dim3(kAttnThreads), smem, s,
+  int warps, qsplit;
+  attention_split((int64_t)N * heads, T, smem, &warps, &qsplit);
+  return launch_kernel(attention_kernel<HD>, dim3((unsigned)(N * heads), (unsigned)qsplit), dim3(32u * warps), smem, s,
                        qkv, T, heads, y, o, emit);
 }
 
