@@ -168,3 +168,43 @@ def test_attention_weights_below_the_normal_range(sp, ctx, far):
     assert want[0, 0] > 0.09
     assert np.abs(got[:, 0] / want[:, 0] - 1).max() <= 0.021 + 2.0 ** -9
     assert not got[:, 1:].any()
+
+
+@pytest.mark.parametrize("N,T,heads,hd", [(40, 17, 12, 64), (26, 64, 12, 16), (52, 100, 8, 32), (40, 129, 12, 16),
+                                          (32, 225, 12, 16), (32, 300, 12, 16), (102, 300, 12, 16), (13, 500, 24, 64),
+                                          (1, 500, 2, 64), (20, 48, 12, 32), (16, 385, 12, 32)])
+def test_attention_splits(sp, ctx, N, T, heads, hd):
+    """Every way a head's query tiles are shared out: a tile per warp, several in
+    turn, one CTA a head and many, tiles that do not come out even."""
+    D = heads * hd
+    qb = _bits((N, T, 3 * D), T + N, 0.0)
+    qb.reshape(N, T, 3 * D)[:, :, 2 * D: 2 * D + 5] = 0
+    y = torch.full((N, T, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+    yo = sp.OccupancyBuffer(N * T, D)
+    yo.buf.fill_(0x11)
+    sp.sparoa_attention(ctx, sp.bits_to_device(qb).view(N, T, 3 * D), y, heads, y_occ=yo)
+    assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), N * T, D), "attention")
+    assert_close(y.float().cpu().numpy(), orc.attention(qb, N, T, heads, hd), what=f"attention {N} {T} {heads} {hd}")
+
+
+@pytest.mark.parametrize("R,C", [(1500, 1312), (3, 2056), (700, 4104), (40000, 8), (9000, 256)])
+def test_layernorm_row_lengths(sp, ctx, R, C):
+    xb = _bits((R, C), R + C)
+    y = torch.full((R, C), float("nan"), dtype=torch.bfloat16, device="cuda")
+    yo = sp.OccupancyBuffer(R, C)
+    yo.buf.fill_(0x77)
+    sp.sparoa_layernorm(ctx, sp.bits_to_device(xb).view(R, C), y, y_occ=yo)
+    assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), R, C), f"layernorm {R}x{C}")
+    assert_close(y.float().cpu().numpy(), orc.layernorm(xb, R, C, None, 1e-6), what=f"layernorm {R}x{C}")
+
+
+@pytest.mark.parametrize("N,H,W,C", [(8, 14, 14, 4096), (7, 8, 16, 64), (40, 16, 16, 264), (2, 300, 9, 8), (70, 9, 29, 64)])
+def test_avgpool_kernels(sp, ctx, N, H, W, C):
+    """Plain (many slices, small maps) and deep kernels around their lines, eight
+    loads a round with remainders."""
+    xb = _bits((N, H, W, C), H + C)
+    y = torch.empty(N, C, dtype=torch.bfloat16, device="cuda")
+    yo = sp.OccupancyBuffer(N, C)
+    sp.sparoa_avgpool_global(ctx, sp.bits_to_device(xb).view(N, H, W, C), y, y_occ=yo)
+    assert_close(y.float().cpu().numpy(), orc.avgpool_global(xb, N, H, W, C), what="avgpool")
+    assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), N, C), "avgpool")
