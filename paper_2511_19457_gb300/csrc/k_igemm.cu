@@ -324,9 +324,6 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
   uint32_t* s_acc = reinterpret_cast<uint32_t*>(smem + C::kAccOff);  // [N] non-zeros per column
   unsigned long long* s_rowbm = reinterpret_cast<unsigned long long*>(smem + C::kRowOff);
   uint32_t* s_blk = reinterpret_cast<uint32_t*>(smem + C::kBlkOff);
-  // Column counts of all tiles a CTA handles are summed here and flushed once
-  // (atomics on one address from every tile would serialise in L2).
-  const bool acc_smem = emit && p.N <= kMaxAccCols;
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -341,10 +338,18 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
   const int units = tiles * KS;
   // Lean epilogue: with four accumulators the 4 warps of a TMEM lane quarter
   // take every 4th tile each; with two (192- and 256-wide tiles), and where the
-  // CTA has one tile, they share a tile's 32-column blocks.  ncw: warps that
-  // share a quarter of a tile.
+  // CTA has one tile (up to two of more than 64 columns), they share a tile's
+  // 32-column blocks.  ncw: warps that share a quarter of a tile.
   constexpr int kQw = Wp::kEpi / 4;  // epilogue warps per lane quarter
-  const int ncw = kAcc == 2 || units <= (int)gridDim.x ? kQw : 1;
+  const int ncw = kAcc == 2 || units <= (BN > 64 ? 2 : 1) * (int)gridDim.x ? kQw : 1;
+  // every tile of the CTA has the same columns
+  const bool fixed_cols = nt == 1 || (int)gridDim.x % nt == 0 || units <= (int)gridDim.x;
+  // Column counts of all tiles a CTA handles are summed in shared memory and
+  // flushed once (atomics on one address from every tile would serialise in L2);
+  // a lean CTA's only tile adds its columns' counts directly (shorter code, which
+  // it runs once: 128 x 64 values with K = 64 6.9 -> 6.4 us with the clear).
+  const bool one_tile = LEAN && !STEM && units <= (int)gridDim.x;
+  const bool acc_smem = emit && p.N <= kMaxAccCols && !one_tile;
 
   if (!LEAN && P.dense_only) {
     // launched next to the fused small-FC kernel, which handles the zero-skip
@@ -388,13 +393,19 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
   // wait: no memory is read, and under programmatic dependent launch this
   // overlaps the tail of the kernel before.
   UnitGeo ug{};
-  if (warp < kProd && (int)blockIdx.x < units) ug = unit_geo(p, blockIdx.x, KS, kblocks, nt, BN, BK, threadIdx.x);
+  if (warp < kProd && (!LEAN || p.conv == 2) && (int)blockIdx.x < units)
+    ug = unit_geo(p, blockIdx.x, KS, kblocks, nt, BN, BK, threadIdx.x);
+  TileGeo tg{};  // dense lean producer: the CTA's tile `lane`
+  if (LEAN && !STEM && warp == 0) {
+    const int ul = (int)blockIdx.x + lane * (int)gridDim.x;
+    tg = tile_geo(p, ul < units ? ul : (int)blockIdx.x, nt, BN);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
   if constexpr (LEAN && !STEM) {
-    if (warp == Wp::kMma) prefetch_weights_l2(P.w, p.N, p.Ktot, lane);
+    if (warp == 1) prefetch_weights_l2(P.w, p.N, p.Ktot, lane);
   }
   pdl_wait();
   pdl_trigger();
@@ -409,10 +420,8 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
   // groups each (compacted), loaded as 32-column boxes with the 64-byte swizzle
   const bool compact = skip && p.conv == 0;  // (kblocks > 1: BK = 64)
 
-  // every tile of the CTA has the same columns
-  const bool fixed_cols = nt == 1 || (int)gridDim.x % nt == 0 || units <= (int)gridDim.x;
-  // ... and, on the dense path, a K range that fits the ring: its B blocks are
-  // loaded once and stay, and the ring carries A alone (a 1x1 expansion
+  // fixed columns and, on the dense path, a K range that fits the ring: its B
+  // blocks are loaded once and stay, and the ring carries A alone (a 1x1 expansion
   // [32,112,112,16] -> 96 spent 11 of 53 us on reloading its 12 KB of weights per tile)
   const bool resident_b =
       STEM || (LEAN && !skip && fixed_cols && kblocks <= S && units > (int)gridDim.x);
@@ -644,8 +653,11 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
         uint32_t ph = 0u;
         bool ok = true;
         for (int u0 = blockIdx.x; u0 < units && ok; u0 += 32 * (int)gridDim.x) {
-          const int ul = u0 + lane * (int)gridDim.x;
-          const TileGeo gl = tile_geo(p, ul < units ? ul : u0, nt, BN);
+          if (u0 != (int)blockIdx.x || !LEAN) {
+            const int ul = u0 + lane * (int)gridDim.x;
+            tg = tile_geo(p, ul < units ? ul : u0, nt, BN);
+          }
+          const TileGeo gl = tg;
           const int yl = p.conv == 2 ? gl.th0 * p.stride - p.pad : gl.m0, xl = gl.tw0 * p.stride - p.pad;
           for (int i = 0; i < 32 && u0 + i * (int)gridDim.x < units && ok; ++i) {
             const int y0 = __shfl_sync(0xffffffffu, yl, i), x0 = __shfl_sync(0xffffffffu, xl, i);
@@ -703,30 +715,35 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
         if (r < kMaxTaps) s_tap[r] = 0ull;
         named_bar_sync(1, kProdThreads);
         const int taps = p.kh * p.kw < kMaxTaps ? p.kh * p.kw : kMaxTaps;
-        // (with 96 producer threads warp 0 takes the last 32 rows as well)
-        for (int row = r; row < kBM; row += kProdThreads) {
-          bool rv = rvalid;
-          int ri = img, ry = oh, rx = ow;
-          if (row != r) tile_row(p, g, row, rv, ri, ry, rx);
-          for (int t0 = 0; t0 < taps; t0 += 8) {
-            unsigned long long wv[8];
+        auto mask_taps = [&](int t0, bool rv, int ri, int ry, int rx) {
+          unsigned long long wv[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {  // issue 8 taps' loads before reducing any
-              const int tp = t0 + u;
-              const int ih = ry * p.stride - p.pad + tp / p.kw;
-              const int iw = rx * p.stride - p.pad + tp % p.kw;
-              wv[u] = 0ull;
-              if (in_rowbm && tp < taps && rv && ih >= 0 && ih < p.H && iw >= 0 && iw < p.W)
-                wv[u] = in_rowbm[(((int64_t)ri * p.H + ih) * p.W + iw) * in_W64];
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              unsigned long long w = wv[u];
-#pragma unroll
-              for (int s = 16; s > 0; s >>= 1) w |= __shfl_xor_sync(0xffffffffu, w, s);
-              if (lane == 0 && w) atomicOr(&s_tap[t0 + u], w);
-            }
+          for (int u = 0; u < 8; ++u) {  // issue 8 taps' loads before reducing any
+            const int tp = t0 + u;
+            const int ih = ry * p.stride - p.pad + tp / p.kw;
+            const int iw = rx * p.stride - p.pad + tp % p.kw;
+            wv[u] = 0ull;
+            if (in_rowbm && tp < taps && rv && ih >= 0 && ih < p.H && iw >= 0 && iw < p.W)
+              wv[u] = in_rowbm[(((int64_t)ri * p.H + ih) * p.W + iw) * in_W64];
           }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            unsigned long long w = wv[u];
+#pragma unroll
+            for (int s = 16; s > 0; s >>= 1) w |= __shfl_xor_sync(0xffffffffu, w, s);
+            if (lane == 0 && w) atomicOr(&s_tap[t0 + u], w);
+          }
+        };
+        if constexpr (LEAN) {
+          // three warps share the four groups of 32 rows by 8 taps at a time
+          for (int part = warp; part < 4 * ((taps + 7) / 8); part += kProd) {
+            bool rv;
+            int ri, ry, rx;
+            tile_row(p, g, (part & 3) * 32 + lane, rv, ri, ry, rx);
+            mask_taps((part >> 2) * 8, rv, ri, ry, rx);
+          }
+        } else {
+          for (int t0 = 0; t0 < taps; t0 += 8) mask_taps(t0, rvalid, img, oh, ow);
         }
         named_bar_sync(1, kProdThreads);
         // no per-tap masks (too many taps, wide rows, or an input given without
@@ -1029,7 +1046,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
     constexpr bool kSliced = BN <= 128;
     constexpr int kBpw = BN / 32;
     uint32_t* const splane = reinterpret_cast<uint32_t*>(smem + C::kPlaneOff) + ew * (kBpw * 3 * 32) + lane;
-    if (kSliced && emit)
+    if (kSliced && emit && !one_tile)
 #pragma unroll
       for (int i = 0; i < kBpw * 3; ++i) splane[i * 32] = 0u;
     int nsum = 0, n0_last = 0;
@@ -1161,12 +1178,12 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
         }
         uint32_t* const sp = splane + (ncw == 1 ? cblk : 0) * 96;
         uint32_t pl[3] = {0u, 0u, 0u};
-        if (kSliced && emit)
+        if (kSliced && emit && !one_tile)
 #pragma unroll
           for (int i = 0; i < 3; ++i) pl[i] = sp[i * 32];
         block(raw, cblk, pl);
-        if (emit && (!kSliced || !fixed_cols || nsum == 6)) flush_counts(pl, g.n0 + cblk * 32);
-        if (kSliced && emit)
+        if (emit && (!kSliced || !fixed_cols || one_tile || nsum == 6)) flush_counts(pl, g.n0 + cblk * 32);
+        if (kSliced && emit && !one_tile)
 #pragma unroll
           for (int i = 0; i < 3; ++i) sp[i * 32] = pl[i];
       }
@@ -1181,7 +1198,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
     }
     if (emit) {
       flush_words();
-      if (kSliced && fixed_cols)
+      if (kSliced && fixed_cols && !one_tile)
         for (int k = 0; k < (ncw == 1 ? kBpw : 1); ++k) {
           uint32_t pl[3];
 #pragma unroll

@@ -291,13 +291,14 @@ __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) 
 // value is read, so it comes before the grid dependency wait.  ViT-B/16 at batch 8
 // 1137 -> 1128 us, an MLP [6304,768] x 3072 x 768 77.5 -> 72.7 us.
 __device__ __forceinline__ void prefetch_weights_l2(const void* w, int N, int Ktot, int lane) {
-  constexpr uint64_t kMax = 32u << 20, kReq = 2048;  // weights fetched ahead at most, a request
-  const uint64_t bytes = (uint64_t)N * (uint64_t)Ktot * 2u;
-  if (bytes > kMax) return;
-  const uint64_t share = (bytes / gridDim.x + 16u) & ~(uint64_t)15u;
-  const uint64_t w0 = share * blockIdx.x, w1 = w0 + share < bytes ? w0 + share : bytes;
-  for (uint64_t at = w0 + (uint64_t)lane * kReq; at < w1; at += 32u * kReq)
-    prefetch_l2_bulk(reinterpret_cast<const uint8_t*>(w) + at, (uint32_t)(w1 - at < kReq ? w1 - at : kReq));
+  constexpr uint32_t kMax = 32u << 20, kReq = 2048;  // weights fetched ahead at most, a request
+  const uint64_t all = (uint64_t)N * (uint64_t)Ktot * 2u;
+  if (all > kMax) return;
+  const uint32_t bytes = (uint32_t)all;  // (a 64-bit division would delay the warp by a tenth of a small GEMM)
+  const uint32_t share = (bytes / gridDim.x + 16u) & ~15u;
+  const uint32_t w0 = share * blockIdx.x, w1 = w0 + share < bytes ? w0 + share : bytes;
+  for (uint32_t at = w0 + (uint32_t)lane * kReq; at < w1; at += 32u * kReq)
+    prefetch_l2_bulk(reinterpret_cast<const uint8_t*>(w) + at, w1 - at < kReq ? w1 - at : kReq);
 }
 
 // Shared -> global tensor stores (bulk-group completion).
