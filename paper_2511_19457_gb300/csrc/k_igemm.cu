@@ -1838,7 +1838,7 @@ cudaError_t launch_igemm(const IgemmArgs& a_in, cudaStream_t s) {
   a.ksplit = ks;
   const int bk = k_block(a);
   if (bn == 64) {
-    const int split = onetile_split(a, mtiles, bk);
+    const int split = onetile_split(a, mtiles, bk, lean);
     if (split > 0) {
       a.ksplit = split;
       return launch_onetile(a, mtiles, bk, s);

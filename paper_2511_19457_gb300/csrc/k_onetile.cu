@@ -24,6 +24,7 @@
 #include <cuda.h>
 
 #include <cstring>
+#include <mutex>
 
 #include "igemm_geo.cuh"
 #include "sparoa_kernels.h"
@@ -499,14 +500,75 @@ cudaError_t launch_bk(const IgemmArgs& a, const CUtensorMap& tA, const CUtensorM
 
 }  // namespace
 
-int onetile_split(const IgemmArgs& a, int64_t mtiles, int bk) {
+// Clusters of `ks` CTAs that the device runs at once, asked once per device: a
+// cluster lies within one GPC and a CTA fills an SM, so 152 SMs hold 15 clusters
+// of 8 and 36 of 4 (a second round doubles the time: 128 x 1024 x 512, 16 tiles,
+// by 8 8.4 us, by 4 4.3 us).
+namespace {
+int clusters_at_once(int ks) {
+  constexpr int kDevices = 64;
+  static std::mutex mu;
+  static int known[kDevices][4];  // 0: not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  const int at = ks == 8 ? 3 : ks == 4 ? 2 : ks == 2 ? 1 : 0;
+  std::lock_guard<std::mutex> lock(mu);
+  if (dev < kDevices && known[dev][at] > 0) return known[dev][at];
+  const void* f = ks == 8   ? reinterpret_cast<const void*>(onetile_kernel<64, 8>)
+                  : ks == 4 ? reinterpret_cast<const void*>(onetile_kernel<64, 4>)
+                  : ks == 2 ? reinterpret_cast<const void*>(onetile_kernel<64, 2>)
+                            : reinterpret_cast<const void*>(onetile_kernel<64, 1>);
+  if (smem_optin(f, (size_t)Lay<64>::kSmem) != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)ks);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = (size_t)Lay<64>::kSmem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)ks;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess) {
+    cudaGetLastError();  // (not the launch's error)
+    return 0;
+  }
+  if (dev < kDevices) known[dev][at] = n;
+  return n;
+}
+}  // namespace
+
+// Cluster size: the largest of 8, 4 and 2 whose clusters all run at once and whose
+// CTAs keep enough K blocks, 1 for long K; else the persistent kernel.  On 128 rows,
+// dense, without / with occupancy (and its clear), us:
+//   K = 64     77 tiles            by 1 5.1 / 7.8   persistent 3.8 / 6.4
+//   K = 256    24 tiles, by 4 4.5 / 6.3             4.3 / 6.9
+//   K = 512    24 tiles, by 4 4.9 / 6.9             5.1 / 7.7
+//              76 tiles, by 2 6.0 / 8.5             5.3 / 7.9
+//   K = 768    76 tiles, by 2 6.2 / 8.7             6.0 / 8.6
+//   K = 1152   14 tiles, by 8 5.0 / 6.8, by 4 4.7 / 6.8
+//              90 tiles            by 1 8.6 / 11.1  7.4 / 10.0
+//   K = 4608   90 tiles            by 1 18.2 / 21.1  19.8 / 22.6
+// A convolution's zero-skip path is much slower in the persistent kernel (its
+// masks, then its loads, tile by tile: [8,28,28,128] 3x3 by 1 13, persistent 19.6;
+// dense 11.4 and 11.2), so it goes there only where the dense path is forced.
+// fp32 output (`lean` false), whose persistent kernel is slower, takes what fits.
+int onetile_split(const IgemmArgs& a, int64_t mtiles, int bk, bool lean) {
   const int64_t tiles = mtiles * ((a.N + kBN - 1) / kBN);
-  const int sms = device_sm_count();
-  if (a.conv == 1 || tiles > sms) return 0;
   const int kblocks = (a.Ktot + bk - 1) / bk;
-  int ks = 8;
-  while (ks > 1 && (tiles * ks > sms || kblocks < ks)) ks /= 2;
-  return ks;
+  if (a.conv == 1 || tiles > device_sm_count()) return 0;
+  for (int ks = 8; ks >= 1; ks /= 2) {
+    const int least = !lean        ? ks
+                      : ks == 8    ? 24
+                      : a.conv     ? (ks > 1 || a.disp.force != 1 ? ks : 48)
+                      : ks == 4    ? (a.emit ? 4 : 8)
+                      : ks == 2    ? (a.emit ? 8 : 12)
+                                   : 48;
+    if (kblocks >= least && tiles * ks <= device_sm_count() && (ks == 1 || tiles <= clusters_at_once(ks))) return ks;
+  }
+  return 0;
 }
 
 cudaError_t launch_onetile(const IgemmArgs& a, int64_t mtiles, int bk, cudaStream_t s) {

@@ -145,9 +145,10 @@ bool stem_plan(const __nv_bfloat16* x, int64_t n, int H, int W, int C, int N, in
                StemGeo* g);
 
 // One 128 x 64 output tile per cluster of up to 8 CTAs that share its K range
-// (k_onetile.cu).  onetile_split: the cluster size for K blocks of `bk`, 0
-// where the shape is not the kernel's (more tiles than SMs, or the gather mode).
-int onetile_split(const IgemmArgs& a, int64_t mtiles, int bk);
+// (k_onetile.cu).  onetile_split: the cluster size for K blocks of `bk`, 0 where
+// the persistent kernel takes the call (more tiles than SMs, the gather mode,
+// too few K blocks).  lean: that kernel's lean variant would.
+int onetile_split(const IgemmArgs& a, int64_t mtiles, int bk, bool lean);
 cudaError_t launch_onetile(const IgemmArgs& a, int64_t mtiles, int bk, cudaStream_t s);  // a.ksplit set
 
 // Streaming multiprocessors of the current device (cached per device).
