@@ -413,8 +413,8 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
   // with dense_only the zero-skip kernel of this launch runs instead
   const bool run = !(!LEAN && P.dense_only && path == 2);
   if (run) record_path(P.disp, path);
-  // (nothing can be left out of a stem's tiles, a GEMM with one K block or an
-  // input without block masks)
+  // (nothing can be left out of the loads of a stem, a GEMM with one K block or
+  // an input without block masks)
   const bool skip = !STEM && path == 2 && !(p.conv == 0 && (kblocks == 1 || in_blk == nullptr));
   // zero-skip GEMM with 64-wide K blocks: stages hold two occupied 32-column
   // groups each (compacted), loaded as 32-column boxes with the 64-byte swizzle
@@ -922,6 +922,8 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
       next();
       return true;
     };
+    const bool halves = !STEM && BK == 64 && path == 2 && p.conv == 0 && kblocks == 1 && kgroups == 2 && in_blk != nullptr;
+    uint32_t half_bits = 0u;  // lane l: the occupied groups of the CTA's tile j + l
     bool ok = !resident_b || mbar_wait_warp(bar_resb, 0u, err, s_abort, kErrTimeoutFull, wlim);
     if (resident_b) tc_fence_after();
     for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++j) {
@@ -943,6 +945,37 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
               if (k < nks)
                 tc_mma_bf16(d, ad + (uint64_t)((k >> 2) * (kBM * BK * 2 / 16) + 2 * (k & 3)),
                             bd0 + (uint64_t)((k >> 2) * (C::kBStage / 16) + 2 * (k & 3)), idesc, 1u);
+            tc_commit(bar_empty + 8 * slot);
+          }
+          __syncwarp();
+          next();
+        }
+      } else if (halves) {
+        // the zero-skip path of one K block of two groups: only the occupied one
+        // (group 0 where the tile has none, so that its accumulator is written)
+        if ((j & 31) == 0) {
+          const int ul = u + lane * (int)gridDim.x;
+          half_bits = 0u;
+          if (ul < units) {
+            const uint32_t* words = in_blk + (int64_t)(ul / nt) * in_C32;
+            half_bits = (words[0] ? 1u : 0u) | (words[1] ? 2u : 0u);
+          }
+        }
+        const uint32_t hv = __shfl_sync(0xffffffffu, half_bits, j & 31);
+        ok = mbar_wait_warp(bar_full + 8 * slot, ph, err, s_abort, kErrTimeoutFull, wlim);
+        if (ok) {
+          tc_fence_after();
+          const uint64_t b0 = resident_b ? bd0 : bd;
+          if (el) {
+            if (hv != 2u) {
+              tc_mma_bf16(d, ad, b0, idesc, 0u);
+              tc_mma_bf16(d, ad + 2, b0 + 2, idesc, 1u);
+            }
+            if (hv & 2u) {
+              if (hv == 3u) tc_mma_bf16(d, ad + 4, b0 + 4, idesc, 1u);
+              else tc_mma_bf16(d, ad + 4, b0 + 4, idesc, 0u);
+              tc_mma_bf16(d, ad + 6, b0 + 6, idesc, 1u);
+            }
             tc_commit(bar_empty + 8 * slot);
           }
           __syncwarp();

@@ -38,7 +38,7 @@ constexpr int kWarps = 8;                     // producers, then epilogue
 constexpr int kWorkers = 32 * kWarps;
 constexpr int kThreads = kWorkers + 32;       // + the MMA warp
 constexpr int kStages = kWarps;               // stage s is filled by warp s
-constexpr int kMaxItems = 2048;               // listed K blocks of a CTA's share (more: none left out)
+constexpr int kMaxItems = 2048;               // K blocks of a CTA's share (more: another kernel)
 constexpr int kMaxTapsHere = 64;
 constexpr int kPitch = kBN + 4;               // floats per row of the partial tile
 constexpr uint32_t kTmemCols = 64;
@@ -54,7 +54,7 @@ struct Lay {
   static constexpr int kNumBars = 2 * kStages + 2;  // full, empty, accumulator, drain
   static constexpr int kFlag = kBar + kNumBars * 8;  // abort, tmem, items, issued[kStages]
   static constexpr int kBits = kFlag + (3 + kStages) * 4 + 4;
-  static constexpr int kTap = (kBits + kMaxItems / 8 + 7) & ~7;
+  static constexpr int kTap = (kBits + 2 * kMaxItems / 8 + 7) & ~7;
   static constexpr int kItems = kTap + kMaxTapsHere * 8;
   static constexpr int kCnt = kItems + kMaxItems * 2;
   static constexpr int kWord = kCnt + kBN * 4;  // [rows of the share][2] non-zero bits
@@ -94,7 +94,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(flags + 1);
   volatile int* s_nitems = flags + 2;
   volatile int* s_issued = flags + 3;  // [kStages] fills of stage s so far
-  uint32_t* s_bits = reinterpret_cast<uint32_t*>(smem + L::kBits);
+  // occupied K blocks of the share: their first and their last 32 columns
+  uint32_t* s_lo = reinterpret_cast<uint32_t*>(smem + L::kBits);
+  uint32_t* s_hi = s_lo + kMaxItems / 32;
   unsigned long long* s_tap = reinterpret_cast<unsigned long long*>(smem + L::kTap);
   uint16_t* s_items = reinterpret_cast<uint16_t*>(smem + L::kItems);
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(smem + L::kCnt);
@@ -131,6 +133,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     prefetch_tmap(&tmB);
   }
   if (warp == kWarps) tmem_alloc(smem_u32(s_tmem), kTmemCols);
+  if (threadIdx.x == kWorkers + 1) s_lo[0] = 0u;
   if (threadIdx.x < kBN) s_cnt[threadIdx.x] = 0u;
   if (threadIdx.x >= 64 && threadIdx.x < 64 + kMaxTapsHere) s_tap[threadIdx.x - 64] = 0ull;
   const int kblocks = (p.Ktot + BK - 1) / BK;
@@ -145,18 +148,52 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t sa = sbase + warp * L::kStage;
   // K block kb into stage `warp`: operand B (the weights), operand A
   auto load_b = [&](int kb) { tma_load_2d(sa + L::kA, &tmB, fb, kb * BK, g.n0); };
-  auto load_a = [&](int kb) {
+  int ac, ax, ay;  // operand A's next box: channel, column, row (GEMM: channel, row)
+  auto seek_a = [&](int kb) {
     if (p.conv == 0) {
-      tma_load_2d(sa, &tmA, fb, kb * BK, g.m0);
+      ac = kb * BK;
+      ax = 0;
+      ay = g.m0;
     } else {
-      const int tp = kb / cbpt, cb = kb - tp * cbpt;
-      const int rr = tp / p.kw, ss = tp - rr * p.kw;
-      tma_load_4d(sa, &tmA, fb, cb * BK, x0 + ss, y0 + rr, g.tn0);
+      const int tp = kb / cbpt;
+      ac = (kb - tp * cbpt) * BK;
+      ay = tp / p.kw;
+      ax = x0 + tp - ay * p.kw;
+      ay += y0;
     }
   };
+  auto load_a = [&]() {
+    if (p.conv == 0) tma_load_2d(sa, &tmA, fb, ac, ay);
+    else tma_load_4d(sa, &tmA, fb, ac, ax, ay, g.tn0);
+  };
+  seek_a(kb0 + warp);
   const uint32_t stage_bytes = (uint32_t)((a_rows + kBN) * BK * 2);
   const bool has_bits = p.conv == 0 ? P.in_blk != nullptr
                                     : (P.in_rowbm != nullptr && P.in_W64 == 1 && p.kh * p.kw <= kMaxTapsHere);
+  const bool masks = has_bits && P.disp.force != 1 && warp < kWarps;
+  const uint32_t* const words = p.conv == 0 && has_bits ? P.in_blk + (int64_t)(g.m0 >> 7) * P.in_C32 : nullptr;
+  // a convolution's share: this thread's taps from tap0 on in steps of 2, up to t1
+  int tap0 = 0, t1 = -1;
+  const uint64_t* px = nullptr;  // row words at the origin of this thread's pixel's window
+  int iy = 0, ix = 0;
+  uint32_t inv_kw = 0u;          // tap / kw = tap * inv_kw >> 16 (taps < 64)
+  if (masks && p.conv == 2) {
+    tap0 = kb0 / cbpt + ((int)threadIdx.x >> 7);
+    t1 = (kb0 + span - 1) / cbpt;
+    inv_kw = 65536u / (uint32_t)p.kw + 1u;
+    bool pv;
+    int pn, oy, ox;
+    tile_row(p, g, threadIdx.x & 127, pv, pn, oy, ox);
+    iy = oy * p.stride - p.pad;
+    ix = ox * p.stride - p.pad;
+    if (pv) px = reinterpret_cast<const uint64_t*>(P.in_rowbm) + ((int64_t)pn * p.H + iy) * p.W + ix;
+  }
+  auto load_tap = [&](int tap) -> unsigned long long {
+    const int tr = (int)((uint32_t)tap * inv_kw >> 16), tc = tap - tr * p.kw;
+    if (px && tap <= t1 && (unsigned)(iy + tr) < (unsigned)p.H && (unsigned)(ix + tc) < (unsigned)p.W)
+      return px[tr * p.W + tc];
+    return 0ull;
+  };
   // output rows and column affine of this thread
   const int c4 = threadIdx.x & 15;
   const int col = g.n0 + 4 * c4;
@@ -184,71 +221,95 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_arrive_expect_tx(fb, stage_bytes);
       load_b(kb0 + warp);
     }
-    load_a(kb0 + warp);
+    load_a();
     s_issued[warp] = 1;
   }
+  // ---- zero-skip path: the occupied K blocks.  The first ring full is loaded
+  // whatever it holds (the masks arrive no sooner than the blocks), of the rest
+  // of the share only occupied blocks; empty blocks, and the empty half of a
+  // GEMM's block (32 columns), are not multiplied.  The masks' first loads are
+  // on their way before the rule is known.  (Short, rolled code: a CTA runs it
+  // once, and every eight instructions cost an instruction cache miss.)
+  unsigned long long w = 0ull;
+  if (masks && p.conv == 2) w = load_tap(tap0);
+  uint32_t glo = 0u, ghi = 0u;
+  auto load_words = [&](int i0) {  // the mask words of K block i0 + lane of the share
+    const int b = kb0 + i0 + lane;
+    glo = ghi = 0u;
+    if (i0 + lane < span) {
+      glo = words[b * (BK / 32)];
+      if (BK == 64 && 2 * b + 1 < P.in_C32) ghi = words[2 * b + 1];
+    }
+  };
+  if (masks && p.conv == 0) load_words(warp * 32);
   const int path = decide_path(P.disp);
   record_path(P.disp, path);
-
-  // ---- zero-skip path: the occupied K blocks.  The first ring full is loaded
-  // and multiplied whatever it holds: reading the masks takes longer (3000
-  // cycles, several dependent loads) than the loads and the MMAs they could
-  // save.  Of the rest of the share only occupied blocks are listed and loaded;
-  // the masks are read while the first ring full is in flight.
-  const bool listed = path == 2 && has_bits && span > kStages && span <= kMaxItems;
+  const bool listed = path == 2 && has_bits;
   if (listed && warp < kWarps) {
+    // nothing but occupied blocks is added to the accumulator
+    tmem_st32_zero(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 32));
     if (p.conv == 2) {
       // per tap of the share: the occupied 64-channel tiles over the tile's pixels
-      const int t0 = kb0 / cbpt, t1 = (kb0 + span - 1) / cbpt;
-      bool v;
-      int img, oh, ow;
-      tile_row(p, g, threadIdx.x & 127, v, img, oh, ow);
-      for (int tb = t0 + ((int)threadIdx.x >> 7); tb <= t1; tb += 8) {
-        unsigned long long w[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {  // four taps' loads in flight
-          const int tp = tb + 2 * i;
-          const int ih = oh * p.stride - p.pad + tp / p.kw, iw = ow * p.stride - p.pad + tp % p.kw;
-          w[i] = 0ull;
-          if (v && tp <= t1 && ih >= 0 && ih < p.H && iw >= 0 && iw < p.W)
-            w[i] = P.in_rowbm[((int64_t)img * p.H + ih) * p.W + iw];
+      const bool direct = BK == 64 && span <= 32;  // a tile is a K block: its bit at once
+#pragma unroll 1
+      for (int tp = tap0; tp <= t1; tp += 2) {
+        const unsigned long long ahead = load_tap(tp + 2);
+        const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)w);
+        const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(w >> 32));
+        const unsigned long long ww = ((unsigned long long)hi << 32) | lo;
+        const int sh = tp * cbpt - kb0;
+        if (lane == 0 && ww) {
+          if (direct) atomicOr(&s_lo[0], (uint32_t)(sh >= 0 ? ww << sh : ww >> -sh) & (0xFFFFFFFFu >> (32 - span)));
+          else atomicOr(&s_tap[tp], ww);
         }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)w[i]);
-          const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(w[i] >> 32));
-          if (lane == 0 && (lo | hi)) atomicOr(&s_tap[tb + 2 * i], ((unsigned long long)hi << 32) | lo);
+        w = ahead;
+      }
+      if (!direct) {
+        named_bar_sync(1, kWorkers);
+        for (int i0 = warp * 32; i0 < span; i0 += kWorkers) {
+          const int b = kb0 + i0 + lane, tp = b / cbpt;
+          const uint32_t bits = __ballot_sync(
+              0xffffffffu, i0 + lane < span && ((s_tap[tp] >> (((b - tp * cbpt) * BK) >> 6)) & 1ull) != 0ull);
+          if (lane == 0) s_lo[i0 >> 5] = bits;
         }
       }
+    } else {
+      for (int i0 = warp * 32; i0 < span; i0 += kWorkers) {
+        if (i0 >= kWorkers) load_words(i0);
+        const uint32_t lo = __ballot_sync(0xffffffffu, glo != 0u), hi = __ballot_sync(0xffffffffu, ghi != 0u);
+        if (lane == 0) {
+          s_lo[i0 >> 5] = lo;
+          s_hi[i0 >> 5] = hi;
+        }
+      }
+    }
+    if (span > 32) {  // (up to 32 blocks, the one word is the list)
       named_bar_sync(1, kWorkers);
-    }
-    const uint32_t* words = p.conv == 0 ? P.in_blk + (int64_t)(g.m0 >> 7) * P.in_C32 : nullptr;
-    for (int i0 = warp * 32; i0 < span; i0 += kWorkers) {
-      const int b = kb0 + i0 + lane;
-      bool occ = false;
-      if (i0 + lane < span) {
-        if (p.conv == 0) {
-          if (BK == 32) occ = words[b] != 0u;
-          else occ = words[2 * b] != 0u || (2 * b + 1 < P.in_C32 && words[2 * b + 1] != 0u);
-        } else {
-          const int tp = b / cbpt;
-          occ = ((s_tap[tp] >> (((b - tp * cbpt) * BK) >> 6)) & 1ull) != 0ull;
+      if (warp == 0) {
+        int n = 0;
+        for (int w32 = 0; w32 * 32 < span; ++w32) {
+          uint32_t bits = p.conv == 2 ? s_lo[w32] : s_lo[w32] | s_hi[w32];
+          if (w32 == 0) bits &= ~((1u << kStages) - 1u);
+          if ((bits >> lane) & 1u) s_items[n + __popc(bits & ((1u << lane) - 1u))] = (uint16_t)(w32 * 32 + lane);
+          n += __popc(bits);
         }
+        if (lane == 0) *s_nitems = n;
       }
-      const uint32_t bits = __ballot_sync(0xffffffffu, occ);
-      if (lane == 0) s_bits[i0 >> 5] = bits;
     }
-    named_bar_sync(1, kWorkers);
-    if (warp == 0) {
-      int n = 0;
-      for (int w = 0; w * 32 < span; ++w) {
-        const uint32_t bits = w == 0 ? s_bits[0] & ~((1u << kStages) - 1u) : s_bits[w];
-        if ((bits >> lane) & 1u) s_items[n + __popc(bits & ((1u << lane) - 1u))] = (uint16_t)(w * 32 + lane);
-        n += __popc(bits);
-      }
-      if (lane == 0) *s_nitems = n;
-    }
+    tmem_wait_st();
+    tc_fence_before();
   }
+  // after the list's barrier: the occupied blocks behind the first ring full
+  auto listed_rest = [&]() -> int {
+    if (span > 32) return *s_nitems;
+    return __popc((p.conv == 2 ? s_lo[0] : s_lo[0] | s_hi[0]) & ~((1u << kStages) - 1u));
+  };
+  auto listed_block = [&](int i) -> int {
+    if (span > 32) return (int)s_items[i];
+    uint32_t bits = (p.conv == 2 ? s_lo[0] : s_lo[0] | s_hi[0]) & ~((1u << kStages) - 1u);
+    for (; i > 0; --i) bits &= bits - 1u;
+    return __ffs(bits) - 1;
+  };
   if (warp == kWarps) {
     // ------------------------------------------------------------------ MMA issue
     constexpr uint32_t idesc = idesc_bf16_f32(kBM, kBN);
@@ -256,31 +317,99 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint64_t ad = smem_desc_kmajor<BK>(sbase), bd = smem_desc_kmajor<BK>(sbase + L::kA);
     bool ok = true;
     uint32_t ph = 0u;
-    int rest = listed ? 0 : span - lap;  // K blocks behind the first ring full
-    // stages s = i % 8 unrolled: the descriptors are constants from the base
-    for (int i0 = 0; ok && i0 < lap + rest; i0 += kStages) {
+    // (the dense path's stages s = i % 8 are unrolled: the descriptors are
+    // constants from the base)
+    if (!listed) {
+      for (int i0 = 0; ok && i0 < span; i0 += kStages) {
 #pragma unroll
-      for (int s = 0; s < kStages; ++s) {
-        if (ok && i0 + s < lap + rest) {
-          ok = mbar_wait_warp(bar_full + 8 * s, ph, err, s_abort, kErrTimeoutFull, wlim);
-          if (ok) {
-            tc_fence_after();
-            const uint64_t a = ad + (uint64_t)(s * (L::kStage / 16)), b = bd + (uint64_t)(s * (L::kStage / 16));
-            if (el) {
-              if (s == 0 && i0 == 0) tc_mma_bf16(tmem, a, b, idesc, 0u);
-              else tc_mma_bf16(tmem, a, b, idesc, 1u);
+        for (int s = 0; s < kStages; ++s) {
+          if (ok && i0 + s < span) {
+            ok = mbar_wait_warp(bar_full + 8 * s, ph, err, s_abort, kErrTimeoutFull, wlim);
+            if (ok) {
+              tc_fence_after();
+              const uint64_t a = ad + (uint64_t)(s * (L::kStage / 16)), b = bd + (uint64_t)(s * (L::kStage / 16));
+              if (el) {
+                if (s == 0 && i0 == 0) tc_mma_bf16(tmem, a, b, idesc, 0u);
+                else tc_mma_bf16(tmem, a, b, idesc, 1u);
 #pragma unroll
-              for (int k = 1; k < BK / 16; ++k) tc_mma_bf16(tmem, a + (uint64_t)(2 * k), b + (uint64_t)(2 * k), idesc, 1u);
-              tc_commit(bar_empty + 8 * s);
+                for (int k = 1; k < BK / 16; ++k) tc_mma_bf16(tmem, a + (uint64_t)(2 * k), b + (uint64_t)(2 * k), idesc, 1u);
+                tc_commit(bar_empty + 8 * s);
+              }
             }
+            __syncwarp();
           }
-          __syncwarp();
         }
+        ph ^= 1u;
       }
-      ph ^= 1u;
-      if (listed && i0 == 0) {
-        named_bar_sync(2, kThreads);  // the list is complete
-        rest = *s_nitems;
+    } else {
+      // the first ring full, whatever the masks say in each stage (rolled: a
+      // block's code once), into an accumulator of zeros
+      named_bar_sync(2, kThreads);  // the list is complete
+      tc_fence_after();
+      const uint32_t wlo = s_lo[0], whi = p.conv == 2 ? wlo : s_hi[0];
+      const int total = lap + listed_rest();
+      uint64_t a = ad, b = bd;
+#pragma unroll 1
+      for (int s = 0; ok && s < lap; ++s) {
+        ok = mbar_wait_warp(bar_full + 8 * s, 0u, err, s_abort, kErrTimeoutFull, wlim);
+        if (ok) {
+          tc_fence_after();
+          if (el) {
+            if ((wlo >> s) & 1u) {
+              tc_mma_bf16(tmem, a, b, idesc, 1u);
+              tc_mma_bf16(tmem, a + 2, b + 2, idesc, 1u);
+            }
+            if (BK == 64 && ((whi >> s) & 1u)) {
+              tc_mma_bf16(tmem, a + 4, b + 4, idesc, 1u);
+              tc_mma_bf16(tmem, a + 6, b + 6, idesc, 1u);
+            }
+            tc_commit(bar_empty + 8 * s);
+          }
+        }
+        __syncwarp();
+        a += L::kStage / 16;
+        b += L::kStage / 16;
+      }
+      ph = 1u;
+      // the listed ones, unrolled again: bit s of mlo, mhi: the first, last 32
+      // columns of stage s take part (a convolution's listed blocks are whole)
+      uint32_t mlo = 0xFFu, mhi = 0xFFu;
+      for (int i0 = kStages; ok && i0 < total; i0 += kStages) {
+        if (p.conv == 0) {
+          bool flo = false, fhi = false;
+          if (lane < kStages && i0 + lane < total) {
+            const int kb = listed_block(i0 - kStages + lane);
+            flo = ((s_lo[kb >> 5] >> (kb & 31)) & 1u) != 0u;
+            fhi = BK == 32 || ((s_hi[kb >> 5] >> (kb & 31)) & 1u) != 0u;
+          }
+          mlo = __ballot_sync(0xffffffffu, flo);
+          mhi = __ballot_sync(0xffffffffu, fhi);
+        }
+#pragma unroll
+        for (int s = 0; s < kStages; ++s) {
+          if (ok && i0 + s < total) {
+            ok = mbar_wait_warp(bar_full + 8 * s, ph, err, s_abort, kErrTimeoutFull, wlim);
+            if (ok) {
+              tc_fence_after();
+              const uint64_t as = ad + (uint64_t)(s * (L::kStage / 16)), bs = bd + (uint64_t)(s * (L::kStage / 16));
+              if (((mlo & mhi) >> s) & 1u) {
+                if (el) {
+#pragma unroll
+                  for (int k = 0; k < BK / 16; ++k)
+                    tc_mma_bf16(tmem, as + (uint64_t)(2 * k), bs + (uint64_t)(2 * k), idesc, 1u);
+                  tc_commit(bar_empty + 8 * s);
+                }
+              } else if (el) {  // one half
+                const uint64_t k0 = ((mlo >> s) & 1u) ? 0u : 4u;
+                tc_mma_bf16(tmem, as + k0, bs + k0, idesc, 1u);
+                tc_mma_bf16(tmem, as + k0 + 2, bs + k0 + 2, idesc, 1u);
+                tc_commit(bar_empty + 8 * s);
+              }
+            }
+            __syncwarp();
+          }
+        }
+        ph ^= 1u;
       }
     }
     // (the error-path tests leave the accumulator unsignalled)
@@ -291,15 +420,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else {
     // ------------------------------------------------------------------ producers
     if (listed) named_bar_sync(2, kThreads);
-    const int rest = listed ? *s_nitems : span - lap;
+    const int rest = listed ? listed_rest() : span - lap;
     if (lane == 0) {
       int fills = warp < lap ? 1 : 0;
       for (int i = warp; i < rest; i += kStages, ++fills) {  // (only when lap == kStages)
         if (!mbar_wait(bar_empty + 8 * warp, (uint32_t)((fills - 1) & 1), err, s_abort, kErrTimeoutEmpty, wlim)) break;
-        const int kb = kb0 + (listed ? (int)s_items[i] : kStages + i);
+        const int kb = kb0 + (listed ? listed_block(i) : kStages + i);
         mbar_arrive_expect_tx(fb, stage_bytes);
         load_b(kb);
-        load_a(kb);
+        seek_a(kb);
+        load_a();
       }
       s_issued[warp] = fills;
     }
@@ -558,7 +688,7 @@ int clusters_at_once(int ks) {
 int onetile_split(const IgemmArgs& a, int64_t mtiles, int bk, bool lean) {
   const int64_t tiles = mtiles * ((a.N + kBN - 1) / kBN);
   const int kblocks = (a.Ktot + bk - 1) / bk;
-  if (a.conv == 1 || tiles > device_sm_count()) return 0;
+  if (a.conv == 1 || tiles > device_sm_count() || kblocks > kMaxItems) return 0;
   for (int ks = 8; ks >= 1; ks /= 2) {
     const int least = !lean        ? ks
                       : ks == 8    ? 24
