@@ -90,3 +90,21 @@ def test_patch_embedding(sp, ctx, B, H, W, C, Co, k, stride, force):
     ref = orc.conv2d(d["x"], B, H, W, C, d["w"], Co, k, k, stride, 0, bn=d["bn"], act=1)
     assert_close(y.float().cpu().numpy(), ref, what="patches")
     assert_occ_equal(yo.to_host(), orc.stats(sp.device_to_bits(y).reshape(-1), R, Co), "patches")
+
+
+def test_stem_rounding(sp, ctx):
+    """The 7x7 stem's sums are no less exact than those over im2col rows: 2-norm of
+    the distance to the correctly rounded result over its norm, 2.66e-5 there.  One
+    accumulator for its eleven k-steps leaves 2.8e-5, two that share them 2.0e-5."""
+    err = ref2 = 0.0
+    for seed in range(4):
+        g = torch.Generator().manual_seed(seed)
+        x = torch.randn(8, 224, 224, 3, generator=g).to(torch.bfloat16).cuda()
+        w = (torch.randn(64, 7, 7, 3, generator=g) / 147 ** 0.5).to(torch.bfloat16).cuda()
+        y = torch.empty(8, 112, 112, 64, dtype=torch.bfloat16, device="cuda")
+        sp.sparoa_conv2d(ctx, x, w, y, stride=2, pad=3)
+        want = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), w.double().permute(0, 3, 1, 2), stride=2,
+                                          padding=3).permute(0, 2, 3, 1).to(torch.bfloat16).double()
+        err += float((y.double() - want).pow(2).sum())
+        ref2 += float(want.pow(2).sum())
+    assert (err / ref2) ** 0.5 <= 2.4e-5
