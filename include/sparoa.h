@@ -295,8 +295,12 @@ sparoa_status sparoa_op_stats(sparoa_ctx *ctx, const void *x, int64_t N, int64_t
  * unless host_out is given.  Dense path: tcgen05 tensor-core GEMM.  Zero-skip
  * path: for M <= 128 with W_kn given, a column-compacting kernel that reads
  * only the rows of W_kn whose activation column is occupied; otherwise a
- * tcgen05 GEMM that stages only the 32-wide K blocks occupied in each 128-row
- * block of x (with few output tiles 64-wide ones, after the first eight).
+ * tcgen05 GEMM that multiplies only the 32-column groups of K occupied in each
+ * 128-row block of x.  Groups that are left out are not loaded either, except, with
+ * few output tiles, in the first eight 64-column blocks of each of the up to eight
+ * shares a tile's K range is cut into (K <= 4096 is then loaded whole).  Weights
+ * that meet left-out groups only do not reach y, whatever their values; a block of
+ * x with nothing but zeros may still multiply its first group.
  *   W_kn    optional [K][N] copy of W (nullable)
  *   y_dtype SPAROA_BF16 or SPAROA_F32
  *   y_occ   occupancy of y to write (nullable; bf16 y only)
