@@ -7,15 +7,6 @@ namespace sparoa {
 
 constexpr int kBM = 128;  // output rows (pixels) of a tile
 
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint32_t bar, int c0,
-                                            int c1, int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
-      : "memory");
-}
-
 // Launch geometry copied out of the kernel parameters into registers once:
 // reading IgemmArgs fields through a reference is a memory load, and every
 // asm statement with a memory clobber would force it again.

@@ -78,15 +78,6 @@ struct Dw3Geo {
   int w_off, aff_off, cnt_off;  // shared-memory carve (bytes); the rings come first
 };
 
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1,
-                                            int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
-      : "memory");
-}
-
 // a bf16 pair widened to fp32 (exact)
 __device__ __forceinline__ f2_t widen(uint32_t w) {
   return f2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));

@@ -3,9 +3,10 @@
 //
 // Persistent: one CTA per SM walks the output tiles (128 rows x BN columns)
 // of y = epilogue(A * B^T) with a static round-robin schedule.  Two tensor-
-// memory accumulators alternate between tiles, so the epilogue of tile i
-// (TMEM -> registers -> swizzled shared memory -> TMA store) overlaps the MMAs
-// of tile i + 1, and the shared-memory stage ring never drains between tiles.
+// memory accumulators (lean kernels up to 128 columns wide: four) alternate
+// between tiles, so the epilogue of tile i (TMEM -> registers -> swizzled shared
+// memory -> TMA store) overlaps the MMAs of tile i + 1, and the shared-memory
+// stage ring never drains between tiles.
 //
 // B [N, K] holds the weights (K-major; [C_out][kh][kw][C] for a convolution)
 // and is loaded by TMA.  A (128 rows of K) comes in one of three ways:
@@ -35,13 +36,14 @@
 // The epilogue applies bias / batch norm / residual / activation, stores y and
 // writes y's Eq. 1 count and occupancy bitmaps for the next operator.
 //
-// Warp roles: producer warps (the skip masks; thread 0 issues TMA; all 128
-// gather in mode 1), epilogue warps from warp 4 on (by TMEM lane quarter, each
-// taking 32-column blocks), one warp for TMEM allocation and MMA issue.
+// Warp roles: producer warps (the skip masks; one lane of warp 0 issues TMA; in
+// mode 1 all 128 threads gather, in stems all seven warps build), epilogue warps
+// from warp 4 (stems: 8) on by TMEM lane quarter, each taking 32-column blocks,
+// one warp for TMEM allocation and MMA issue.
 //
-// Each tile shape is compiled three times: the general kernel, and lean ones
-// for modes 0 and 2 without a K split or fp32 output, without a residual and
-// with one (N % 8 == 0).  Small-K problems are bound by the epilogue's latency
+// Each tile shape is compiled three times: the general kernel (mode 1, fp32
+// output, the dense half of a small FC), and lean ones for modes 0 and 2 with
+// bf16 output, without a residual and with one (N % 8 == 0).  Small-K problems are bound by the epilogue's latency
 // and by what feeds it, so the lean kernel has 16 epilogue warps that never wait
 // for each other, four accumulators in flight (up to 128-wide tiles), one
 // converged producer warp that lays out 32 tiles at a time, and keeps weights
@@ -253,10 +255,6 @@ __device__ __forceinline__ UnitGeo unit_geo(const Geo& p, int u, int KS, int kbl
   return q;
 }
 
-template <bool B>
-struct BoolConst {
-  static constexpr bool value = B;
-};
 template <int I>
 struct IntConst {
   static constexpr int value = I;
@@ -280,8 +278,9 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
   const Geo p = make_geo(P);
   // lean kernels (LEAN 1: no residual, 2: a residual and N % 8 == 0): TMA
   // producers only (mode 0 or 2), no K split, bf16 output (the host launches
-  // them only then)
+  // them only then); the general kernel has modes 0 and 1
   if (LEAN) __builtin_assume(p.conv != 1);
+  else __builtin_assume(p.conv != 2);
   if (STEM) __builtin_assume(p.conv == 0);
   const EpiDev ep = P.ep;
   const int act = P.ep.act;
@@ -637,7 +636,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
         if (lane == 0) *s_issued = it;  // stages this CTA filled (TMA copies issued)
       }
     } else if (p.conv != 1 && !skip) {
-      // Dense path: one converged warp, one elected lane issues.  The tiles'
+      // Dense path (mode 2: lean kernels only): one converged warp, one elected lane issues.  The tiles'
       // origins (a few integer divisions each) are computed for 32 tiles at a
       // time, one per lane.
       if (warp == 0) {
@@ -697,8 +696,8 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
         if (lane == 0) *s_issued = it;  // stages this CTA filled (TMA copies issued)
       }
     } else {
+    // The gather of mode 1 (general kernel), or mode 2 on the zero-skip path (lean).
     const int r = threadIdx.x;
-    const int cb_per_tap = p.Cp / BK;
     int it = 0;        // stages filled so far (ring position)
     int pending = 0;   // mode 1: filled stages whose A arrivals are still owed
     bool ok = true;
@@ -781,21 +780,19 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
         }
       }
       if (!ok) continue;  // keep the skip-mask barriers in step; issue nothing more
-      if (LEAN || p.conv != 1) {
+      if constexpr (LEAN) {
         if (r == 0) {
-          // The issuing lane is slow at anything but issuing: ring slot, phase
-          // and the (tap, channel block) of each K block advance incrementally,
-          // with no divisions in the loop, and the ring's first lap (whose
-          // slots are free by construction) waits for nothing.
+          // Ring slot, phase and the (tap, channel block) of each K block advance
+          // incrementally, with no divisions in the loop, and the ring's first lap
+          // (whose slots are free by construction) waits for nothing.
+          const int cb_per_tap = p.Cp / BK;
           int slot = it % S;
           uint32_t ph = (uint32_t)((it / S) & 1);
-          int cb = ug.cb, rr = ug.rr, ss = ug.ss;  // conv = 2: channel block and tap of block kb
+          int cb = ug.cb, rr = ug.rr, ss = ug.ss;  // channel block and tap of block kb
           const int iy0 = ug.iy0, ix0 = ug.ix0;
           const uint32_t fb0 = bar_full, eb0 = bar_empty;
           for (int kb = kb0; kb <= last; ++kb) {
-            const bool issue =
-                !(skip && kb != last && kb < kMaxKWords * 32 && !((s_kbits[kb >> 5] >> (kb & 31)) & 1u));
-            if (issue) {
+            if (kb == last || kb >= kMaxKWords * 32 || ((s_kbits[kb >> 5] >> (kb & 31)) & 1u)) {
               if (it >= S && !mbar_wait(eb0 + 8 * slot, ph ^ 1u, err, s_abort, kErrTimeoutEmpty, wlim)) {
                 ok = false;
                 break;
@@ -803,10 +800,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
               const uint32_t fb = fb0 + 8 * slot;
               stage_last[slot] = (kb == last) ? 1 : 0;
               mbar_arrive_expect_tx(fb, (uint32_t)C::kStageBytes);
-              if (p.conv == 0)
-                tma_load_2d(sA + slot * C::kAStage, &tmA, fb, kb * BK, g.m0);
-              else
-                tma_load_4d(sA + slot * C::kAStage, &tmA, fb, cb * BK, ix0 + ss, iy0 + rr, g.tn0);
+              tma_load_4d(sA + slot * C::kAStage, &tmA, fb, cb * BK, ix0 + ss, iy0 + rr, g.tn0);
               tma_load_2d(sB + slot * C::kBStage, &tmB, fb, kb * BK, g.n0);
               ++it;
               if (++slot == S) {
@@ -814,7 +808,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
                 ph ^= 1u;
               }
             }
-            if (p.conv == 2 && ++cb == cb_per_tap) {
+            if (++cb == cb_per_tap) {
               cb = 0;
               if (++ss == p.kw) {
                 ss = 0;
@@ -879,7 +873,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
       }
     }
     if (r == 0) *s_issued = it;  // stages this CTA filled (TMA copies issued)
-    if (!LEAN && p.conv == 1) {
+    if (!LEAN) {
       cp_async_wait<0>();
       fence_proxy_async_smem();
       for (int q = pending; q > 0; --q) mbar_arrive(bar_full + 8 * ((it - q) % S));
@@ -1280,15 +1274,6 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
     const int et = threadIdx.x - kEpiThread0;  // 0..kEpiThreads-1
     const bool vec = (p.N % 8) == 0;
     const bool affine = ep.bias != nullptr || ep.bn != nullptr;  // else the column affine is 1, 0
-    // this warp's 32-row sub-box of the tile: {32 channels, bw', bh', bn'} for
-    // spatial tiles, 32 consecutive rows otherwise
-    int sw_ = 0, sh_ = 0, sn_ = 0;
-    if (p.conv == 2) {
-      const int rho = q * 32;
-      sw_ = rho % p.bw;
-      sh_ = (rho / p.bw) % p.bh;
-      sn_ = rho / (p.bw * p.bh);
-    }
     const uint32_t stg_base = sStg + (uint32_t)(ew * 2 * kWarpStgBytes);
     // Tile t covers columns (t % nt) BN..; when every tile of this CTA has the
     // same columns (one column tile, or a grid that is a multiple of the column
@@ -1371,9 +1356,6 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
         }
       }
       const OccDev o = P.out_occ;  // registers, not parameter-space loads
-      const int blk = mvalid ? (int)(m >> 7) : -1;
-      const uint32_t grp = p.conv == 2 ? __match_any_sync(0xffffffffu, blk) : 0xffffffffu;
-      const bool leader = (__ffs(grp) - 1) == lane;
       unsigned long long tl = 0ull;  // this row's occupied 64-column tiles
       // One 64-column group per iteration, kept as a loop (not unrolled) so the
       // epilogue's instructions stay in the instruction cache across groups.
@@ -1523,10 +1505,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
-            if (p.conv == 2)
-              tma_store_4d(&tmY, stg, ncol0, g.tw0 + sw_, g.th0 + sh_, g.tn0 + sn_);
-            else
-              tma_store_2d(&tmY, stg, ncol0, g.m0 + q * 32);
+            tma_store_2d(&tmY, stg, ncol0, g.m0 + q * 32);
             bulk_commit();
           }
           ++stg_count;
@@ -1534,12 +1513,8 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
         if (emit) {
           // this block's share of the output occupancy
           if (rw) tl |= 1ull << ((nbase >> 6) & 63);
-          const uint32_t bits = __reduce_or_sync(grp, rw);
-          const int word = (nbase >> 5) + hf;
-          if (leader && blk >= 0 && bits && word < o.C32) {
-            if (p.conv == 2) atomicOr(&o.blk_mask[blk * o.C32 + word], bits);
-            else atomicOr(&s_blk[gcol * 2 + hf], bits);  // the tile is the whole block
-          }
+          const uint32_t bits = __reduce_or_sync(0xffffffffu, rw);
+          if (lane == 0 && bits) atomicOr(&s_blk[gcol * 2 + hf], bits);  // the tile is the whole 128-row block
           // lane j: non-zeros of column 32 hf + j of this group in the warp's 32 rows
           s_cnt[q * BN + gcol * 64 + hf * 32 + lane] = __popc(warp_transpose32(rw));
         }
@@ -1562,7 +1537,7 @@ __global__ void __launch_bounds__(Warps<LEAN, STEM>::kThreads, 1)
             else if (v) atomicOr(dst, v);
           }
         }
-        if (p.conv != 2 && et < BN / 32) {
+        if (et < BN / 32) {
           const uint32_t v = s_blk[et];
           s_blk[et] = 0u;
           const int word = (g.n0 >> 5) + et;
@@ -1871,6 +1846,7 @@ cudaError_t launch_igemm(const IgemmArgs& a_in, cudaStream_t s) {
                          : launch_cfg<64, 64, 1, true>(a, tB, tB, tY, tB, tB, tiles, s);
   }
   if (a.conv == 2 && (a.Cp % 32 != 0 || a.bw * a.bh * a.bn != 128)) return cudaErrorInvalidValue;
+  if (a.conv == 2 && (reinterpret_cast<uintptr_t>(a.ep.residual) & 15u) != 0) return cudaErrorInvalidValue;  // (lean kernels only)
   const int64_t mtiles =
       a.conv == 2 ? (int64_t)((a.Nimg + a.bn - 1) / a.bn) * a.th * a.tw : (a.M + kBM - 1) / kBM;
   int bn = 64, ks = 1;

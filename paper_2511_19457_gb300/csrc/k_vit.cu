@@ -335,11 +335,6 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-template <bool B>
-struct BoolConst {
-  static constexpr bool value = B;
-};
-
 template <int HD>
 __global__ void __launch_bounds__(kAttnThreads, 2)
     attention_kernel(const __nv_bfloat16* __restrict__ qkv, int T, int heads, __nv_bfloat16* __restrict__ y,

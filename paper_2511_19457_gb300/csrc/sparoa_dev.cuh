@@ -280,6 +280,15 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, uint
       : "memory");
 }
 
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint32_t bar, int c0,
+                                            int c1, int c2, int c3) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
+      : "memory");
+}
+
 // Requests `bytes` (a multiple of 16) at a 16-byte aligned global address into L2.
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(p)), "r"(bytes) : "memory");
@@ -349,7 +358,11 @@ __device__ __forceinline__ void cp_async_wait() {
 // Programmatic dependent launch.  Every kernel of the library runs its
 // on-chip prologue (barrier init, TMEM allocation, tensor-map prefetch), then
 // pdl_wait(): the grid launched before it on the stream has completed and its
-// memory is visible.  No global memory is read or written before that wait.
+// memory is visible.  Before that wait nothing is written to global memory, and
+// nothing read but what the host knows to be complete: weights and parameters
+// where another kernel of the same call lies between their producer and this grid
+// (IgemmArgs::early, early_w), and weights requested into L2 without a use of
+// their values (prefetch_weights_l2).
 // pdl_trigger() right after lets the next grid start its own prologue while
 // this one works.  Both are no-ops for a launch without the attribute.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -653,6 +666,12 @@ __device__ __forceinline__ f2_t fmul2(f2_t a, f2_t b) {
 __device__ __forceinline__ uint32_t nz_pairs(uint32_t w) {
   return __hneu2_mask(*reinterpret_cast<const __nv_bfloat162*>(&w), __floats2bfloat162_rn(0.f, 0.f)) & 0x00010001u;
 }
+
+// A compile-time flag to pass to a generic lambda.
+template <bool B>
+struct BoolConst {
+  static constexpr bool value = B;
+};
 
 // Two fp32 values through the activation to a bf16 pair (round to nearest
 // even), `lo` in the low half; ReLU is applied by the conversion itself.
