@@ -7,8 +7,9 @@ of every CTA (a barrier phase that nothing else completes).  The epilogue's
 wait runs out, every CTA unwinds (waiting, bounded again, for the copies and
 MMAs it already issued), the call that synchronises returns
 SPAROA_ERR_TIMEOUT, and the same context then computes the operator correctly.
-This is done for the implicit-GEMM kernel (a GEMM and a strided convolution)
-and for the 3x3 slab kernel.
+This is done for the implicit-GEMM kernel (GEMMs of one and of many tiles a CTA,
+weights that stay in shared memory, a strided convolution, a stem), the one-tile
+kernel and the 3x3 slab kernel.
 
 Allocation failure: injected on the host; the next workspace allocation of the
 context fails, the call returns SPAROA_ERR_OOM, and the next call succeeds.
@@ -63,9 +64,19 @@ def _conv_case(sp, N, H, W, C, Co, k, stride, seed):
 
 
 CASES = {
-    # implicit-GEMM kernel: several tiles per CTA on 152 SMs
+    # implicit-GEMM kernel: one tile per CTA on 152 SMs
     "gemm": lambda sp: _gemm_case(sp, 4096, 512, 512, 1),
-    # implicit-GEMM kernel, strided convolution (4-D TMA boxes)
+    # ... and several, 32-column groups in pairs on the zero-skip path
+    "gemm_tiles": lambda sp: _gemm_case(sp, 8192, 256, 1024, 5),
+    # a 1x1 expansion, six tiles per CTA: weights that stay, one epilogue warp per
+    # quarter of a tile (dense path), the ring's loads (zero-skip path)
+    "expansion": lambda sp: _conv_case(sp, 8, 112, 112, 96, 96, 1, 1, 6),
+    # strided convolution with more tiles than SMs (4-D TMA boxes; the masks of the
+    # zero-skip path tile by tile)
+    "conv3x3s2_tiles": lambda sp: _conv_case(sp, 8, 128, 128, 32, 64, 3, 2, 7),
+    # an RGB stem, about five tiles per CTA (A tiles built by the producer warps)
+    "stem": lambda sp: _conv_case(sp, 8, 224, 224, 3, 24, 7, 2, 8),
+    # one-tile kernel: a strided convolution, clusters of CTAs
     "conv3x3s2": lambda sp: _conv_case(sp, 4, 28, 28, 64, 128, 3, 2, 2),
     # 3x3 slab kernel: one and two tiles per CTA
     "conv3x3s1": lambda sp: _conv_case(sp, 8, 56, 56, 64, 64, 3, 1, 3),
