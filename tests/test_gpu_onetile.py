@@ -46,7 +46,11 @@ def _sparse(shape, g, block=None):
 @pytest.mark.parametrize("M,K,N,act,f32", [
     (1, 64, 8, 0, False), (1, 32, 64, 1, True), (37, 72, 200, 3, False), (127, 4096, 64, 2, False),
     (128, 2048, 72, 1, True), (129, 3072, 136, 1, False), (256, 648, 768, 0, False), (400, 256, 712, 3, False),
-    (640, 1096, 256, 2, False), (1216, 128, 256, 1, False)])
+    (640, 1096, 256, 2, False), (1216, 128, 256, 1, False),
+    # (bf16 outputs of few K blocks run in the persistent kernel: fp32 ones here)
+    (1, 64, 8, 0, True), (37, 72, 200, 3, True), (400, 256, 712, 3, True), (1216, 128, 256, 1, True),
+    # one CTA a tile and a long K; 15 and 16 tiles around the clusters of 8 that fit
+    (128, 3104, 4992, 1, False), (128, 1600, 960, 1, False), (128, 1600, 1024, 3, False)])
 @pytest.mark.parametrize("force", [1, 2])
 def test_gemm(sp, ctx, M, K, N, act, f32, force):
     g = torch.Generator().manual_seed(M + K + N)
