@@ -43,6 +43,21 @@ NBUF = 40   # rotating input/output sets per step, 40 x 6.6 MB > 129 MB L2
 LAUNCHES_PER_CONV_STEP = 3
 
 
+def config_summary(full):
+    """The headline number of every other configuration: us, images/s, crossover."""
+    out = {}
+    if isinstance(full.get("fc"), dict) and "step_us" in full["fc"]:
+        out["fc_step_us"] = round(full["fc"]["step_us"], 2)
+    graphs = {k: round(r["images_per_s"], 1) for k, r in full.get("graphs", {}).items()
+              if isinstance(r, dict) and "images_per_s" in r}
+    if graphs:
+        out["images_per_s"] = graphs
+    sweep = full.get("mlp_sweep")
+    if isinstance(sweep, dict) and "crossover_rho" in sweep:
+        out["mlp_crossover_rho"] = {k: v for k, v in sweep["crossover_rho"].items() if v is not None}
+    return out
+
+
 def parse_args():
     p = argparse.ArgumentParser()
     p.add_argument("--gpus", type=int, default=1)
@@ -1278,6 +1293,11 @@ def main():
             for rec in line["other_configs"].get("graphs", {}).values():
                 if isinstance(rec, dict):
                     rec.pop("decisions", None)
+            # whole records on stderr; the line itself stays short enough (3000
+            # characters) for a reader that keeps the end of stdout only
+            full = line.pop("other_configs")
+            print(json.dumps({"other_configs": full}), file=sys.stderr, flush=True)
+            line["other_configs"] = config_summary(full)
     elif args.workload in ("resnet18", "mobilenet_v2", "vit_b16"):
         line = run_graph_workload(args, rank, local_rank, world, peaks, args.workload)
     elif args.workload == "fc":

@@ -65,3 +65,14 @@ def test_traffic_entries_name_committed_commands(bench_mod):
         # the hash covers files that exist
         for f in bench_mod.COMMON_SOURCES + bench_mod.KERNEL_SOURCES[key]:
             assert os.path.exists(os.path.join(ROOT, "paper_2511_19457_gb300", "csrc", f)), f
+
+
+def test_config_summary_is_short_and_keeps_the_headline_numbers():
+    import bench
+    full = {"fc": {"step_us": 7.527416, "roofline": {"x": "y" * 500}},
+            "graphs": {"resnet18_b1": {"images_per_s": 5575.379, "ops": {}}, "vit": {"error": "no"}},
+            "mobilenet_v2_dense_ops": [{"us": 1.0}] * 40,
+            "mlp_sweep": {"crossover_rho": {"M256_block32": 0.9, "M256_token": None}, "table": [{"M": 1}] * 600}}
+    s = bench.config_summary(full)
+    assert s == {"fc_step_us": 7.53, "images_per_s": {"resnet18_b1": 5575.4}, "mlp_crossover_rho": {"M256_block32": 0.9}}
+    assert len(json.dumps(bench.config_summary({"fc": {"error": "no device"}, "graphs": {}, "mlp_sweep": None}))) == 2
