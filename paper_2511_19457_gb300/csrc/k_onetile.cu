@@ -683,7 +683,7 @@ int clusters_at_once(int ks) {
 //   K = 4608   90 tiles            by 1 18.2 / 21.1  19.8 / 22.6
 // A convolution's zero-skip path is much slower in the persistent kernel (its
 // masks, then its loads, tile by tile: [8,28,28,128] 3x3 by 1 13, persistent 19.6;
-// dense 11.4 and 11.2), so it goes there only where the dense path is forced.
+// dense 11.4 and 11.2), so unless the dense path is forced it takes what fits.
 // fp32 output (`lean` false), whose persistent kernel is slower, takes what fits.
 int onetile_split(const IgemmArgs& a, int64_t mtiles, int bk, bool lean) {
   const int64_t tiles = mtiles * ((a.N + kBN - 1) / kBN);
@@ -692,7 +692,7 @@ int onetile_split(const IgemmArgs& a, int64_t mtiles, int bk, bool lean) {
   for (int ks = 8; ks >= 1; ks /= 2) {
     const int least = !lean        ? ks
                       : ks == 8    ? 24
-                      : a.conv     ? (ks > 1 || a.disp.force != 1 ? ks : 48)
+                      : a.conv && a.disp.force != 1 ? ks
                       : ks == 4    ? (a.emit ? 4 : 8)
                       : ks == 2    ? (a.emit ? 8 : 12)
                                    : 48;
