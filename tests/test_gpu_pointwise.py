@@ -107,3 +107,14 @@ def test_tiles_of_96_and_160_columns(sp, ctx, M, K, N, act, res, force):
     v = {0: lambda t: t, 1: torch.relu, 2: lambda t: t.clamp(0, 6),
          3: lambda t: torch.nn.functional.gelu(t, approximate="tanh")}[act](v)
     assert_close(y.float().cpu().numpy(), v.cpu().numpy(), what="gemm")
+
+
+@pytest.mark.parametrize("M,K,N,act,res", [
+    (19451, 64, 96, 1, False), (19584, 128, 128, 1, True), (38912, 64, 128, 0, False), (38913, 64, 128, 2, True),
+    (19500, 40, 64, 1, True), (5000, 128, 640, 1, True), (300, 64, 72, 3, False), (128, 64, 4928, 1, True),
+    (1000, 96, 4160, 0, False)])
+@pytest.mark.parametrize("force", [1, 2])
+def test_one_and_two_tiles_a_cta(sp, ctx, M, K, N, act, res, force):
+    """around one and two tiles per CTA of 152, where the epilogue warps share tiles
+    and a lone tile's counts go straight out; one and two groups of K"""
+    test_tiles_of_96_and_160_columns(sp, ctx, M, K, N, act, res, force)
