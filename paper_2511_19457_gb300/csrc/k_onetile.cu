@@ -6,10 +6,10 @@
 // blocks per CTA, then the sum over the K shares, then the epilogue.  Against
 // the persistent kernel with its split K through global memory: ResNet-18 at
 // batch 1 311 -> 177 us, a strided basic block at batch 8 (28x28x128 -> 14x14x256,
-// three convolutions) 47 -> 33 us; one call (with its occupancy clear) 7.7 us on
-// [1,14,14,256] 3x3 and 8.8 us on [1,7,7,512] 3x3, of which (clock64) 1.2 us to
-// the first operands, 0.5-1.5 us of MMAs, 0.4 us to read the accumulator, 0.6 us
-// at the cluster barrier, 1.2 us for the sum and the stores, 0.7 us of occupancy.  So
+// three convolutions) 47 -> 33 us when it came, 173 and 28 us now; one call (with its occupancy clear) 8.1 us on [1,14,14,256]
+// 3x3 and 9.2 us on [1,7,7,512] 3x3, of which (clock64) 1.2 us to the first
+// operands, 0.5-1.5 us of MMAs, 0.4 us to read the accumulator, 0.6 us at the
+// cluster barrier, 1.2 us for the sum and the stores, 0.7 us of occupancy.  So
 //   - the K range of a tile is cut over up to 8 CTAs of one cluster, and the
 //     fp32 partial tiles meet in distributed shared memory: no partials in
 //     global memory, no arrival tickets, no CTA left with the whole epilogue;
