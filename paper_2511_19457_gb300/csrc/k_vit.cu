@@ -656,7 +656,9 @@ namespace {
 //     SMs gave.  Where one CTA a head leaves the last round mostly empty (some
 //     hundred pairs of more than 15 tiles, two CTAs an SM), a tile per warp.
 //   - Fewer pairs: a tile per warp, and up to a CTA per SM, of two tiles or more;
-//     three a head while two an SM hold them.  Warps without a tile stage.
+//     three a head while two an SM hold them; as many as two an SM hold where each
+//     keeps four tiles (48 pairs, T = 384 16.1 -> 12, 96 pairs 23 -> 19.6 us).  Warps
+//     without a tile stage.
 // Times with occupancy, us: CTAs of 7 warps with a tile per warp / this rule:
 //   pairs, dimension  T = 16       64         128        197        257       512
 //   12, 64           3.4 / 3.5  4.0 / 3.9  4.9 / 4.8  7.3 / 6.0  8.3 / 6.9  12 / 9.7
@@ -677,8 +679,11 @@ void attention_split(int64_t pairs, int T, size_t smem, int* warps, int* qsplit)
     const int64_t fill = sms / pairs;
     if (fill > q) q = (int)(fill < up(tiles, 2) ? fill : up(tiles, 2));
     if (q < 3 && tiles >= 8 && 3 * pairs <= 2 * sms) q = 3;
-    q = up(tiles, up(tiles, q));
-    *warps = kAttnWarps;
+    const int64_t even = two ? 2 * sms / pairs : 0;  // CTAs of a head that fill the SMs twice
+    if (even >= 3 && 4 * even <= tiles) q = (int)even;
+    const int per = up(tiles, q);
+    q = up(tiles, per);
+    *warps = per > kAttnWarps ? up(per, 2) : kAttnWarps;
   }
   *qsplit = q;
 }
