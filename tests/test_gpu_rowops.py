@@ -172,7 +172,8 @@ def test_attention_weights_below_the_normal_range(sp, ctx, far):
 
 @pytest.mark.parametrize("N,T,heads,hd", [(40, 17, 12, 64), (26, 64, 12, 16), (52, 100, 8, 32), (40, 129, 12, 16),
                                           (32, 225, 12, 16), (32, 300, 12, 16), (102, 300, 12, 16), (13, 500, 24, 64),
-                                          (1, 500, 2, 64), (20, 48, 12, 32), (16, 385, 12, 32)])
+                                          (1, 500, 2, 64), (20, 48, 12, 32), (16, 385, 12, 32),
+                                          (4, 384, 12, 64), (8, 380, 12, 32), (10, 330, 6, 16)])
 def test_attention_splits(sp, ctx, N, T, heads, hd):
     """Every way a head's query tiles are shared out: a tile per warp, several in
     turn, one CTA a head and many, tiles that do not come out even."""
